@@ -31,6 +31,7 @@
 #include <unordered_map>
 
 #include "../../include/trotter.h"
+#include "common.cuh"
 #include "ffloat.cuh"
 #include "grid.h"
 #include "internal.h"
@@ -93,6 +94,7 @@ __global__ void grad_finalize_kernel(const float *__restrict__ g_rh, const float
                                      int nx, int ny, int64_t pitch, double c_re, double c_im,
                                      double two_dt, float *__restrict__ grad)
 {
+    ts::grid_dep_sync();
     const int64_t n = (int64_t)nx * ny;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -293,8 +295,7 @@ ts_status ts_adjoint_backward_depth(ts_grid *g, void *ws, size_t ws_bytes, int K
     }
     const int64_t sites = (int64_t)nx * ny;
     int blocks = (int)std::min<int64_t>((sites + 255) / 256, 152 * 32);
-    grad_finalize_kernel<<<blocks, 256, 0, st>>>(
-        (const float *)plane(WS_G), (const float *)plane(WS_G + 1), (const float *)plane(WS_G + 2),
+    ts::launch_pdl(grad_finalize_kernel, blocks, 256, 0, st, (const float *)plane(WS_G), (const float *)plane(WS_G + 1), (const float *)plane(WS_G + 2),
         (const float *)plane(WS_G + 3), nx, ny, pitch, a.c_re, a.c_im, 2.0 * g->dt, grad);
     ts::count_launches(1);
     e = cudaGetLastError();

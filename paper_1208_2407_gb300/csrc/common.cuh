@@ -156,6 +156,13 @@ __device__ __forceinline__ void angle_versine(double phi, double &g, double &s)
     s = sin(phi);
 }
 
+// Wait until the kernel before this one in the stream has completed and its
+// writes are visible.  See launch_pdl in internal.h.
+__device__ __forceinline__ void grid_dep_sync()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 __device__ __forceinline__ uint64_t globaltimer_ns()
 {
     uint64_t t;

@@ -1336,6 +1336,7 @@ fused_kernel(const __grid_constant__ CUtensorMap tm_state,
     const int gw = blockIdx.x * Cfg<K>::WPC + warp;
     if (gw >= p.total_warps) return;
     WarpRings r = carve_rings<K, phase_planes(MODE), MODE == 4, state_planes(MODE), MODE>(smem_raw, warp, lane);
+    grid_dep_sync();
     if (p.strip_warps > 0) {
         // strip-aligned split: warp (sx, i) takes row range i of strip sx, so
         // warps of neighbouring strips walk the same rows at the same time and
@@ -1385,6 +1386,7 @@ fused3d_kernel(const __grid_constant__ CUtensorMap tm_state,
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     WarpRings r = carve_rings<K, phase_planes(6), false, state_planes(6), 6>(smem_raw, warp, lane);
     const int64_t slab = (int64_t)p.ny * p.pitch;
+    grid_dep_sync();
     for (int64_t u = blockIdx.x; u < p.units; u += gridDim.x) {
         const int zb = (int)(u % p.n_zblocks);
         const int64_t t = u / p.n_zblocks;
@@ -1452,6 +1454,7 @@ fused_multi_kernel(const EpochEntry *__restrict__ tab, int n_grids, int64_t tota
     const int gw = blockIdx.x * C::WPC + warp;
     if (gw >= total_warps) return;
     WarpRings r = carve_rings<K>(smem_raw, warp, lane);
+    grid_dep_sync();
     if (aligned) {
         // the grid of warp gw: the last entry whose first warp is <= gw
         int lo = 0, hi = n_grids - 1;
@@ -1580,7 +1583,7 @@ cudaError_t launch3_k(const FusedLaunch &a, int nz, cudaStream_t st)
     p.s2 = a.s2;
     p.err = a.err;
     const int grid = (int)std::min<int64_t>(p.units, ctas);
-    fused3d_kernel<1><<<grid, NW * 32, C::SMEM, st>>>(*a.tm_state, *a.tm_phase, p);
+    launch_pdl(fused3d_kernel<1>, grid, NW * 32, C::SMEM, st, *a.tm_state, *a.tm_phase, p);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -1648,8 +1651,7 @@ cudaError_t launch_k(const FusedLaunch &a, cudaStream_t st)
     p.tab = a.tab;
     p.sab = a.sab;
     const int blocks = (p.total_warps + C::WPC - 1) / C::WPC;
-    fused_kernel<K, MODE><<<blocks, C::WPC * 32, C::SMEM, st>>>(
-        *a.tm_state, *a.tm_phase, a.tm_b ? *a.tm_b : *a.tm_phase, p);
+    launch_pdl(fused_kernel<K, MODE>, blocks, C::WPC * 32, C::SMEM, st, *a.tm_state, *a.tm_phase, a.tm_b ? *a.tm_b : *a.tm_phase, p);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -1693,8 +1695,7 @@ cudaError_t launch_multi_k(const EpochEntry *tab, int n_grids, const MultiPlan &
     const Occupancy &occ = multi_occupancy<K>();
     if (occ.err != cudaSuccess) return occ.err;
     const int blocks = (plan.warps + C::WPC - 1) / C::WPC;
-    fused_multi_kernel<K><<<blocks, C::WPC * 32, C::SMEM, st>>>(
-        tab, n_grids, plan.units, plan.warps, plan.aligned ? 1 : 0, flip, err);
+    launch_pdl(fused_multi_kernel<K>, blocks, C::WPC * 32, C::SMEM, st, tab, n_grids, plan.units, plan.warps, plan.aligned ? 1 : 0, flip, err);
     count_launches(1);
     return cudaGetLastError();
 }

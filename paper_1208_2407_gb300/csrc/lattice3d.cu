@@ -27,6 +27,7 @@ template <typename T, bool LIFT = false>
 __global__ void sweep_y3_kernel(T *__restrict__ re, T *__restrict__ im, int nx, int ny, int nz,
                                 int64_t pitch, int parity, T g, T s)
 {
+    grid_dep_sync();
     const int per_slab = (ny - parity) / 2;
     const int64_t npairs = (int64_t)per_slab * nz;
     for (int64_t q = blockIdx.y; q < npairs; q += gridDim.y) {
@@ -50,6 +51,7 @@ template <typename T, bool LIFT = false>
 __global__ void sweep_z_kernel(T *__restrict__ re, T *__restrict__ im, int nx, int ny, int nz,
                                int64_t pitch, int parity, T g, T s)
 {
+    grid_dep_sync();
     const int npz = (nz - parity) / 2;
     const int64_t nrows = (int64_t)npz * ny;
     const int64_t slab = (int64_t)ny * pitch;
@@ -79,11 +81,11 @@ cudaError_t launch_plain_sweep_y3(void *re, void *im, bool f64, int nx, int ny, 
     if (npairs <= 0) return cudaSuccess;
     dim3 grid = grid2d(nx, npairs);
     if (f64 && lift)
-        sweep_y3_kernel<double, true><<<grid, kThreads, 0, st>>>((double *)re, (double *)im, nx, ny, nz, pitch, parity, g, s);
+        launch_pdl(sweep_y3_kernel<double, true>, grid, kThreads, 0, st, (double *)re, (double *)im, nx, ny, nz, pitch, parity, g, s);
     else if (f64)
-        sweep_y3_kernel<double><<<grid, kThreads, 0, st>>>((double *)re, (double *)im, nx, ny, nz, pitch, parity, g, s);
+        launch_pdl(sweep_y3_kernel<double>, grid, kThreads, 0, st, (double *)re, (double *)im, nx, ny, nz, pitch, parity, g, s);
     else
-        sweep_y3_kernel<float><<<grid, kThreads, 0, st>>>((float *)re, (float *)im, nx, ny, nz, pitch, parity, (float)g, (float)s);
+        launch_pdl(sweep_y3_kernel<float>, grid, kThreads, 0, st, (float *)re, (float *)im, nx, ny, nz, pitch, parity, (float)g, (float)s);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -96,11 +98,11 @@ cudaError_t launch_plain_sweep_z(void *re, void *im, bool f64, int nx, int ny, i
     if (nrows <= 0) return cudaSuccess;
     dim3 grid = grid2d(nx, nrows);
     if (f64 && lift)
-        sweep_z_kernel<double, true><<<grid, kThreads, 0, st>>>((double *)re, (double *)im, nx, ny, nz, pitch, parity, g, s);
+        launch_pdl(sweep_z_kernel<double, true>, grid, kThreads, 0, st, (double *)re, (double *)im, nx, ny, nz, pitch, parity, g, s);
     else if (f64)
-        sweep_z_kernel<double><<<grid, kThreads, 0, st>>>((double *)re, (double *)im, nx, ny, nz, pitch, parity, g, s);
+        launch_pdl(sweep_z_kernel<double>, grid, kThreads, 0, st, (double *)re, (double *)im, nx, ny, nz, pitch, parity, g, s);
     else
-        sweep_z_kernel<float><<<grid, kThreads, 0, st>>>((float *)re, (float *)im, nx, ny, nz, pitch, parity, (float)g, (float)s);
+        launch_pdl(sweep_z_kernel<float>, grid, kThreads, 0, st, (float *)re, (float *)im, nx, ny, nz, pitch, parity, (float)g, (float)s);
     count_launches(1);
     return cudaGetLastError();
 }

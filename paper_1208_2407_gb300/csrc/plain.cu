@@ -67,6 +67,7 @@ template <bool IN, typename Ts, typename Td>
 __global__ void convert_kernel(const Ts *__restrict__ src, Td *__restrict__ dst, int nx, int ny,
                                int64_t pitch, bool vec4)
 {
+    grid_dep_sync();
     for (int64_t y = blockIdx.y; y < ny; y += gridDim.y) {
         const Ts *s = src + y * (IN ? (int64_t)nx : pitch);
         Td *d = dst + y * (IN ? pitch : (int64_t)nx);
@@ -95,6 +96,7 @@ __global__ void phase_table_kernel(const double *__restrict__ V, T *__restrict__
                                    T *__restrict__ ps, T *__restrict__ vp, int nx, int ny,
                                    int64_t pitch, double dt)
 {
+    grid_dep_sync();
     const int64_t n = (int64_t)nx * ny;
     for (Walk w(nx, blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
                 (int64_t)gridDim.x * blockDim.x);
@@ -185,6 +187,7 @@ __global__ void phase_table_f32_kernel(const double *__restrict__ V, float *__re
 {
     __shared__ float4 sc[256];
     for (int i = threadIdx.x; i < 256; i += blockDim.x) sc[i] = tab.sc[i];
+    grid_dep_sync();
     __syncthreads();
     const int64_t n = (int64_t)nx * ny;
     for (Walk w(nx, blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
@@ -249,6 +252,7 @@ template <typename T, bool LIFT = false>
 __global__ void plain_sweep_x_kernel(T *__restrict__ re, T *__restrict__ im, int nx, int ny,
                                      int64_t pitch, int parity, T g, T s)
 {
+    grid_dep_sync();
     const int npr = (nx - parity) / 2;   // pairs per row
     if (npr <= 0) return;
     for (int y = blockIdx.y; y < ny; y += gridDim.y) {
@@ -273,6 +277,7 @@ template <typename T, bool LIFT = false>
 __global__ void plain_sweep_y_kernel(T *__restrict__ re, T *__restrict__ im, int nx, int ny,
                                      int64_t pitch, int parity, T g, T s)
 {
+    grid_dep_sync();
     const int npc = (ny - parity) / 2;   // pairs per column
     for (int q = blockIdx.y; q < npc; q += gridDim.y) {
         int64_t y = parity + 2 * q;
@@ -295,6 +300,7 @@ __global__ void plain_phase_kernel(T *__restrict__ re, T *__restrict__ im,
                                    const T *__restrict__ pg, const T *__restrict__ ps, int nx,
                                    int ny, int64_t pitch)
 {
+    grid_dep_sync();
     for (int y = blockIdx.y; y < ny; y += gridDim.y) {
         int64_t o = (int64_t)y * pitch;
         for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < nx;
@@ -311,6 +317,7 @@ template <typename T>
 __global__ void plain_drive_kernel(T *__restrict__ re, T *__restrict__ im,
                                    const T *__restrict__ v1, int nx, int ny, int64_t pitch, T adt)
 {
+    grid_dep_sync();
     for (int y = blockIdx.y; y < ny; y += gridDim.y) {
         int64_t o = (int64_t)y * pitch;
         for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < nx;
@@ -341,13 +348,13 @@ cudaError_t launch_convert(const void *src, bool src_f64, void *dst, bool dst_f6
     const bool vec4 = (nx % 4) == 0 && ((uintptr_t)src % 16) == 0 && ((uintptr_t)dst % 16) == 0;
     dim3 grid = grid2d(vec4 ? nx / 4 : nx, ny);
     if (src_f64 && dst_f64)
-        convert_kernel<IN, double, double><<<grid, kThreads, 0, st>>>((const double *)src, (double *)dst, nx, ny, pitch, vec4);
+        launch_pdl(convert_kernel<IN, double, double>, grid, kThreads, 0, st, (const double *)src, (double *)dst, nx, ny, pitch, vec4);
     else if (src_f64)
-        convert_kernel<IN, double, float><<<grid, kThreads, 0, st>>>((const double *)src, (float *)dst, nx, ny, pitch, vec4);
+        launch_pdl(convert_kernel<IN, double, float>, grid, kThreads, 0, st, (const double *)src, (float *)dst, nx, ny, pitch, vec4);
     else if (dst_f64)
-        convert_kernel<IN, float, double><<<grid, kThreads, 0, st>>>((const float *)src, (double *)dst, nx, ny, pitch, vec4);
+        launch_pdl(convert_kernel<IN, float, double>, grid, kThreads, 0, st, (const float *)src, (double *)dst, nx, ny, pitch, vec4);
     else
-        convert_kernel<IN, float, float><<<grid, kThreads, 0, st>>>((const float *)src, (float *)dst, nx, ny, pitch, vec4);
+        launch_pdl(convert_kernel<IN, float, float>, grid, kThreads, 0, st, (const float *)src, (float *)dst, nx, ny, pitch, vec4);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -369,7 +376,7 @@ cudaError_t launch_phase_table(const double *V, void *pg, void *ps, void *vplane
 {
     int grid = grid_for((int64_t)nx * ny, kThreads);
     if (f64) {
-        phase_table_kernel<double><<<grid, kThreads, 0, st>>>(V, (double *)pg, (double *)ps, (double *)vplane, nx, ny, pitch, dt);
+        launch_pdl(phase_table_kernel<double>, grid, kThreads, 0, st, V, (double *)pg, (double *)ps, (double *)vplane, nx, ny, pitch, dt);
     } else {
         thread_local TrigTable tab;   // per thread: grids may be prepared concurrently
         thread_local double tab_dt = std::nan("");
@@ -397,7 +404,7 @@ cudaError_t launch_phase_table(const double *V, void *pg, void *ps, void *vplane
             tab.hdt_lo = (float)(tab.hdt - tab.hdt_hi);
             tab_dt = dt;
         }
-        phase_table_f32_kernel<<<grid, kThreads, 0, st>>>(V, (float *)pg, (float *)ps, (float *)vplane, nx, ny, pitch, tab);
+        launch_pdl(phase_table_f32_kernel, grid, kThreads, 0, st, V, (float *)pg, (float *)ps, (float *)vplane, nx, ny, pitch, tab);
     }
     count_launches(1);
     return cudaGetLastError();
@@ -410,19 +417,19 @@ cudaError_t launch_plain_sweep(void *re, void *im, bool f64, int nx, int ny, int
     if (axis == 0) {
         dim3 grid = grid2d((nx - parity) / 2, ny);
         if (f64 && lift)
-            plain_sweep_x_kernel<double, true><<<grid, kThreads, 0, st>>>((double *)re, (double *)im, nx, ny, pitch, parity, g, s);
+            launch_pdl(plain_sweep_x_kernel<double, true>, grid, kThreads, 0, st, (double *)re, (double *)im, nx, ny, pitch, parity, g, s);
         else if (f64)
-            plain_sweep_x_kernel<double><<<grid, kThreads, 0, st>>>((double *)re, (double *)im, nx, ny, pitch, parity, g, s);
+            launch_pdl(plain_sweep_x_kernel<double>, grid, kThreads, 0, st, (double *)re, (double *)im, nx, ny, pitch, parity, g, s);
         else
-            plain_sweep_x_kernel<float><<<grid, kThreads, 0, st>>>((float *)re, (float *)im, nx, ny, pitch, parity, (float)g, (float)s);
+            launch_pdl(plain_sweep_x_kernel<float>, grid, kThreads, 0, st, (float *)re, (float *)im, nx, ny, pitch, parity, (float)g, (float)s);
     } else {
         dim3 grid = grid2d(nx, (ny - parity) / 2);
         if (f64 && lift)
-            plain_sweep_y_kernel<double, true><<<grid, kThreads, 0, st>>>((double *)re, (double *)im, nx, ny, pitch, parity, g, s);
+            launch_pdl(plain_sweep_y_kernel<double, true>, grid, kThreads, 0, st, (double *)re, (double *)im, nx, ny, pitch, parity, g, s);
         else if (f64)
-            plain_sweep_y_kernel<double><<<grid, kThreads, 0, st>>>((double *)re, (double *)im, nx, ny, pitch, parity, g, s);
+            launch_pdl(plain_sweep_y_kernel<double>, grid, kThreads, 0, st, (double *)re, (double *)im, nx, ny, pitch, parity, g, s);
         else
-            plain_sweep_y_kernel<float><<<grid, kThreads, 0, st>>>((float *)re, (float *)im, nx, ny, pitch, parity, (float)g, (float)s);
+            launch_pdl(plain_sweep_y_kernel<float>, grid, kThreads, 0, st, (float *)re, (float *)im, nx, ny, pitch, parity, (float)g, (float)s);
     }
     count_launches(1);
     return cudaGetLastError();
@@ -433,9 +440,9 @@ cudaError_t launch_plain_drive(void *re, void *im, const void *v1, bool f64, int
 {
     dim3 grid = grid2d(nx, ny);
     if (f64)
-        plain_drive_kernel<double><<<grid, kThreads, 0, st>>>((double *)re, (double *)im, (const double *)v1, nx, ny, pitch, adt);
+        launch_pdl(plain_drive_kernel<double>, grid, kThreads, 0, st, (double *)re, (double *)im, (const double *)v1, nx, ny, pitch, adt);
     else
-        plain_drive_kernel<float><<<grid, kThreads, 0, st>>>((float *)re, (float *)im, (const float *)v1, nx, ny, pitch, (float)adt);
+        launch_pdl(plain_drive_kernel<float>, grid, kThreads, 0, st, (float *)re, (float *)im, (const float *)v1, nx, ny, pitch, (float)adt);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -445,9 +452,9 @@ cudaError_t launch_plain_phase(void *re, void *im, const void *pg, const void *p
 {
     dim3 grid = grid2d(nx, ny);
     if (f64)
-        plain_phase_kernel<double><<<grid, kThreads, 0, st>>>((double *)re, (double *)im, (const double *)pg, (const double *)ps, nx, ny, pitch);
+        launch_pdl(plain_phase_kernel<double>, grid, kThreads, 0, st, (double *)re, (double *)im, (const double *)pg, (const double *)ps, nx, ny, pitch);
     else
-        plain_phase_kernel<float><<<grid, kThreads, 0, st>>>((float *)re, (float *)im, (const float *)pg, (const float *)ps, nx, ny, pitch);
+        launch_pdl(plain_phase_kernel<float>, grid, kThreads, 0, st, (float *)re, (float *)im, (const float *)pg, (const float *)ps, nx, ny, pitch);
     count_launches(1);
     return cudaGetLastError();
 }

@@ -89,6 +89,7 @@ observe_f32_kernel(const float *__restrict__ re, const float *__restrict__ im,
                    const float *__restrict__ vp, int nx, int ny, int64_t pitch, float J_hi,
                    float J_lo, double *__restrict__ partials)
 {
+    grid_dep_sync();
     constexpr int NQ = NORM_ONLY ? 1 : OBS_Q;
     FF acc[NQ];
 #pragma unroll
@@ -179,6 +180,7 @@ inner_f32_kernel(const float *__restrict__ ar, const float *__restrict__ ai,
                  const float *__restrict__ br, const float *__restrict__ bi, int nx, int ny,
                  int64_t pitch, double *__restrict__ partials)
 {
+    grid_dep_sync();
     FF sr = ff_make(0.f), si = ff_make(0.f);
     const int chunks_per_row = (nx + 3) / 4;
     const int64_t nchunks = (int64_t)chunks_per_row * ny;
@@ -217,6 +219,7 @@ __global__ void __launch_bounds__(kThreads)
 observe_kernel(const T *__restrict__ re, const T *__restrict__ im, const T *__restrict__ vp,
                int nx, int ny, int64_t pitch, double J, double *__restrict__ partials)
 {
+    grid_dep_sync();
     constexpr int NQ = NORM_ONLY ? 1 : OBS_Q;
     Neu acc[NQ];
 #pragma unroll
@@ -302,6 +305,7 @@ __global__ void __launch_bounds__(kThreads)
 observe3_kernel(const T *__restrict__ re, const T *__restrict__ im, const T *__restrict__ vp,
                 int nx, int ny, int nz, int64_t pitch, double J, double *__restrict__ partials)
 {
+    grid_dep_sync();
     constexpr int NQ = OBS_Q3;
     Neu acc[NQ];
 #pragma unroll
@@ -382,6 +386,7 @@ __global__ void __launch_bounds__(kThreads)
 observe_finalize_kernel(const double *__restrict__ partials, int nblocks, int nq, int stride,
                         double *__restrict__ result)
 {
+    grid_dep_sync();
     __shared__ double sh_s[kThreads / 32], sh_c[kThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int q = 0; q < nq; ++q) {
@@ -427,17 +432,17 @@ cudaError_t launch_observe(const void *re, const void *im, const void *vplane, b
     int nblocks = (int)(b < 1 ? 1 : (b > OBS_MAX_BLOCKS ? OBS_MAX_BLOCKS : b));
     if (f64) {
         if (norm_only)
-            observe_kernel<double, true><<<nblocks, kThreads, 0, st>>>((const double *)re, (const double *)im, (const double *)vplane, nx, ny, pitch, J, partials);
+            launch_pdl(observe_kernel<double, true>, nblocks, kThreads, 0, st, (const double *)re, (const double *)im, (const double *)vplane, nx, ny, pitch, J, partials);
         else
-            observe_kernel<double, false><<<nblocks, kThreads, 0, st>>>((const double *)re, (const double *)im, (const double *)vplane, nx, ny, pitch, J, partials);
+            launch_pdl(observe_kernel<double, false>, nblocks, kThreads, 0, st, (const double *)re, (const double *)im, (const double *)vplane, nx, ny, pitch, J, partials);
     } else {
         const float J_hi = (float)J, J_lo = (float)(J - (double)J_hi);
         if (norm_only)
-            observe_f32_kernel<true><<<nblocks, kThreads, 0, st>>>((const float *)re, (const float *)im, (const float *)vplane, nx, ny, pitch, J_hi, J_lo, partials);
+            launch_pdl(observe_f32_kernel<true>, nblocks, kThreads, 0, st, (const float *)re, (const float *)im, (const float *)vplane, nx, ny, pitch, J_hi, J_lo, partials);
         else
-            observe_f32_kernel<false><<<nblocks, kThreads, 0, st>>>((const float *)re, (const float *)im, (const float *)vplane, nx, ny, pitch, J_hi, J_lo, partials);
+            launch_pdl(observe_f32_kernel<false>, nblocks, kThreads, 0, st, (const float *)re, (const float *)im, (const float *)vplane, nx, ny, pitch, J_hi, J_lo, partials);
     }
-    observe_finalize_kernel<<<1, kThreads, 0, st>>>(partials, nblocks, norm_only ? 1 : OBS_Q, OBS_Q,
+    launch_pdl(observe_finalize_kernel, 1, kThreads, 0, st, partials, nblocks, norm_only ? 1 : OBS_Q, OBS_Q,
                                                     result);
     count_launches(2);
     return cudaGetLastError();
@@ -451,10 +456,10 @@ cudaError_t launch_observe3(const void *re, const void *im, const void *vplane, 
     int64_t b = (nchunks + kThreads * 8 - 1) / (kThreads * 8);
     int nblocks = (int)(b < 1 ? 1 : (b > OBS_MAX_BLOCKS ? OBS_MAX_BLOCKS : b));
     if (f64)
-        observe3_kernel<double><<<nblocks, kThreads, 0, st>>>((const double *)re, (const double *)im, (const double *)vplane, nx, ny, nz, pitch, J, partials);
+        launch_pdl(observe3_kernel<double>, nblocks, kThreads, 0, st, (const double *)re, (const double *)im, (const double *)vplane, nx, ny, nz, pitch, J, partials);
     else
-        observe3_kernel<float><<<nblocks, kThreads, 0, st>>>((const float *)re, (const float *)im, (const float *)vplane, nx, ny, nz, pitch, J, partials);
-    observe_finalize_kernel<<<1, kThreads, 0, st>>>(partials, nblocks, OBS_Q3, OBS_Q3, result);
+        launch_pdl(observe3_kernel<float>, nblocks, kThreads, 0, st, (const float *)re, (const float *)im, (const float *)vplane, nx, ny, nz, pitch, J, partials);
+    launch_pdl(observe_finalize_kernel, 1, kThreads, 0, st, partials, nblocks, OBS_Q3, OBS_Q3, result);
     count_launches(2);
     return cudaGetLastError();
 }
@@ -466,9 +471,9 @@ cudaError_t launch_inner(const float *phi_re, const float *phi_im, const float *
     const int64_t nchunks = (int64_t)((nx + 3) / 4) * ny;
     int64_t b = (nchunks + kThreads * 8 - 1) / (kThreads * 8);
     int nblocks = (int)(b < 1 ? 1 : (b > OBS_MAX_BLOCKS ? OBS_MAX_BLOCKS : b));
-    inner_f32_kernel<<<nblocks, kThreads, 0, st>>>(phi_re, phi_im, psi_re, psi_im, nx, ny, pitch,
+    launch_pdl(inner_f32_kernel, nblocks, kThreads, 0, st, phi_re, phi_im, psi_re, psi_im, nx, ny, pitch,
                                                    partials);
-    observe_finalize_kernel<<<1, kThreads, 0, st>>>(partials, nblocks, 2, OBS_Q, result);
+    launch_pdl(observe_finalize_kernel, 1, kThreads, 0, st, partials, nblocks, 2, OBS_Q, result);
     count_launches(2);
     return cudaGetLastError();
 }
