@@ -19,8 +19,9 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(ROOT, "_build")
 LIB = os.path.join(PKG, "libtrotter.so")
-SOURCES = ["api.cu", "plain.cu", "fused.cu", "reduce.cu", "adjoint.cu", "server.cu",
-           "noalloc.cu", "lattice3d.cu", "selftest.cu"]
+SOURCES = ["api.cu", "plain.cu", "reduce.cu", "adjoint.cu", "server.cu", "noalloc.cu",
+           "lattice3d.cu", "selftest.cu"]
+FUSED_PARTS = 16   # fused.cu is compiled in parts (-DTS_FUSED_PART=n), in parallel
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -32,7 +33,7 @@ def nvcc() -> str:
 
 
 def _flags(verbose: bool):
-    f = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I" + INCLUDE,
+    f = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-diag-suppress", "177", "-Xcompiler", "-fPIC", "-I" + INCLUDE,
                 "-I" + CSRC]
     if verbose:
         f += ["-Xptxas", "-v"]
@@ -46,19 +47,22 @@ def _headers():
 
 def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(BUILD, exist_ok=True)
-    srcs = list(SOURCES)
+    # (source, object, extra flags); fused.cu's parts first, they take longest
+    units = [("fused.cu", "fused_%d.o" % n, ["-DTS_FUSED_PART=%d" % n])
+             for n in reversed(range(FUSED_PARTS))]
+    units += [(s, s.replace(".cu", ".o"), []) for s in SOURCES]
     newest_dep = max(os.path.getmtime(p) for p in _headers())
     objs, jobs = [], []
-    for s in srcs:
+    for s, o, extra in units:
         src = os.path.join(CSRC, s)
-        obj = os.path.join(BUILD, s.replace(".cu", ".o"))
+        obj = os.path.join(BUILD, o)
         objs.append(obj)
         stale = (force or not os.path.exists(obj)
                  or os.path.getmtime(obj) < max(os.path.getmtime(src), newest_dep))
         if stale:
-            jobs.append([nvcc(), "-c", src, "-o", obj] + _flags(verbose))
+            jobs.append([nvcc(), "-c", src, "-o", obj] + extra + _flags(verbose))
     if jobs:
-        with cf.ThreadPoolExecutor(max_workers=len(jobs)) as ex:
+        with cf.ThreadPoolExecutor(max_workers=os.cpu_count() or 4) as ex:
             results = list(ex.map(lambda c: subprocess.run(c, capture_output=True, text=True), jobs))
         for cmd, r in zip(jobs, results):
             if verbose or r.returncode != 0:

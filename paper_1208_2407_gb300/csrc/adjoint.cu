@@ -272,6 +272,12 @@ ts_status ts_adjoint_backward_depth(ts_grid *g, void *ws, size_t ws_bytes, int K
     bw.g_ih = (float *)plane(WS_G + 2);
     bw.g_il = (float *)plane(WS_G + 3);
 
+    const double th = -g->theta;
+    const bool scaled = std::fabs(th) <= ts::SCALED_MAX_THETA;
+    const double sub[ts::FUSED_ADJ_MAX_K] = {th, th, th, th};
+    ts::ScaledCoef sc;
+    int sc_k = 0;
+
     int q = 0;   // psi and lambda in quad q (0: QA, 1: QB)
     auto quad = [&](int i) { return i ? WS_QB : WS_QA; };
     for (int64_t k = w.n_ck - 1; k >= 0; --k) {
@@ -282,6 +288,11 @@ ts_status ts_adjoint_backward_depth(ts_grid *g, void *ws, size_t ws_bytes, int K
         if (e != cudaSuccess) return cuda_err(e, "ts_adjoint_backward: restore checkpoint");
         for (int64_t i = n; i > 0;) {            // steps i, i - 1, ..., i - kk + 1 of the segment
             const int kk = (int)std::min<int64_t>(KA, i);
+            if (scaled && kk != sc_k) {
+                ts::scaled_coef(sub, kk, nx, ny, 1, sc);
+                sc_k = kk;
+            }
+            bw.sc = scaled ? &sc : nullptr;
             bw.tm_state = &tmQ[q];
             bw.out_re = (float *)plane(quad(q ^ 1));
             bw.out_im = (float *)plane(quad(q ^ 1) + 1);

@@ -38,11 +38,11 @@ ts_status cuda_fail(cudaError_t e, const char *what)
 constexpr int64_t kMaxSide = int64_t(1) << 20;
 
 // Depth of the fused path when the caller passes K = 0.  On one GB300 at
-// 8192^2 (site-steps/s): K=1 2.2e11, K=2 5.2e11, K=3 7.5e11, K=4 7.75e11,
-// K=5 7.2e11.  K = 3 runs at 88 % of the HBM copy bandwidth; K = 4 is 4 %
-// faster there but bound by instruction latency, so its speed follows the SM
-// clock (which drops under a power cap) while K = 3's follows HBM.
-int auto_depth() { return 3; }
+// 8192^2 (site-steps/s) with scaled rotations: K=2 4.6e11, K=3 8.0e11, K=4
+// 9.4e11, K=5 8.9e11, K=6 9.1e11; at 2048^2 K=3 4.7e11, K=4 4.8e11, K=5 4.6e11.
+// In the lifting form (larger angles): K=2 5.2e11, K=3 7.5e11 (88 % of the HBM
+// copy bandwidth), K=4 7.8e11, but K=4 is slower than K=3 at 2048^2.
+int auto_depth(bool scaled = true) { return scaled ? 4 : 3; }
 constexpr int kPlanes = 7;   // re_a, im_a, re_b, im_b, gamma_V, s_V, V
 
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -116,6 +116,78 @@ RotCoef rot_coef(double theta)
                    std::sin(2.0 * theta), std::tan(theta)};
 }
 
+void scaled_coef(const double *sub, int K, int64_t nx, int64_t ny, int64_t nz, ScaledCoef &c)
+{
+    std::memset(&c, 0, sizeof(c));
+    // Each tangent is rounded to FP32; the angle that a later sweep of the same
+    // family still owes takes up the error of the earlier ones, so that the
+    // sum over the launch is off by about one rounding, not K of them.
+    auto tan32 = [](double a) { return (float)std::tan(a); };
+    auto angle = [](float t) { return std::atan((double)t); };
+    const bool u4 = K == 5 && sub[2] != sub[0];
+    c.to_a = tan32(sub[0]);
+    c.to_b = tan32(2.0 * sub[0] - angle(c.to_a));
+    c.to_sub = u4 ? tan32(sub[2]) : c.to_a;
+    c.te_mid = tan32(2.0 * sub[0]);
+    c.te_ab = u4 ? tan32(sub[0] + sub[2]) : c.te_mid;
+    double sum = 0.0;
+    for (int i = 0; i < K; ++i) sum += 2.0 * sub[i];
+    double mid = 0.0;
+    for (int k = 1; k < K; ++k) mid += angle(u4 && (k == 2 || k == 3) ? c.te_ab : c.te_mid);
+    c.te_end = tan32(0.5 * (sum - mid));
+
+    auto te = [&](int k) -> double {
+        return k == 0 || k == K ? c.te_end : u4 && (k == 2 || k == 3) ? c.te_ab : c.te_mid;
+    };
+    auto to = [&](int m) -> double {
+        return u4 && m / 2 == 2 ? c.to_sub : (m & 1) ? c.to_b : c.to_a;
+    };
+    auto grow = [](double t) { return std::sqrt(1.0 + t * t); };   // 1 / cos
+    // 1 / rho of a site left out by the odd sweeps (the first one, and the last
+    // one of an even side) before even sweep k, and of one left out by the
+    // even sweeps (the last one of an odd side) before odd sweep m: what the
+    // others have grown by
+    double odd = 1.0, even = 1.0;
+    for (int k = 0; k <= K; ++k) {
+        c.edge.elo[k] = (float)(te(k) / odd);
+        c.edge.ehi[k] = (float)(te(k) * odd);
+        if (k == K) break;
+        odd *= grow(to(2 * k));
+        even *= grow(te(k));
+        for (int m = 2 * k; m <= 2 * k + 1; ++m) {
+            c.edge.olo[m] = (float)(to(m) / even);
+            c.edge.ohi[m] = (float)(to(m) * even);
+        }
+        if (k < FUSED_ADJ_MAX_K) {   // the phase of step k: odd sweeps to 2k, even to k
+            const double s[3] = {1.0 / (odd * even), 1.0, 1.0};
+            auto at = [&](int place, int64_t n) {
+                return place == 0 ? s[0]
+                       : n == 1   ? 1.0
+                       : place == 1 || n % 2 == 0 ? 1.0 / even : 1.0 / odd;
+            };
+            for (int y = 0; y < 3; ++y)
+                for (int x = 0; x < 3; ++x) {
+                    const double f = at(y, ny) * at(x, nx);
+                    c.edge.f[k][3 * y + x] = (float)(f * f);
+                }
+        }
+        odd *= grow(to(2 * k + 1));
+    }
+    even *= grow(te(K));
+    auto scale = [&](int place, int64_t n) {
+        return place == 0             ? 1.0 / (odd * even)
+               : n == 1               ? 1.0
+               : place == 1 || n % 2 == 0 ? 1.0 / even
+                                          : 1.0 / odd;
+    };
+    for (int z = 0; z < 3; ++z)
+        for (int y = 0; y < 3; ++y)
+            for (int x = 0; x < 3; ++x) {
+                const double sz = nz > 1 ? scale(z, nz) : 1.0;
+                c.edge.h[9 * z + 3 * y + x] = (float)(1.0 - sz * scale(y, ny) * scale(x, nx));
+            }
+}
+
 void grid_set_coefficients(ts_grid *g, double dt, double theta, cudaStream_t st)
 {
     g->dt = dt;
@@ -148,14 +220,20 @@ void grid_write_desc(ts_grid *g, cudaStream_t st)
     d.g1 = (float)g->g1;
     d.t2 = (float)g->t2;
     d.s2 = (float)g->s2;
+    const double sub[FUSED_MAX_K] = {g->theta, g->theta, g->theta, g->theta,
+                                     g->theta, g->theta, g->theta, g->theta};
+    for (int K = 1; K <= FUSED_MAX_K; ++K)
+        scaled_coef(sub, K, g->L.nx, g->L.ny, g->L.nz, d.sc[K - 1]);
     // pageable source: the call returns once the host struct is staged, and
     // the device copy lands in stream order before later kernels read it
     cudaMemcpyAsync(g->desc_dev, &d, sizeof(GridDesc), cudaMemcpyHostToDevice, st);
 }
 
-cudaError_t evolve_multi(ts_grid *const *gs, const int64_t *steps, int n, int K, cudaStream_t st)
+cudaError_t evolve_multi(ts_grid *const *gs, const int64_t *steps, int n, int K, bool scaled,
+                         cudaStream_t st)
 {
     if (n == 0) return cudaSuccess;
+    if (!scaled && K > FUSED_LIFT_MAX_K) K = FUSED_LIFT_MAX_K;
     // Each grid runs floor(steps/K) launches at depth K, then one at depth
     // steps % K -- the same sequence as evolving it alone.  All grids with a
     // launch left share each launch; a table is rebuilt when the set changes.
@@ -180,12 +258,12 @@ cudaError_t evolve_multi(ts_grid *const *gs, const int64_t *steps, int n, int K,
             hx.push_back((int)gs[i]->L.nx);
             hy.push_back((int)gs[i]->L.ny);
         }
-        const MultiPlan plan = fused_multi_plan(depth, (int)h.size(), hx.data(), hy.data(), h.data());
+        const MultiPlan plan = fused_multi_plan(depth, scaled, (int)h.size(), hx.data(), hy.data(), h.data());
         if (plan.warps < 1) return cudaErrorInvalidConfiguration;
         cudaError_t err = cudaMemcpyAsync(tab, h.data(), sizeof(EpochEntry) * h.size(),
                                           cudaMemcpyHostToDevice, st);
         for (int64_t t = 0; t < launches && err == cudaSuccess; ++t)
-            err = launch_fused_multi(depth, tab, (int)h.size(), plan, (int)(t & 1),
+            err = launch_fused_multi(depth, scaled, tab, (int)h.size(), plan, (int)(t & 1),
                                      gs[idx[0]]->err, st);
         if (err == cudaSuccess && (launches & 1))
             for (int i : idx) gs[i]->cur ^= 1;
@@ -746,15 +824,26 @@ ts_status merged_run(ts_grid *g, int64_t n, SubAt sub, cudaStream_t st)
 }  // extern "C++"
 
 // `steps` second-order steps on the fused path at depth K (a remainder runs
-// at a smaller depth), with the coefficients c and the phase table map tm.
-ts_status fused_run(ts_grid *g, int64_t steps, int K, const ts::RotCoef &c,
-                    const CUtensorMap *tm, cudaStream_t st, const double *drive_adt = nullptr)
+// at a smaller depth), at kinetic half angle theta with the phase table map tm.
+ts_status fused_run(ts_grid *g, int64_t steps, int K, double theta, const CUtensorMap *tm,
+                    cudaStream_t st, const double *drive_adt = nullptr)
 {
     if (!g->tmaps_ok) return fail(TS_ERR_STATE, "fused path: tensor maps missing");
+    const bool scaled = std::fabs(theta) <= ts::SCALED_MAX_THETA;
+    if (!scaled && K > ts::FUSED_LIFT_MAX_K) K = ts::FUSED_LIFT_MAX_K;
+    const ts::RotCoef c = ts::rot_coef(theta);
+    const double sub[ts::FUSED_MAX_K] = {theta, theta, theta, theta, theta, theta, theta, theta};
+    ts::ScaledCoef sc;
+    int sc_k = 0;
     int64_t left = steps;
     while (left > 0) {
         const int k = (int)(left >= K ? K : left);
+        if (scaled && k != sc_k) {
+            ts::scaled_coef(sub, k, g->L.nx, g->rows(), 1, sc);
+            sc_k = k;
+        }
         ts::FusedLaunch a;
+        a.sc = scaled ? &sc : nullptr;
         a.tm_state = &g->tm_state[g->cur];
         a.tm_phase = tm;
         a.out_re = (float *)g->re_other();
@@ -791,7 +880,7 @@ ts_status plain_steps(ts_grid *g, int64_t steps, cudaStream_t st)
 
 ts_status fused_steps(ts_grid *g, int64_t steps, int K, cudaStream_t st)
 {
-    return fused_run(g, steps, K, grid_coef(g), &g->tm_phase, st);
+    return fused_run(g, steps, K, g->theta, &g->tm_phase, st);
 }
 
 // Fourth-order steps (Eq. fourthorder): the substeps a = U2(p dt) and
@@ -810,8 +899,12 @@ ts_status evolve3_fused(ts_grid *g, int64_t steps, cudaStream_t st)
 {
     if (!g->tmaps_ok) return fail(TS_ERR_STATE, "fused path: tensor maps missing");
     const ts::RotCoef c = grid_coef(g);
+    const bool scaled = std::fabs(g->theta) <= ts::SCALED_MAX_THETA;
+    ts::ScaledCoef sc;
+    if (scaled) ts::scaled_coef(&g->theta, 1, g->L.nx, g->L.ny, g->L.nz, sc);
     for (int64_t n = 0; n < steps; ++n) {
         ts::FusedLaunch a;
+        a.sc = scaled ? &sc : nullptr;
         a.tm_state = &g->tm_state[g->cur];
         a.tm_phase = &g->tm_phase;
         a.out_re = (float *)g->re_other();
@@ -852,7 +945,7 @@ ts_status evolve_driven(ts_grid *g, int64_t steps, int K, bool plain, cudaStream
         // site-steps/s against 3.8e11 at depth 3)
         int depth = K == 0 ? ts::FUSED_DRIVE_MAX_K : K;
         if (depth > ts::FUSED_DRIVE_MAX_K) depth = ts::FUSED_DRIVE_MAX_K;
-        s = fused_run(g, steps, depth, grid_coef(g), &g->tm_drive, st, adt.data());
+        s = fused_run(g, steps, depth, g->theta, &g->tm_drive, st, adt.data());
     }
     if (s == TS_OK) g->drive_pos += steps;
     return s;
@@ -868,8 +961,14 @@ ts_status fused_u4_steps(ts_grid *g, int64_t steps, cudaStream_t st)
     const ts::RotCoef &A = g->sub[0], &B = g->sub[1];
     const double p4 = 1.0 / (4.0 - std::cbrt(4.0));
     const ts::RotCoef AB = ts::rot_coef((1.0 - 3.0 * p4) * g->theta);   // angle a + b
+    const double wa = p4 * g->theta, wb = (1.0 - 4.0 * p4) * g->theta;
+    const bool scaled = std::fabs(wb) <= ts::SCALED_MAX_THETA;   // the larger of the two
+    const double sub[5] = {wa, wa, wb, wa, wa};
+    ts::ScaledCoef sc;
+    if (scaled) ts::scaled_coef(sub, 5, g->L.nx, g->rows(), 1, sc);
     for (int64_t n = 0; n < steps; ++n) {
         ts::FusedLaunch a;
+        a.sc = scaled ? &sc : nullptr;
         a.tm_state = &g->tm_state[g->cur];
         a.tm_phase = &g->tm_phase;
         a.tm_b = &g->tm_phase_b;
@@ -900,19 +999,21 @@ ts_status evolve4(ts_grid *g, int64_t steps, int K, bool plain, cudaStream_t st)
 {
     if (!plain && K == 0) return fused_u4_steps(g, steps, st);
     const int depth = K;
+    const double p4 = 1.0 / (4.0 - std::cbrt(4.0));
+    const double w[2] = {p4, 1.0 - 4.0 * p4};
     auto run_a = [&](int64_t r) -> ts_status {
         if (plain) return plain_run(g, r, g->sub[0], g->pg(), g->ps(), st);
         const int64_t n = (r + depth - 1) / depth;
         for (int64_t i = 0; i < n; ++i) {
             const int64_t k = r / n + (i < r % n ? 1 : 0);
-            ts_status s = fused_run(g, k, (int)k, g->sub[0], &g->tm_phase, st);
+            ts_status s = fused_run(g, k, (int)k, w[0] * g->theta, &g->tm_phase, st);
             if (s != TS_OK) return s;
         }
         return TS_OK;
     };
     auto run_b = [&]() -> ts_status {
         if (plain) return plain_run(g, 1, g->sub[1], g->pg_b(), g->ps_b(), st);
-        return fused_run(g, 1, 1, g->sub[1], &g->tm_phase_b, st);
+        return fused_run(g, 1, 1, w[1] * g->theta, &g->tm_phase_b, st);
     };
     ts_status s = run_a(2);
     for (int64_t n = 0; n < steps && s == TS_OK; ++n) {
@@ -985,7 +1086,8 @@ ts_status ts_evolve(ts_grid *g, int64_t steps, int K, void *stream)
     // (|2 theta| <= pi/2).  Larger angles -- far beyond any useful Trotter
     // step -- run the one-sweep-per-kernel path.
     if (std::fabs(g->theta) > 0.25 * M_PI) return plain_steps(g, steps, st);
-    return fused_steps(g, steps, K == 0 ? auto_depth() : K, st);
+    const bool scaled = std::fabs(g->theta) <= ts::SCALED_MAX_THETA;
+    return fused_steps(g, steps, K == 0 ? auto_depth(scaled) : K, st);
 }
 
 ts_status ts_check_wait_timeout(ts_grid *g, int64_t limit_ns, void *stream)
@@ -1016,11 +1118,11 @@ ts_status ts_evolve_batched(ts_grid *const *gs, int n, const int64_t *steps, int
     if (n < 0 || (n > 0 && (!gs || !steps))) return fail(TS_ERR_ARG, "ts_evolve_batched: bad arguments");
     if (K < 0 || K > ts::FUSED_MAX_K) return fail(TS_ERR_ARG, "ts_evolve_batched: K must be in [0, 8]");
     cudaStream_t st = (cudaStream_t)stream;
-    const int depth = K == 0 ? auto_depth() : K;
     // grids the multi-grid kernel can take: 2-D, FP32, second order, no
     // drive, |theta| <= pi/4; the rest evolve one by one
-    std::vector<ts_grid *> multi;
-    std::vector<int64_t> msteps;
+    // (those with scaled rotations, then those in the lifting form)
+    std::vector<ts_grid *> multi[2];
+    std::vector<int64_t> msteps[2];
     for (int i = 0; i < n; ++i) {
         if (!gs[i] || steps[i] < 0) return fail(TS_ERR_ARG, "ts_evolve_batched: grid %d", i);
         if (steps[i] == 0) continue;
@@ -1030,12 +1132,17 @@ ts_status ts_evolve_batched(ts_grid *const *gs, int n, const int64_t *steps, int
             ts_status s = ts_evolve(gs[i], steps[i], gs[i]->f64() ? 0 : K, stream);
             if (s != TS_OK) return s;
         } else {
-            multi.push_back(gs[i]);
-            msteps.push_back(steps[i]);
+            const int form = std::fabs(gs[i]->theta) <= ts::SCALED_MAX_THETA ? 0 : 1;
+            multi[form].push_back(gs[i]);
+            msteps[form].push_back(steps[i]);
         }
     }
-    cudaError_t e = ts::evolve_multi(multi.data(), msteps.data(), (int)multi.size(), depth, st);
-    if (e != cudaSuccess) return cuda_fail(e, "ts_evolve_batched: multi-grid launch");
+    for (int form = 0; form < 2; ++form) {
+        const int depth = K == 0 ? auto_depth(form == 0) : K;
+        cudaError_t e = ts::evolve_multi(multi[form].data(), msteps[form].data(),
+                                         (int)multi[form].size(), depth, form == 0, st);
+        if (e != cudaSuccess) return cuda_fail(e, "ts_evolve_batched: multi-grid launch");
+    }
     return TS_OK;
 }
 

@@ -60,7 +60,35 @@
 #include "internal.h"
 #include "mbar.cuh"
 
+// This file is compiled in parts (build.py), so that its kernels build in
+// parallel: part 0 has the dispatch and the plans, the others instantiate the
+// kernels listed at the end of the file.
+#ifndef TS_FUSED_PART
+#error "compile fused.cu with -DTS_FUSED_PART=n"
+#endif
+
 namespace ts {
+
+// Resident blocks per SM and SM count of a kernel at its dynamic shared
+// memory size, set up once per kernel (the first caller's function-local
+// static initialisation, which C++ runs exactly once even when threads race).
+struct Occupancy {
+    cudaError_t err;
+    int blocks_per_sm, num_sms;
+};
+
+
+// Launches of one kernel: K steps of a mode, in the lifting form or with
+// scaled rotations (SC); one 3-D step; the multi-grid kernel.
+template <int K, int MODE, bool SC>
+cudaError_t launch_k(const FusedLaunch &a, cudaStream_t st);
+template <bool SC>
+cudaError_t launch3_k(const FusedLaunch &a, int nz, cudaStream_t st);
+template <int K, bool SC>
+const Occupancy &multi_occupancy();
+template <int K, bool SC>
+cudaError_t launch_multi_k(const EpochEntry *tab, int n_grids, const MultiPlan &plan, int flip,
+                           int *err, cudaStream_t st);
 
 namespace {
 
@@ -87,6 +115,9 @@ namespace {
 #endif
 #ifndef TS_FUSED_MIN_BLOCKS_K4   // ... for K = 4
 #define TS_FUSED_MIN_BLOCKS_K4 1
+#endif
+#ifndef TS_FUSED_SC_MIN_BLOCKS_K4     // ... and with scaled rotations: 168 registers
+#define TS_FUSED_SC_MIN_BLOCKS_K4 12
 #endif
 #ifndef TS_FUSED_MULTI_MIN_BLOCKS_K3   // multi-grid kernel, K = 3
 #define TS_FUSED_MULTI_MIN_BLOCKS_K3 1
@@ -153,11 +184,11 @@ __host__ __device__ constexpr int state_planes(int mode) { return mode == 5 || m
 // __launch_bounds__ minimum resident blocks of the single-grid kernel; the
 // backward adjoint steps (MODE 5) carry two states and are not held to the
 // forward depth's occupancy
-__host__ __device__ constexpr int min_blocks(int K, int MODE = 0)
+__host__ __device__ constexpr int min_blocks(int K, int MODE, bool SC)
 {
     return MODE == 5   ? TS_FUSED_MIN_BLOCKS
            : K == 3    ? TS_FUSED_MIN_BLOCKS_K3
-           : K == 4    ? TS_FUSED_MIN_BLOCKS_K4
+           : K == 4    ? (SC ? TS_FUSED_SC_MIN_BLOCKS_K4 : TS_FUSED_MIN_BLOCKS_K4)
                        : TS_FUSED_MIN_BLOCKS;
 }
 
@@ -169,7 +200,26 @@ __host__ __device__ constexpr int multi_min_blocks(int K)
                     : TS_FUSED_MIN_BLOCKS;
 }
 
-template <int K, int PP = 2, bool BRING = false, int SP = 2, int M = 0>
+// Scaled rotations (see pair_s): a warp's coefficients in shared memory, written
+// once per segment.  recv has what the columns of a lane receive in each X
+// sweep, by the kind of lane: only the lanes at the grid's two edges differ
+// from the rest, so a sweep reads 16 bytes, mostly the same ones for the whole
+// warp, and strips at the edges cost what the others do.  (With selects instead
+// of the table, for edge strips alone, those strips took 1.4 times as long and
+// held up the launch.)  lohi, h and f serve the rows at the edges.  Sweep
+// k < K + 1 is even sweep k, sweep K + 1 + m odd sweep m.
+template <int K, bool ADJ>
+struct EdgeTab {
+    static constexpr int SWEEPS = 3 * K + 1, CLASSES = 8;
+    float4 recv[SWEEPS][CLASSES];
+    float4 hrow[2][CLASSES];    // h and f of the columns of a lane, bulk rows
+    float4 frow[ADJ ? K : 1][CLASSES];
+    float2 lohi[SWEEPS];
+    float h[18];     // 3 x 3 (rows by columns); MODE 6: of slab z, then of slab z + 1
+    float f[ADJ ? 9 * K : 1];
+};
+
+template <int K, int PP = 2, bool BRING = false, int SP = 2, int M = 0, bool SC = false>
 struct Cfg {
     // MODE 6 (3-D steps): one CTA of TS_FUSED3D_WARPS warps, two slabs each
     static constexpr int WPC = M == 6 ? TS_FUSED3D_WARPS
@@ -180,12 +230,18 @@ struct Cfg {
                               : K == 1 ? TS_FUSED_PF_K1
                               : K == 2 ? TS_FUSED_PF_K2
                                        : TS_FUSED_PF_DEEP;
-    static constexpr bool PINGPONG = M != 5 && K >= TS_FUSED_PINGPONG_MIN_K && K <= TS_FUSED_PINGPONG_MAX_K;
-    // The backward adjoint steps carry two states: one carry set, which
-    // leaves registers for the deeper pipelines, and interior row pairs one
-    // per loop trip instead of two, a smaller loop body (2-3 % faster for
-    // them; about 1 % slower for one state and for the 3-D steps).
-    static constexpr bool ONE_PAIR = M == 5;
+    static constexpr bool PINGPONG =
+        !SC && M != 5 && K >= TS_FUSED_PINGPONG_MIN_K && K <= TS_FUSED_PINGPONG_MAX_K;
+    // Scaled rotations leave fewer instructions per row pair, so what the carry
+    // sets and the unrolled body cost counts for more.  One carry set (at the
+    // price of moving 2K rows per row pair) takes depth 4 from 219 to 166
+    // registers, 8 to 12 warps per SM: 8.8e11 -> 9.4e11 site-steps/s at 8192^2.
+    // One row pair per loop trip halves the loop body, which measured 16 %
+    // faster at 512^2 (depths 3 and 4) and 4 % at depth 5, 8192^2, and even at
+    // depth 4; a body of K + 1 row pairs, which moves no rows at all, ran 24 %
+    // slower: the instruction caches are what it outgrows.  The backward
+    // adjoint steps (two states) take the same form in either kind.
+    static constexpr bool ONE_PAIR = M == 5 || (SC && K >= 2);
     // packed FP32 FMAs in the Y sweeps and the phase: 0 never, 1 for every
     // depth but 2 (where the scalar form measured faster), 2 always
     static constexpr bool PACKED = TS_FUSED_FFMA2 == 2 || (TS_FUSED_FFMA2 == 1 && K != 2);
@@ -215,13 +271,16 @@ struct Cfg {
     // MODE 5: G's rows for the next commit, staged by cp.async (two rows of
     // four planes, [row][plane][lane] as float4)
     static constexpr int GST_BYTES = M == 5 ? 4096 : 0;
-    static constexpr int WARP_SMEM = NSS * SSLOT + NSP * PSLOT + NSB * SLOT_BYTES + SUMS_BYTES + GST_BYTES;
+    // scaled rotations: the warp's edge values (EdgeTab)
+    static constexpr int EDGE_BYTES = SC ? (sizeof(EdgeTab<K, M == 5>) + 127) / 128 * 128 : 0;
+    static constexpr int WARP_SMEM = NSS * SSLOT + NSP * PSLOT + NSB * SLOT_BYTES + SUMS_BYTES +
+                                     GST_BYTES + EDGE_BYTES;
     static constexpr int SMEM = 1024 + WPC * (WARP_SMEM + NBAR * 8);
 };
 
 // The configuration of a mode's kernel at depth K.
-template <int K, int MODE>
-using CfgM = Cfg<K, phase_planes(MODE), MODE == 4, state_planes(MODE), MODE>;
+template <int K, int MODE, bool SC>
+using CfgM = Cfg<K, phase_planes(MODE), MODE == 4, state_planes(MODE), MODE, SC>;
 
 // Four columns of one row of one state, held by one lane.
 struct Frag {
@@ -269,6 +328,11 @@ struct KParams {
     // s2 are the a substep's; the b substep's angle (lifting tb, sb; versine
     // gb) and the merged angle of an a-b boundary (lifting tab, sab)
     float tb, sb, gb, tab, sab;
+    // scaled rotations (SC kernels): see ScaledCoef.  ed points at the
+    // values of pairs and sites on the grid's edges
+    float te_end, te_mid, to_a, to_b;
+    float te_ab, to_sub;     // MODE 4: even sweeps a + b, odd sweeps of b
+    const ScaledEdge *ed;
 };
 
 // ---- PTX wrappers (the mbarrier helpers are in mbar.cuh) ------------------
@@ -327,6 +391,89 @@ __device__ __forceinline__ void x_odd(Frag &f, const XOdd &c)
     rot1(f.re.x, f.im.x, pr, pi, c.gL, c.sL);
 }
 
+// Scaled rotations (SC kernels).  A pair rotation divided by its cosine,
+//   a' = a + i t b,  b' = b + i t a,   t = tan(theta),
+// takes one FMA per real component: 4 per pair against the lifting form's 6
+// (and the versine form's 8).  A sweep so applied leaves every paired site
+// 1/cos(theta) too large; all sites share that factor, so it commutes with
+// every later factor and the launch takes it out once, at the end, by
+// a -= h a with h = 1 - (product of the cosines).  A site at the grid's edge
+// that a sweep leaves unpaired does not grow: beside its neighbours it is then
+// rho = cos(theta) times too small, so its later pairs take the coefficients
+// t rho_a / rho_b (into a) and t rho_b / rho_a (into b), and it has its own h.
+// These values are the same along an edge and depend on the sweep's place in
+// the launch only (ScaledEdge, computed in FP64 from the rounded t).
+__device__ __forceinline__ void pair_s(float &ar, float &ai, float &br, float &bi, float ta,
+                                       float tb)
+{
+    const float r = ar, m = ai;
+    ar = fmaf(-ta, bi, ar);
+    ai = fmaf(ta, br, ai);
+    br = fmaf(-tb, m, br);
+    bi = fmaf(tb, r, bi);
+}
+
+// what a lane's columns receive from their partners in an X sweep
+struct Recv {
+    float c0, c1, c2, c3;
+};
+
+__device__ __forceinline__ void x_even_s(Frag &f, const Recv &e)
+{
+    pair_s(f.re.x, f.im.x, f.re.y, f.im.y, e.c0, e.c1);
+    pair_s(f.re.z, f.im.z, f.re.w, f.im.w, e.c2, e.c3);
+}
+
+__device__ __forceinline__ void x_odd_s(Frag &f, const Recv &o)
+{
+    const float nr = __shfl_down_sync(FULL, f.re.x, 1);
+    const float ni = __shfl_down_sync(FULL, f.im.x, 1);
+    const float pr = __shfl_up_sync(FULL, f.re.w, 1);
+    const float pi = __shfl_up_sync(FULL, f.im.w, 1);
+    pair_s(f.re.y, f.im.y, f.re.z, f.im.z, o.c1, o.c2);
+    f.re.w = fmaf(-o.c3, ni, f.re.w);
+    f.im.w = fmaf(o.c3, nr, f.im.w);
+    f.re.x = fmaf(-o.c0, pi, f.re.x);
+    f.im.x = fmaf(o.c0, pr, f.im.x);
+}
+
+__device__ __forceinline__ void x_even_s(Frag2 &f, const Recv &e)
+{
+    x_even_s(f.a, e);
+    x_even_s(f.b, e);
+}
+
+__device__ __forceinline__ void x_odd_s(Frag2 &f, const Recv &o)
+{
+    x_odd_s(f.a, o);
+    x_odd_s(f.b, o);
+}
+
+// How a pair lies on the grid, and what its members receive at a sweep whose
+// bulk coefficient is t: at an edge the edge member takes lo, its partner hi.
+// (A pair with both members on an edge, a side of two sites, is a bulk pair.)
+enum : int { PAIR_OFF = 0, PAIR_BULK = 1, PAIR_LOW = 2, PAIR_HIGH = 3 };
+
+__device__ __forceinline__ int pair_kind(int a, int n)
+{
+    return a < 0 || a + 1 >= n      ? PAIR_OFF
+           : n == 2                 ? PAIR_BULK
+           : a == 0                 ? PAIR_LOW
+           : a + 2 == n             ? PAIR_HIGH
+                                    : PAIR_BULK;
+}
+
+__device__ __forceinline__ void pair_coef(int kind, float t, float lo, float hi, float &first,
+                                          float &second)
+{
+    first = kind == PAIR_BULK ? t : kind == PAIR_LOW ? lo : kind == PAIR_HIGH ? hi : 0.f;
+    second = kind == PAIR_BULK ? t : kind == PAIR_LOW ? hi : kind == PAIR_HIGH ? lo : 0.f;
+}
+
+// A site's place along an axis of n sites, for the tables of ScaledEdge:
+// 0 bulk, 1 the first site, 2 the last.
+__device__ __forceinline__ int edge_kind(int i, int n) { return i == 0 ? 1 : i == n - 1 ? 2 : 0; }
+
 // Packed forms (Cfg<K>::PACKED): the column halves (x, y) and (z, w) of a
 // lane's float4 are register pairs, and __ffma2_rn applies one FMA to both
 // elements with the rounding of fmaf, so the results are bit for bit those of
@@ -381,6 +528,52 @@ __device__ __forceinline__ void y_pair(Frag &a, Frag &b, float t, float s)
     rot_lift(a.re.z, a.im.z, b.re.z, b.im.z, t, s);
     rot_lift(a.re.w, a.im.w, b.re.w, b.im.w, t, s);
     }
+}
+
+// Scaled Y (or Z) pair rotation of two rows; a receives ta, b receives tb.
+template <bool PACKED>
+__device__ __forceinline__ void y_pair_s(Frag &a, Frag &b, float ta, float tb)
+{
+    if constexpr (PACKED) {
+        const float2 na = make_float2(-ta, -ta), pa = make_float2(ta, ta);
+        const float2 nb = make_float2(-tb, -tb), pb = make_float2(tb, tb);
+        auto half = [&](float2 &ar, float2 &ai, float2 &br, float2 &bi) {
+            const float2 r = ar, m = ai;
+            ar = __ffma2_rn(na, bi, ar);
+            ai = __ffma2_rn(pa, br, ai);
+            br = __ffma2_rn(nb, m, br);
+            bi = __ffma2_rn(pb, r, bi);
+        };
+        float2 ar = lo2(a.re), ai = lo2(a.im), br = lo2(b.re), bi = lo2(b.im);
+        float2 cr = hi2(a.re), ci = hi2(a.im), dr = hi2(b.re), di = hi2(b.im);
+        half(ar, ai, br, bi);
+        half(cr, ci, dr, di);
+        a.re = join2(ar, cr);
+        a.im = join2(ai, ci);
+        b.re = join2(br, dr);
+        b.im = join2(bi, di);
+    } else {
+        pair_s(a.re.x, a.im.x, b.re.x, b.im.x, ta, tb);
+        pair_s(a.re.y, a.im.y, b.re.y, b.im.y, ta, tb);
+        pair_s(a.re.z, a.im.z, b.re.z, b.im.z, ta, tb);
+        pair_s(a.re.w, a.im.w, b.re.w, b.im.w, ta, tb);
+    }
+}
+
+template <bool PACKED>
+__device__ __forceinline__ void y_pair_s(Frag2 &a, Frag2 &b, float ta, float tb)
+{
+    y_pair_s<PACKED>(a.a, b.a, ta, tb);
+    y_pair_s<PACKED>(a.b, b.b, ta, tb);
+}
+
+// a -= h a, h per column
+__device__ __forceinline__ void unscale(Frag &f, float4 h)
+{
+    const float2 n0 = make_float2(-h.x, -h.y), n1 = make_float2(-h.z, -h.w);
+    const float2 r0 = lo2(f.re), r1 = hi2(f.re), m0 = lo2(f.im), m1 = hi2(f.im);
+    f.re = join2(__ffma2_rn(n0, r0, r0), __ffma2_rn(n1, r1, r1));
+    f.im = join2(__ffma2_rn(n0, m0, m0), __ffma2_rn(n1, m1, m1));
 }
 
 template <bool PACKED>
@@ -553,9 +746,36 @@ struct Owned {
     int Y0, Y1;        // output rows [Y0, Y1)
     int xg;            // the lane's first column
     bool lane_ok;      // the lane's 4 columns are inside the valid strip and < nx
+    unsigned cols;     // SC: the places of the lane's columns along x (2 bits each)
+    const unsigned char *edge;   // SC: the warp's EdgeTab
+    int lane_class;    // SC: the lane's entry in it
     float4 *sums;      // MODE 5: the lane's running sums (shared memory)
     float4 *gst;       // MODE 5: the lane's staged G rows (shared memory)
 };
+
+__device__ __forceinline__ unsigned col_places(int xg, int nx)
+{
+    unsigned v = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v |= (unsigned)edge_kind(xg + i, nx) << (2 * i);
+    return v;
+}
+
+// Lanes with the same class receive the same coefficients in every sweep:
+// 0 off the grid, 1 inside, 2 holds the first column, 3 the last, 4 both,
+// 5 beside the lane whose first column is the last one, 6 that and the first.
+__device__ __forceinline__ int lane_class(int xg, int nx)
+{
+    const bool L = xg == 0, R = xg < nx && nx <= xg + 4, B = xg + 5 == nx;
+    return xg < 0 || xg >= nx ? 0 : L && R ? 4 : L && B ? 6 : L ? 2 : R ? 3 : B ? 5 : 1;
+}
+
+// the entries of a 3 x 3 edge table (rows by columns) for one row of the lane
+__device__ __forceinline__ float4 edge4(const float *tab, int row, int ny, unsigned cols)
+{
+    const float *t = tab + 3 * edge_kind(row, ny);
+    return make_float4(t[cols & 3], t[cols >> 2 & 3], t[cols >> 4 & 3], t[cols >> 6 & 3]);
+}
 
 __device__ __forceinline__ bool owns_row(const Owned &w, const KParams &p, int row)
 {
@@ -577,6 +797,17 @@ __device__ __forceinline__ Frag adj_term(const Frag &lt, const Frag &m)
                        fmaf(lt.re.z, m.im.z, -lt.im.z * m.re.z),
                        fmaf(lt.re.w, m.im.w, -lt.im.w * m.re.w));
     return t;
+}
+
+// a + f b (the scale of the step's phase point), per column
+__device__ __forceinline__ Frag frag_fma(const Frag &a, float4 f, const Frag &b)
+{
+    Frag r;
+    r.re = make_float4(fmaf(f.x, b.re.x, a.re.x), fmaf(f.y, b.re.y, a.re.y),
+                       fmaf(f.z, b.re.z, a.re.z), fmaf(f.w, b.re.w, a.re.w));
+    r.im = make_float4(fmaf(f.x, b.im.x, a.im.x), fmaf(f.y, b.im.y, a.im.y),
+                       fmaf(f.z, b.im.z, a.im.z), fmaf(f.w, b.im.w, a.im.w));
+    return r;
 }
 
 __device__ __forceinline__ Frag frag_add(const Frag &a, const Frag &b)
@@ -656,13 +887,18 @@ __device__ __forceinline__ void adj_commit(const Frag &t, int row, int slot, con
 // iteration to this step.  Step K - 1 adds the finished sum into G (owned
 // rows only; other rows' sums are never stored).  Each lane touches only its
 // own entries, so no synchronisation is needed.
-template <int K>
+// SC: both states carry the scale of the sweeps so far, whose square fP, fQ
+// (per column) takes out of the term.
+template <int K, bool SC>
 __device__ __forceinline__ void adj_step(int k, const Frag2 &P, const Frag2 &Q, int y1,
                                          Frag &carP, Frag &carQ, const Owned &w,
-                                         const KParams &p)
+                                         const KParams &p, float4 fP, float4 fQ)
 {
     Frag tP = adj_term(P.b, P.a), tQ = adj_term(Q.b, Q.a);
-    if (k > 0) {
+    if constexpr (SC) {
+        tP = frag_fma(k > 0 ? carP : zero_frag(), fP, tP);
+        tQ = frag_fma(k > 0 ? carQ : zero_frag(), fQ, tQ);
+    } else if (k > 0) {
         tP = frag_add(carP, tP);
         tQ = frag_add(carQ, tQ);
     }
@@ -700,7 +936,9 @@ __device__ __forceinline__ float4 neg4(float4 v) { return make_float4(-v.x, -v.y
 // -theta; the phase is conjugated here) that accumulate G at each step's
 // phase point, with the running sums of the rows in flight in shared memory
 // (updated in place).
-template <int K, bool INTERIOR, int MODE, typename S = StateT<MODE>>
+// SC: scaled rotations (see pair_s); INTERIOR then also means that none of the
+// strip's columns lies on an edge of the grid.  The rows leave scaled.
+template <int K, bool INTERIOR, int MODE, bool SC, typename S = StateT<MODE>>
 __device__ __forceinline__ void pipeline_step(const S (&cin)[2 * K], S (&cout)[2 * K],
                                               S a, S b, int yin, int j,
                                               const unsigned char *ring_p, int pos_p,
@@ -709,7 +947,7 @@ __device__ __forceinline__ void pipeline_step(const S (&cin)[2 * K], S (&cout)[2
                                               const Owned &w, S &O0, S &O1)
 {
     static_assert(MODE != 4 || K == 5, "the fused fourth-order step has five substeps");
-    using C = CfgM<K, MODE>;
+    using C = CfgM<K, MODE, SC>;
     constexpr bool CONJ = MODE == 5;   // backward steps: exp(+i V dt), sine -s_V
     // MODE 4: substep k of U4 = a a b a a is b for k == 2 (angle and table)
     auto is_b = [](int k) { return MODE == 4 && k == 2; };
@@ -725,24 +963,86 @@ __device__ __forceinline__ void pipeline_step(const S (&cin)[2 * K], S (&cout)[2
     auto slot_b = [&](int back) -> const unsigned char * {   // b-ring slot of row pair j - back
         return ring_b + ((cnt_b + j - back) % (C::NSB > 0 ? C::NSB : 1)) * SLOT_BYTES;
     };
+    // The sweeps of a launch, in order: even sweep 0, odd sweep 0, phase 0,
+    // odd 1, even 1, odd 2, phase 1, ..., phase K - 1, odd 2K - 1, even K (of
+    // each axis).  Odd sweep m belongs to substep m / 2, even sweep k joins
+    // substeps k - 1 and k (MODE 4: a and b differ).
+    auto mixed = [&](int k) { return k > 0 && k < K && is_b(k - 1) != is_b(k); };
+    auto te = [&](int k) { return mixed(k) ? p.te_ab : k == 0 || k == K ? p.te_end : p.te_mid; };
+    auto to = [&](int m) { return is_b(m / 2) ? p.to_sub : (m & 1) ? p.to_b : p.to_a; };
+    const EdgeTab<K, MODE == 5> *et = reinterpret_cast<const EdgeTab<K, MODE == 5> *>(w.edge);
+    auto XE = [&](S &f, int k) {
+        if constexpr (SC) {
+            const float4 r = et->recv[k][w.lane_class];
+            x_even_s(f, Recv{r.x, r.y, r.z, r.w});
+        } else {
+            x_even(f, mixed(k) ? c.Eab : k == 0 || k == K ? c.E1 : c.E2);
+        }
+    };
+    auto XO = [&](S &f, int m) {
+        if constexpr (SC) {
+            const float4 r = et->recv[K + 1 + m][w.lane_class];
+            x_odd_s(f, Recv{r.x, r.y, r.z, r.w});
+        } else {
+            x_odd(f, is_b(m / 2) ? c.Ob : c.O);
+        }
+    };
+    // Y sweeps of the rows (y, y + 1)
+    auto YE = [&](S &f0, S &f1, int y, int k) {
+        if constexpr (SC) {
+            float ta = te(k), tb = ta;
+            if constexpr (!INTERIOR) {
+                const float2 lh = et->lohi[k];
+                pair_coef(pair_kind(y, p.ny), te(k), lh.x, lh.y, ta, tb);
+            }
+            y_pair_s<C::PACKED>(f0, f1, ta, tb);
+        } else {
+            const float t = mixed(k) ? p.tab : k == 0 || k == K ? p.t1 : p.t2;
+            const float sn = mixed(k) ? p.sab : k == 0 || k == K ? p.s1 : p.s2;
+            const bool v = yok(y);
+            y_pair<C::PACKED>(f0, f1, v ? t : 0.f, v ? sn : 0.f);
+        }
+    };
+    auto YO = [&](S &f0, S &f1, int y, int m) {
+        if constexpr (SC) {
+            float ta = to(m), tb = ta;
+            if constexpr (!INTERIOR) {
+                const float2 lh = et->lohi[K + 1 + m];
+                pair_coef(pair_kind(y, p.ny), to(m), lh.x, lh.y, ta, tb);
+            }
+            y_pair_s<C::PACKED>(f0, f1, ta, tb);
+        } else {
+            const bool bk = is_b(m / 2), v = yok(y);
+            y_pair<C::PACKED>(f0, f1, v ? (bk ? p.tb : p.t1) : 0.f, v ? (bk ? p.sb : p.s1) : 0.f);
+        }
+    };
+    // MODE 5 at step k's phase point: rows (y, y + 1)
+    Frag carP, carQ;   // running sums handed from step k - 1 to step k
+    auto ADJ = [&](int k, const S &f0, const S &f1, int y) {
+        if constexpr (MODE == 5) {
+            float4 fP = {}, fQ = {};
+            if constexpr (SC) {
+                if constexpr (INTERIOR) {
+                    fP = fQ = et->frow[k][w.lane_class];
+                } else {
+                    fP = edge4(et->f + 9 * k, y, p.ny, w.cols);
+                    fQ = edge4(et->f + 9 * k, y + 1, p.ny, w.cols);
+                }
+            }
+            adj_step<K, SC>(k, f0, f1, y, carP, carQ, w, p, fP, fQ);
+        }
+    };
     // step 0, first half: Xe, Xo (row-local), Ye aligned, Yo shifted
-    x_even(a, c.E1);
-    x_even(b, c.E1);
-    x_odd(a, c.O);
-    x_odd(b, c.O);
-    {
-        const bool v = yok(yin);
-        y_pair<C::PACKED>(a, b, v ? p.t1 : 0.f, v ? p.s1 : 0.f);
-    }
+    XE(a, 0);
+    XE(b, 0);
+    XO(a, 0);
+    XO(b, 0);
+    YE(a, b, yin, 0);
     S P = cin[0], Q = a;          // rows (yin-1, yin)
-    {
-        const bool v = yok(yin - 1);
-        y_pair<C::PACKED>(P, Q, v ? p.t1 : 0.f, v ? p.s1 : 0.f);
-    }
+    YO(P, Q, yin - 1, 0);
     cout[0] = b;
     int y1 = yin - 1;
-    Frag carP, carQ;   // MODE 5: running sums handed from step k - 1 to step k
-    if constexpr (MODE == 5) adj_step<K>(0, P, Q, y1, carP, carQ, w, p);
+    ADJ(0, P, Q, y1);
     // the phase of step k on one row from phase slot sp (row 0 or 1 of the
     // slot): conjugated in a backward step (exp(+i V dt) has sine -s_V); with
     // the drive term for MODE 3; MODE 6 holds two slabs, each with its table
@@ -767,45 +1067,31 @@ __device__ __forceinline__ void pipeline_step(const S (&cin)[2 * K], S (&cout)[2
     }
 #pragma unroll
     for (int k = 1; k < K; ++k) {
-        // angles of the two steps that meet here (MODE 4: a or b) and of
-        // their merged factors (2a, or a + b)
-        const bool bp = is_b(k - 1), bk = is_b(k), mixed = bp != bk;
-        const float tp = bp ? p.tb : p.t1, sp_ = bp ? p.sb : p.s1;
-        const float tk = bk ? p.tb : p.t1, sk = bk ? p.sb : p.s1;
-        const float tm = mixed ? p.tab : p.t2, sm = mixed ? p.sab : p.s2;
-        const XOdd &Op = bp ? c.Ob : c.O, &Ok = bk ? c.Ob : c.O;
-        const XEven &Em = mixed ? c.Eab : c.E2;
-        {   // Yo (theta of step k-1), aligned on (y1, y1+1), y1 odd
-            const bool v = yok(y1);
-            y_pair<C::PACKED>(P, Q, v ? tp : 0.f, v ? sp_ : 0.f);
-        }
+        // while the pipeline fills, stage k has nothing to do: the first rows
+        // that the segment's output needs of it come at row pair 2k - 1
+        if (!INTERIOR && j < 2 * k - 1) return;
+        YO(P, Q, y1, 2 * k - 1);          // Yo of step k-1, aligned on (y1, y1+1), y1 odd
         // X group between two phases: Xo, Xe(merged), Xo
-        x_odd(P, Op);
-        x_odd(Q, Op);
-        x_even(P, Em);
-        x_even(Q, Em);
-        x_odd(P, Ok);
-        x_odd(Q, Ok);
+        XO(P, 2 * k - 1);
+        XO(Q, 2 * k - 1);
+        XE(P, k);
+        XE(Q, k);
+        XO(P, 2 * k);
+        XO(Q, 2 * k);
         S P2 = cin[2 * k - 1], Q2 = P;        // rows (y1-1, y1)
-        {   // Ye (merged), shifted: pair (y1-1, y1)
-            const bool v = yok(y1 - 1);
-            y_pair<C::PACKED>(P2, Q2, v ? tm : 0.f, v ? sm : 0.f);
-        }
+        YE(P2, Q2, y1 - 1, k);                // Ye (merged), shifted: pair (y1-1, y1)
         cout[2 * k - 1] = Q;
         P = cin[2 * k];                       // rows (y1-2, y1-1)
-        {   // Yo (theta of step k), shifted: pair (y1-2, y1-1)
-            const bool v = yok(y1 - 2);
-            y_pair<C::PACKED>(P, P2, v ? tk : 0.f, v ? sk : 0.f);
-        }
+        YO(P, P2, y1 - 2, 2 * k);             // Yo of step k, shifted: pair (y1-2, y1-1)
         cout[2 * k] = Q2;
         Q = P2;
         y1 -= 2;
-        if constexpr (MODE == 5) adj_step<K>(k, P, Q, y1, carP, carQ, w, p);
+        ADJ(k, P, Q, y1);
         // phase of step k on rows (y1, y1+1): rows 0 and 1 of slot j-k
         // (without PSHIFT, MODE 4: slot j-k-1 row 1, slot j-k row 0, and the
         // b substep's table from the b ring; MODE 5: the conjugate phase,
         // sine -s_V)
-        auto slot_k = [&](int back) { return bk ? slot_b(back) : slot_p(back); };
+        auto slot_k = [&](int back) { return is_b(k) ? slot_b(back) : slot_p(back); };
         if constexpr (C::PSHIFT) {
             if (INTERIOR || j - k >= 0) {   // rows 0 and 1 of slot j-k
                 phase_row(P, slot_p(k), 0, k);
@@ -817,21 +1103,16 @@ __device__ __forceinline__ void pipeline_step(const S (&cin)[2 * K], S (&cout)[2
         }
     }
     // last step, second half: Yo aligned, Ye shifted, Xo, Xe
-    {
-        const bool v = yok(y1);
-        y_pair<C::PACKED>(P, Q, v ? p.t1 : 0.f, v ? p.s1 : 0.f);
-    }
+    if (!INTERIOR && K > 1 && j < 2 * K - 1) return;
+    YO(P, Q, y1, 2 * K - 1);
     O0 = cin[2 * K - 1];      // rows (y1-1, y1) = (yin-2K, yin-2K+1)
     O1 = P;
-    {
-        const bool v = yok(y1 - 1);
-        y_pair<C::PACKED>(O0, O1, v ? p.t1 : 0.f, v ? p.s1 : 0.f);
-    }
+    YE(O0, O1, y1 - 1, K);
     cout[2 * K - 1] = Q;
-    x_odd(O0, c.O);
-    x_odd(O1, c.O);
-    x_even(O0, c.E1);
-    x_even(O1, c.E1);
+    XO(O0, 2 * K - 1);
+    XO(O1, 2 * K - 1);
+    XE(O0, K);
+    XE(O1, K);
 }
 
 // A warp's two slot rings: barriers, buffers, and the ring positions and
@@ -841,6 +1122,7 @@ struct WarpRings {
     uint64_t *bar_s, *bar_p, *bar_b;
     unsigned char *ring_s, *ring_p, *ring_b;
     float4 *sums, *gst;   // MODE 5: running sums, staged G rows (this lane's)
+    unsigned char *edge;  // SC: the warp's EdgeTab
     int pos_s, pos_p;
     uint32_t par_s, par_p;
     // b ring: b copies are numbered across the warp's segments; copy L sits
@@ -849,10 +1131,10 @@ struct WarpRings {
     int cnt_b;
 };
 
-template <int K, int PP = 2, bool BRING = false, int SP = 2, int M = 0>
+template <int K, int MODE, bool SC>
 __device__ __forceinline__ WarpRings carve_rings(unsigned char *smem_raw, int warp, int lane)
 {
-    using C = Cfg<K, PP, BRING, SP, M>;
+    using C = CfgM<K, MODE, SC>;
     constexpr int NSS = C::NSS, NSP = C::NSP, NBAR = C::NBAR;
     WarpRings r;
     // barriers first, then 1 KiB-aligned slots (state ring, phase ring, b ring)
@@ -867,6 +1149,7 @@ __device__ __forceinline__ WarpRings carve_rings(unsigned char *smem_raw, int wa
     r.ring_b = r.ring_p + NSP * C::PSLOT;
     r.sums = reinterpret_cast<float4 *>(r.ring_b + C::NSB * SLOT_BYTES) + lane;
     r.gst = reinterpret_cast<float4 *>(r.ring_b + C::NSB * SLOT_BYTES + C::SUMS_BYTES) + lane;
+    r.edge = r.ring_b + C::NSB * SLOT_BYTES + C::SUMS_BYTES + C::GST_BYTES;
     r.pos_s = r.pos_p = 0;
     r.par_s = r.par_p = 0;
     r.cnt_b = 0;
@@ -963,9 +1246,17 @@ __device__ __forceinline__ void issue_phase(WarpRings &r, const Seg &s, int pos,
 // segment).  So no warp overwrites rows another warp still reads.
 __device__ __forceinline__ bool on_grid(int z, const KParams &p) { return z >= 0 && z < p.nz; }
 
-template <bool PACKED>
-__device__ __forceinline__ void z_even(Frag2 &r0, Frag2 &r1, const Seg &s, const KParams &p)
+template <bool PACKED, bool SC>
+__device__ __forceinline__ void z_even(Frag2 &r0, Frag2 &r1, const Seg &s, const KParams &p, int k)
 {
+    if constexpr (SC) {
+        float ta, tb;
+        const float2 lh = reinterpret_cast<const EdgeTab<1, false> *>(s.own.edge)->lohi[k];
+        pair_coef(pair_kind(s.z, p.nz), p.te_end, lh.x, lh.y, ta, tb);
+        y_pair_s<PACKED>(r0.a, r0.b, ta, tb);
+        y_pair_s<PACKED>(r1.a, r1.b, ta, tb);
+        return;
+    }
     const bool v = on_grid(s.z, p) && on_grid(s.z + 1, p);
     y_pair<PACKED>(r0.a, r0.b, v ? p.t1 : 0.f, v ? p.s1 : 0.f);
     y_pair<PACKED>(r1.a, r1.b, v ? p.t1 : 0.f, v ? p.s1 : 0.f);
@@ -978,8 +1269,8 @@ __device__ __forceinline__ void z_even(Frag2 &r0, Frag2 &r1, const Seg &s, const
 // lane fences its generic writes before the barrier.  `after` runs right
 // after the barrier unless a warp failed: the slots that the barrier frees
 // are refilled there, before this exchange's reads and updates.
-template <int NW, int WSTRIDE, typename F>
-__device__ __forceinline__ bool z_odd(Frag2 &r0, Frag2 &r1, const Seg &s, const KParams &p,
+template <int NW, int WSTRIDE, bool SC, typename F>
+__device__ __forceinline__ bool z_odd(Frag2 &r0, Frag2 &r1, const Seg &s, const KParams &p, int m,
                                       float4 *mine, bool fail, F &&after)
 {
     const int lane = s.lane;
@@ -995,6 +1286,28 @@ __device__ __forceinline__ bool z_odd(Frag2 &r0, Frag2 &r1, const Seg &s, const 
     const bool any_fail = __syncthreads_or(fail);
     if (any_fail) return true;
     after();
+    if constexpr (SC) {
+        auto take = [&](Frag &f, const float4 *q, int row, float t) {   // f <- f + i t q
+            const float4 qr = q[64 * row + lane], qi = q[64 * row + 32 + lane];
+            const float2 n = make_float2(-t, -t), u = make_float2(t, t);
+            f.re = join2(__ffma2_rn(n, lo2(qi), lo2(f.re)), __ffma2_rn(n, hi2(qi), hi2(f.re)));
+            f.im = join2(__ffma2_rn(u, lo2(qr), lo2(f.im)), __ffma2_rn(u, hi2(qr), hi2(f.im)));
+        };
+        const float t = m == 0 ? p.to_a : p.to_b;
+        const float2 lh = reinterpret_cast<const EdgeTab<1, false> *>(s.own.edge)->lohi[2 + m];
+        float mine_t, other;
+        if (s.w + 1 < NW && on_grid(s.z + 1, p) && on_grid(s.z + 2, p)) {
+            pair_coef(pair_kind(s.z + 1, p.nz), t, lh.x, lh.y, mine_t, other);
+            take(r0.b, mine + WSTRIDE, 0, mine_t);
+            take(r1.b, mine + WSTRIDE, 1, mine_t);
+        }
+        if (s.w > 0 && on_grid(s.z - 1, p) && on_grid(s.z, p)) {
+            pair_coef(pair_kind(s.z - 1, p.nz), t, lh.x, lh.y, other, mine_t);
+            take(r0.a, mine - WSTRIDE + 128, 0, mine_t);
+            take(r1.a, mine - WSTRIDE + 128, 1, mine_t);
+        }
+        return false;
+    }
     const float g = p.g1, sn = p.s1;
     const float2 ng = make_float2(-g, -g), ns = make_float2(-sn, -sn), ps = make_float2(sn, sn);
     auto one = [&](Frag &f, const float4 *q, int row) {   // f <- f - g f + i s q, four columns
@@ -1029,12 +1342,12 @@ struct Issued {
     int s, p, b;
 };
 
-template <int K, int MODE, bool INTERIOR, typename S = StateT<MODE>>
+template <int K, int MODE, bool INTERIOR, bool SC, typename S = StateT<MODE>>
 __device__ __forceinline__ bool row_pair(WarpRings &r, const Seg &s, const KParams &p, int j,
                                          const S (&cin)[2 * K], S (&cout)[2 * K],
                                          Issued &iss)
 {
-    using C = CfgM<K, MODE>;
+    using C = CfgM<K, MODE, SC>;
     constexpr int NSS = C::NSS, NSP = C::NSP, NSB = C::NSB;
     const int lane = s.lane;
     // MODE 6 waits for its phase slot just before the phase point: the slot
@@ -1105,14 +1418,14 @@ __device__ __forceinline__ bool row_pair(WarpRings &r, const Seg &s, const KPara
     // state slot and then its phase slot (see z_odd).
     constexpr int WSTRIDE = C::WARP_SMEM / 16;
     if constexpr (MODE == 6) {
-        z_even<C::PACKED>(a, b, s, p);
+        z_even<C::PACKED, SC>(a, b, s, p, 0);
         float4 *xs = reinterpret_cast<float4 *>(r.ring_s + r.pos_s * C::SSLOT);
         // past this barrier every warp has read the previous row pair's
         // second exchange, in its phase slot: refill that slot with row pair
         // j - 1 + NSP.  (Both 3-D refills are issued right after the barrier
         // that frees their slot; issued after the exchange's updates and at
         // the end of the row pair, they measured 5 % slower.)
-        if (z_odd<C::WPC, WSTRIDE>(a, b, s, p, xs, !ok, [&]() {
+        if (z_odd<C::WPC, WSTRIDE, SC>(a, b, s, p, 0, xs, !ok, [&]() {
                 const int jq = j - 1 + NSP;
                 if (j >= 1 && jq < s.n_iter) {
                     if (lane == 0) {
@@ -1129,14 +1442,14 @@ __device__ __forceinline__ bool row_pair(WarpRings &r, const Seg &s, const KPara
     bool okp = true;
     if constexpr (LATE_P)
         okp = __all_sync(FULL, mbar_wait(&r.bar_p[r.pos_p], r.par_p, WAIT_LIMIT_NS));
-    S O0, O1;
-    pipeline_step<K, INTERIOR, MODE>(cin, cout, a, b, yin, j, r.ring_p, r.pos_p, r.ring_b,
+    S O0 = zero_state<S>(), O1 = zero_state<S>();
+    pipeline_step<K, INTERIOR, MODE, SC>(cin, cout, a, b, yin, j, r.ring_p, r.pos_p, r.ring_b,
                                      r.cnt_b, s.c, p, lane, s.own, O0, O1);
     if constexpr (MODE == 6) {
         float4 *xp = reinterpret_cast<float4 *>(r.ring_p + r.pos_p * C::PSLOT);
         // past this barrier every warp has read this row pair's first
         // exchange, in its state slot: refill that slot with row pair j + NSS
-        if (z_odd<C::WPC, WSTRIDE>(O0, O1, s, p, xp, !okp, [&]() {
+        if (z_odd<C::WPC, WSTRIDE, SC>(O0, O1, s, p, 1, xp, !okp, [&]() {
                 const int js = j + NSS;
                 if (js < s.n_iter) {
                     if (lane == 0) {
@@ -1147,9 +1460,46 @@ __device__ __forceinline__ bool row_pair(WarpRings &r, const Seg &s, const KPara
                 }
             }))
             return give_up();
-        z_even<C::PACKED>(O0, O1, s, p);
+        z_even<C::PACKED, SC>(O0, O1, s, p, 1);
     }
     const int yo = yin - 2 * K;
+    if constexpr (SC) {   // take the launch's scale out
+        const EdgeTab<K, MODE == 5> *et = reinterpret_cast<const EdgeTab<K, MODE == 5> *>(s.own.edge);
+        auto edge = [&](int slab, int row) {
+            return edge4(et->h + 9 * slab, row, p.ny, s.own.cols);
+        };
+        if constexpr (MODE == 6) {
+            if constexpr (INTERIOR) {
+                const float4 ha = et->hrow[0][s.own.lane_class], hb = et->hrow[1][s.own.lane_class];
+                unscale(O0.a, ha);
+                unscale(O1.a, ha);
+                unscale(O0.b, hb);
+                unscale(O1.b, hb);
+            } else {
+                unscale(O0.a, edge(0, yo));
+                unscale(O1.a, edge(0, yo + 1));
+                unscale(O0.b, edge(1, yo));
+                unscale(O1.b, edge(1, yo + 1));
+            }
+        } else {
+            float4 h0, h1;
+            if constexpr (INTERIOR) {
+                h0 = h1 = et->hrow[0][s.own.lane_class];
+            } else {
+                h0 = edge(0, yo);
+                h1 = edge(0, yo + 1);
+            }
+            if constexpr (MODE == 5) {
+                unscale(O0.a, h0);
+                unscale(O1.a, h1);
+                unscale(O0.b, h0);
+                unscale(O1.b, h1);
+            } else {
+                unscale(O0, h0);
+                unscale(O1, h1);
+            }
+        }
+    }
     if (s.store_lane && yo >= s.Y0 && yo < s.Y1) {
         if constexpr (MODE == 6) {
             if (s.store_a) store_rows(O0.a, O1.a, p.out_re, p.out_im, yo);
@@ -1194,13 +1544,13 @@ __device__ __forceinline__ bool row_pair(WarpRings &r, const Seg &s, const KPara
 // Stream the row pairs [q0, q1) of strip sx of one grid through the K-step
 // pipeline: rows [2 q0, 2 q1) are written to (p.out_re, p.out_im).  Returns
 // false if a bounded wait gave up.
-template <int K, int MODE>
+template <int K, int MODE, bool SC>
 __device__ __forceinline__ bool run_segment(WarpRings &r, const CUtensorMap *tm_state,
                                             const CUtensorMap *tm_phase, const CUtensorMap *tm_b,
                                             const KParams &p, int sx,
                                             int q0, int q1, int lane, const Slab3 &sl = Slab3())
 {
-    using C = CfgM<K, MODE>;
+    using C = CfgM<K, MODE, SC>;
     using S = StateT<MODE>;
     constexpr int NSS = C::NSS, NSP = C::NSP, NSB = C::NSB, HALO = C::HALO, VALID = C::VALID;
     static_assert(NSB <= NSP, "the prologue issues the b ring inside the phase ring's loop");
@@ -1222,8 +1572,9 @@ __device__ __forceinline__ bool run_segment(WarpRings &r, const CUtensorMap *tm_
     s.Ys = s.Y0 - 2 * K;                 // first loaded row
     s.n_iter = (s.Y1 - s.Y0) / 2 + 2 * K;   // row pairs loaded
 
-    // pair (x, x+1) is rotated iff both sites are on the grid
     const int xg = s.xg;
+    if constexpr (!SC) {
+    // pair (x, x+1) is rotated iff both sites are on the grid
     auto xok = [&](int x) { return x >= 0 && x + 1 < p.nx; };
     const bool e0 = xok(xg), e1 = xok(xg + 2), o0 = xok(xg + 1), oR = xok(xg + 3),
                oL = xok(xg - 1);
@@ -1236,8 +1587,10 @@ __device__ __forceinline__ bool run_segment(WarpRings &r, const CUtensorMap *tm_
                   oR ? p.sb : 0.f, oL ? p.gb : 0.f, oL ? p.sb : 0.f};
         s.c.Eab = {e0 ? p.tab : 0.f, e0 ? p.sab : 0.f, e1 ? p.tab : 0.f, e1 ? p.sab : 0.f};
     }
+    }
     s.store_lane = lane >= HALO / 4 && lane < 32 - HALO / 4 && xg < p.nx;
-    s.own = {s.Y0, s.Y1, xg, s.store_lane, r.sums, r.gst};
+    s.own = {s.Y0, s.Y1, xg, s.store_lane, SC ? col_places(xg, p.nx) : 0u, r.edge,
+             SC ? lane_class(xg, p.nx) : 0, r.sums, r.gst};
 
     const int n_pro_s = s.n_iter < NSS ? s.n_iter : NSS;
     const int n_pro_p = s.n_iter < NSP ? s.n_iter : NSP;
@@ -1253,6 +1606,47 @@ __device__ __forceinline__ bool run_segment(WarpRings &r, const CUtensorMap *tm_
         }
     }
     Issued iss = {n_pro_s, n_pro_p, n_pro_b};
+    if constexpr (SC) {   // the edge values (while the first copies are under way)
+        EdgeTab<K, MODE == 5> *et = reinterpret_cast<EdgeTab<K, MODE == 5> *>(r.edge);
+        constexpr int NE = K + 1;
+        for (int i = lane; i < 3 * K + 1; i += 32)
+            et->lohi[i] = i < NE ? make_float2(p.ed->elo[i], p.ed->ehi[i])
+                                 : make_float2(p.ed->olo[i - NE], p.ed->ohi[i - NE]);
+        if (lane < 18) {
+            const int z = s.z + (lane >= 9);
+            et->h[lane] = p.ed->h[(MODE == 6 ? 9 * edge_kind(z, p.nz) : 0) + lane % 9];
+        }
+        if constexpr (MODE == 5) {
+            for (int i = lane; i < 9 * K; i += 32) et->f[i] = p.ed->f[i / 9][i % 9];
+        }
+        __syncwarp();
+        const int cls = s.own.lane_class;   // (all lanes of a class write the same values)
+        for (int i = 0; i < 2; ++i) et->hrow[i][cls] = edge4(et->h + 9 * i, -1, p.ny, s.own.cols);
+        if constexpr (MODE == 5) {
+            for (int i = 0; i < K; ++i) et->frow[i][cls] = edge4(et->f + 9 * i, -1, p.ny, s.own.cols);
+        }
+#pragma unroll 1
+        for (int i = 0; i < 3 * K + 1; ++i) {
+            const float2 lh = et->lohi[i];
+            float4 c;
+            float other;
+            if (i < NE) {
+                const float t = MODE == 4 && (i == 2 || i == 3) ? p.te_ab
+                                : i == 0 || i == K              ? p.te_end
+                                                                : p.te_mid;
+                pair_coef(pair_kind(xg, p.nx), t, lh.x, lh.y, c.x, c.y);
+                pair_coef(pair_kind(xg + 2, p.nx), t, lh.x, lh.y, c.z, c.w);
+            } else {
+                const int m = i - NE;
+                const float t = MODE == 4 && m / 2 == 2 ? p.to_sub : (m & 1) ? p.to_b : p.to_a;
+                pair_coef(pair_kind(xg + 1, p.nx), t, lh.x, lh.y, c.y, c.z);
+                pair_coef(pair_kind(xg + 3, p.nx), t, lh.x, lh.y, c.w, other);
+                pair_coef(pair_kind(xg - 1, p.nx), t, lh.x, lh.y, other, c.x);
+            }
+            et->recv[i][cls] = c;
+        }
+        __syncwarp();
+    }
 
     // Carried rows: interior row pairs go in twos; for deep pipelines the
     // first reads set A and writes set B and the second goes back into A, so
@@ -1274,13 +1668,13 @@ __device__ __forceinline__ bool run_segment(WarpRings &r, const CUtensorMap *tm_
     }
     auto interior = [&](int j) {
         const int yin = s.Ys + 2 * j;
-        return j >= K && yin - 2 * K >= 0 && yin + 1 < p.ny;
+        return j >= K && yin - 2 * K >= (SC ? 2 : 0) && yin + (SC ? 2 : 1) < p.ny;
     };
     for (int j = 0; j < s.n_iter;) {
         if (C::ONE_PAIR) {
             if (interior(j)) {
-                if (!row_pair<K, MODE, true>(r, s, p, j, cA, cA, iss)) return false;
-            } else if (!row_pair<K, MODE, false>(r, s, p, j, cA, cA, iss)) {
+                if (!row_pair<K, MODE, true, SC>(r, s, p, j, cA, cA, iss)) return false;
+            } else if (!row_pair<K, MODE, false, SC>(r, s, p, j, cA, cA, iss)) {
                 return false;
             }
             j += 1;
@@ -1288,17 +1682,17 @@ __device__ __forceinline__ bool run_segment(WarpRings &r, const CUtensorMap *tm_
         }
         if (j + 1 < s.n_iter && interior(j) && interior(j + 1)) {
             if (C::PINGPONG) {
-                if (!row_pair<K, MODE, true>(r, s, p, j, cA, cB, iss)) return false;
-                if (!row_pair<K, MODE, true>(r, s, p, j + 1, cB, cA, iss))
+                if (!row_pair<K, MODE, true, SC>(r, s, p, j, cA, cB, iss)) return false;
+                if (!row_pair<K, MODE, true, SC>(r, s, p, j + 1, cB, cA, iss))
                     return false;
             } else {
-                if (!row_pair<K, MODE, true>(r, s, p, j, cA, cA, iss)) return false;
-                if (!row_pair<K, MODE, true>(r, s, p, j + 1, cA, cA, iss))
+                if (!row_pair<K, MODE, true, SC>(r, s, p, j, cA, cA, iss)) return false;
+                if (!row_pair<K, MODE, true, SC>(r, s, p, j + 1, cA, cA, iss))
                     return false;
             }
             j += 2;
         } else {
-            if (!row_pair<K, MODE, false>(r, s, p, j, cA, cA, iss)) return false;
+            if (!row_pair<K, MODE, false, SC>(r, s, p, j, cA, cA, iss)) return false;
             j += 1;
         }
     }
@@ -1322,20 +1716,28 @@ __device__ __forceinline__ bool run_segment(WarpRings &r, const CUtensorMap *tm_
     return true;
 }
 
+// The edge values of a launch, a kernel parameter of the scaled form (the
+// lifting form has none).
+struct NoEdge {};
+template <bool SC>
+using EdgeArg = std::conditional_t<SC, ScaledEdge, NoEdge>;
+
 // One grid; the (strip, row-pair) units are split into equal contiguous
 // ranges, one per warp of a persistent launch.
-template <int K, int MODE>
-__global__ void __launch_bounds__(Cfg<K>::WPC * 32, min_blocks(K, MODE))
+template <int K, int MODE, bool SC>
+__global__ void __launch_bounds__(Cfg<K>::WPC * 32, min_blocks(K, MODE, SC))
 fused_kernel(const __grid_constant__ CUtensorMap tm_state,
              const __grid_constant__ CUtensorMap tm_phase,
              const __grid_constant__ CUtensorMap tm_b,
-             const KParams p)
+             const KParams pk, const __grid_constant__ EdgeArg<SC> ed)
 {
+    KParams p = pk;
+    if constexpr (SC) p.ed = &ed;
     extern __shared__ unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int gw = blockIdx.x * Cfg<K>::WPC + warp;
     if (gw >= p.total_warps) return;
-    WarpRings r = carve_rings<K, phase_planes(MODE), MODE == 4, state_planes(MODE), MODE>(smem_raw, warp, lane);
+    WarpRings r = carve_rings<K, MODE, SC>(smem_raw, warp, lane);
     grid_dep_sync();
     if (p.strip_warps > 0) {
         // strip-aligned split: warp (sx, i) takes row range i of strip sx, so
@@ -1344,7 +1746,7 @@ fused_kernel(const __grid_constant__ CUtensorMap tm_state,
         const int sx = gw / p.strip_warps, i = gw - sx * p.strip_warps;
         const int q0 = (int)((int64_t)i * p.n_pairs / p.strip_warps);
         const int q1 = (int)((int64_t)(i + 1) * p.n_pairs / p.strip_warps);
-        if (q1 > q0) run_segment<K, MODE>(r, &tm_state, &tm_phase, &tm_b, p, sx, q0, q1, lane);
+        if (q1 > q0) run_segment<K, MODE, SC>(r, &tm_state, &tm_phase, &tm_b, p, sx, q0, q1, lane);
         return;
     }
     const int64_t u_begin = (int64_t)gw * p.units / p.total_warps;
@@ -1355,7 +1757,7 @@ fused_kernel(const __grid_constant__ CUtensorMap tm_state,
         const int64_t q1_want = (int64_t)q0 + (u_end - u);
         const int q1 = (int)(q1_want < p.n_pairs ? q1_want : (int64_t)p.n_pairs);
         u += q1 - q0;
-        if (!run_segment<K, MODE>(r, &tm_state, &tm_phase, &tm_b, p, sx, q0, q1, lane)) return;
+        if (!run_segment<K, MODE, SC>(r, &tm_state, &tm_phase, &tm_b, p, sx, q0, q1, lane)) return;
     }
 }
 
@@ -1372,19 +1774,20 @@ fused_kernel(const __grid_constant__ CUtensorMap tm_state,
 // pair with nothing.  Units (z-block fastest, then strip, then row range) go
 // round robin over the resident CTAs, so the CTAs of neighbouring z-blocks
 // run together and read their shared halo slabs through L2.
-template <int K>
+template <int K, bool SC>
 __global__ void __launch_bounds__(TS_FUSED3D_WARPS * 32, 1)
 fused3d_kernel(const __grid_constant__ CUtensorMap tm_state,
-               const __grid_constant__ CUtensorMap tm_phase, const KParams p)
+               const __grid_constant__ CUtensorMap tm_phase, const KParams p,
+               const __grid_constant__ EdgeArg<SC> ed)
 {
     static_assert(K == 1, "3-D steps run one step per launch");
-    using C = CfgM<K, 6>;
+    using C = CfgM<K, 6, SC>;
     constexpr int NW = C::WPC, VZ = 2 * NW - 4;
     static_assert(VZ > 0 && VZ % 2 == 0, "the block's first slab must stay even");
     static_assert(NW <= 16, "the host's row-coordinate guard assumes at most 16 warps");
     extern __shared__ unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    WarpRings r = carve_rings<K, phase_planes(6), false, state_planes(6), 6>(smem_raw, warp, lane);
+    WarpRings r = carve_rings<K, 6, SC>(smem_raw, warp, lane);
     const int64_t slab = (int64_t)p.ny * p.pitch;
     grid_dep_sync();
     for (int64_t u = blockIdx.x; u < p.units; u += gridDim.x) {
@@ -1402,6 +1805,7 @@ fused3d_kernel(const __grid_constant__ CUtensorMap tm_state,
         sl.store_a = inner && sl.z >= 0 && sl.z < p.nz;
         sl.store_b = inner && sl.z + 1 >= 0 && sl.z + 1 < p.nz;
         KParams pw = p;
+        if constexpr (SC) pw.ed = &ed;
         if (sl.store_a) {
             pw.out_re = p.out_re + sl.z * slab;
             pw.out_im = p.out_im + sl.z * slab;
@@ -1410,7 +1814,7 @@ fused3d_kernel(const __grid_constant__ CUtensorMap tm_state,
             pw.out2_re = p.out_re + (sl.z + 1) * slab;
             pw.out2_im = p.out_im + (sl.z + 1) * slab;
         }
-        if (!run_segment<K, 6>(r, &tm_state, &tm_phase, nullptr, pw, sx, q0, q1, lane, sl))
+        if (!run_segment<K, 6, SC>(r, &tm_state, &tm_phase, nullptr, pw, sx, q0, q1, lane, sl))
             return;
     }
 }
@@ -1426,6 +1830,7 @@ fused3d_kernel(const __grid_constant__ CUtensorMap tm_state,
 //    warp -- balanced for any mix, but without that alignment.
 // A grid's tensor maps live in its descriptor in global memory, written once
 // when the grid was set up.
+template <int K, bool SC>
 __device__ __forceinline__ void multi_params(KParams &p, const GridDesc *d, int cur, int *err)
 {
     p.nx = d->nx;
@@ -1433,27 +1838,36 @@ __device__ __forceinline__ void multi_params(KParams &p, const GridDesc *d, int 
     p.pitch = d->pitch;
     p.out_re = d->re[cur ^ 1];
     p.out_im = d->im[cur ^ 1];
-    p.t1 = d->t1;
-    p.s1 = d->s1;
-    p.g1 = d->g1;
-    p.t2 = d->t2;
-    p.s2 = d->s2;
+    if constexpr (SC) {
+        const ScaledCoef &c = d->sc[K - 1];
+        p.te_end = c.te_end;
+        p.te_mid = c.te_mid;
+        p.to_a = c.to_a;
+        p.to_b = c.to_b;
+        p.ed = &c.edge;
+    } else {
+        p.t1 = d->t1;
+        p.s1 = d->s1;
+        p.g1 = d->g1;
+        p.t2 = d->t2;
+        p.s2 = d->s2;
+    }
     p.err = err;
     p.n_pairs = (p.ny + 1) / 2;
     p.strip_warps = 0;
 }
 
-template <int K>
+template <int K, bool SC>
 __global__ void __launch_bounds__(Cfg<K>::WPC * 32, multi_min_blocks(K))
 fused_multi_kernel(const EpochEntry *__restrict__ tab, int n_grids, int64_t total_units,
                    int total_warps, int aligned, int flip, int *err)
 {
-    using C = Cfg<K>;
+    using C = CfgM<K, 0, SC>;
     extern __shared__ unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int gw = blockIdx.x * C::WPC + warp;
     if (gw >= total_warps) return;
-    WarpRings r = carve_rings<K>(smem_raw, warp, lane);
+    WarpRings r = carve_rings<K, 0, SC>(smem_raw, warp, lane);
     grid_dep_sync();
     if (aligned) {
         // the grid of warp gw: the last entry whose first warp is <= gw
@@ -1474,13 +1888,13 @@ fused_multi_kernel(const EpochEntry *__restrict__ tab, int n_grids, int64_t tota
         }
         __syncwarp();
         KParams p;
-        multi_params(p, d, cur, err);
+        multi_params<K, SC>(p, d, cur, err);
         const int w = e.strip_warps, l = gw - (int)e.begin;
         const int sx = l / w, i = l - sx * w;
         const int q0 = (int)((int64_t)i * p.n_pairs / w);
         const int q1 = (int)((int64_t)(i + 1) * p.n_pairs / w);
         if (q1 > q0)
-            run_segment<K, 0>(r, &d->tm_state[cur], &d->tm_phase, nullptr, p, sx, q0, q1, lane);
+            run_segment<K, 0, SC>(r, &d->tm_state[cur], &d->tm_phase, nullptr, p, sx, q0, q1, lane);
         return;
     }
     const int64_t u_begin = (int64_t)gw * total_units / total_warps;
@@ -1500,7 +1914,7 @@ fused_multi_kernel(const EpochEntry *__restrict__ tab, int n_grids, int64_t tota
             fenced = gi;
         }
         KParams p;
-        multi_params(p, d, cur, err);
+        multi_params<K, SC>(p, d, cur, err);
         const int64_t local = u - e.begin;
         const int64_t g_units = (gi + 1 < n_grids ? tab[gi + 1].begin : total_units) - e.begin;
         const int sx = (int)(local / p.n_pairs);
@@ -1510,17 +1924,9 @@ fused_multi_kernel(const EpochEntry *__restrict__ tab, int n_grids, int64_t tota
         if (q1_want > q0 + left_in_grid) q1_want = q0 + left_in_grid;
         const int q1 = (int)(q1_want < p.n_pairs ? q1_want : (int64_t)p.n_pairs);
         u += q1 - q0;
-        if (!run_segment<K, 0>(r, &d->tm_state[cur], &d->tm_phase, nullptr, p, sx, q0, q1, lane)) return;
+        if (!run_segment<K, 0, SC>(r, &d->tm_state[cur], &d->tm_phase, nullptr, p, sx, q0, q1, lane)) return;
     }
 }
-
-// Resident blocks per SM and SM count of a kernel at its dynamic shared
-// memory size, set up once per kernel (the first caller's function-local
-// static initialisation, which C++ runs exactly once even when threads race).
-struct Occupancy {
-    cudaError_t err;
-    int blocks_per_sm, num_sms;
-};
 
 // Fewest row pairs a warp takes.  Each warp runs a chain of dependent
 // iterations, and each of its segments first fills a pipeline of 2K row
@@ -1535,15 +1941,52 @@ inline int64_t min_pairs_per_warp(int64_t units, int num_sms)
     return std::min<int64_t>(TS_FUSED_MAX_MIN_PAIRS, std::max<int64_t>(TS_FUSED_MIN_PAIRS, by_work));
 }
 
+#if TS_FUSED_PART != 0
+
 template <typename F>
-Occupancy occupancy_of(F kernel, int threads, int smem);
+Occupancy occupancy_of(F kernel, int threads, int smem)
+{
+    Occupancy o = {cudaSuccess, 0, 0};
+    o.err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (o.err != cudaSuccess) return o;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&o.num_sms, cudaDevAttrMultiProcessorCount, dev);
+    o.err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o.blocks_per_sm, kernel, threads, smem);
+    if (o.err == cudaSuccess && o.blocks_per_sm < 1) o.err = cudaErrorInvalidConfiguration;
+    return o;
+}
+
+// The kernel parameters of a launch's scaled rotations.
+void set_scaled(KParams &p, const ScaledCoef &c)
+{
+    p.te_end = c.te_end;
+    p.te_mid = c.te_mid;
+    p.to_a = c.to_a;
+    p.to_b = c.to_b;
+    p.te_ab = c.te_ab;
+    p.to_sub = c.to_sub;
+    p.ed = nullptr;   // the kernel points it at its own copy
+}
+
+template <bool SC>
+EdgeArg<SC> edge_arg(const FusedLaunch &a)
+{
+    if constexpr (SC)
+        return a.sc->edge;
+    else
+        return NoEdge{};
+}
+
+}  // namespace
 
 // One 3-D step over an nx x ny x nz FP32 grid (a.ny = ny rows per slab).
+template <bool SC>
 cudaError_t launch3_k(const FusedLaunch &a, int nz, cudaStream_t st)
 {
-    using C = CfgM<1, 6>;
+    using C = CfgM<1, 6, SC>;
     constexpr int NW = C::WPC, VZ = 2 * NW - 4;
-    static const Occupancy occ = occupancy_of(fused3d_kernel<1>, NW * 32, C::SMEM);
+    static const Occupancy occ = occupancy_of(fused3d_kernel<1, SC>, NW * 32, C::SMEM);
     if (occ.err != cudaSuccess) return occ.err;
     KParams p = {};
     p.out_re = a.out_re;
@@ -1582,31 +2025,19 @@ cudaError_t launch3_k(const FusedLaunch &a, int nz, cudaStream_t st)
     p.t2 = a.t2;
     p.s2 = a.s2;
     p.err = a.err;
+    if constexpr (SC) set_scaled(p, *a.sc);
     const int grid = (int)std::min<int64_t>(p.units, ctas);
-    launch_pdl(fused3d_kernel<1>, grid, NW * 32, C::SMEM, st, *a.tm_state, *a.tm_phase, p);
+    launch_pdl(fused3d_kernel<1, SC>, grid, NW * 32, C::SMEM, st, *a.tm_state, *a.tm_phase, p,
+               edge_arg<SC>(a));
     count_launches(1);
     return cudaGetLastError();
 }
 
-template <typename F>
-Occupancy occupancy_of(F kernel, int threads, int smem)
-{
-    Occupancy o = {cudaSuccess, 0, 0};
-    o.err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (o.err != cudaSuccess) return o;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&o.num_sms, cudaDevAttrMultiProcessorCount, dev);
-    o.err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o.blocks_per_sm, kernel, threads, smem);
-    if (o.err == cudaSuccess && o.blocks_per_sm < 1) o.err = cudaErrorInvalidConfiguration;
-    return o;
-}
-
-template <int K, int MODE>
+template <int K, int MODE, bool SC>
 cudaError_t launch_k(const FusedLaunch &a, cudaStream_t st)
 {
-    using C = CfgM<K, MODE>;
-    static const Occupancy occ = occupancy_of(fused_kernel<K, MODE>, C::WPC * 32, C::SMEM);
+    using C = CfgM<K, MODE, SC>;
+    static const Occupancy occ = occupancy_of(fused_kernel<K, MODE, SC>, C::WPC * 32, C::SMEM);
     if (occ.err != cudaSuccess) return occ.err;
     const int blocks_per_sm = occ.blocks_per_sm, num_sms = occ.num_sms;
     KParams p;
@@ -1650,115 +2081,202 @@ cudaError_t launch_k(const FusedLaunch &a, cudaStream_t st)
     p.gb = a.gb;
     p.tab = a.tab;
     p.sab = a.sab;
+    if constexpr (SC) set_scaled(p, *a.sc);
     const int blocks = (p.total_warps + C::WPC - 1) / C::WPC;
-    launch_pdl(fused_kernel<K, MODE>, blocks, C::WPC * 32, C::SMEM, st, *a.tm_state, *a.tm_phase, a.tm_b ? *a.tm_b : *a.tm_phase, p);
+    launch_pdl(fused_kernel<K, MODE, SC>, blocks, C::WPC * 32, C::SMEM, st, *a.tm_state,
+               *a.tm_phase, a.tm_b ? *a.tm_b : *a.tm_phase, p, edge_arg<SC>(a));
     count_launches(1);
     return cudaGetLastError();
 }
+
+template <int K, bool SC>
+const Occupancy &multi_occupancy()
+{
+    using C = CfgM<K, 0, SC>;
+    static const Occupancy occ = occupancy_of(fused_multi_kernel<K, SC>, C::WPC * 32, C::SMEM);
+    return occ;
+}
+
+template <int K, bool SC>
+cudaError_t launch_multi_k(const EpochEntry *tab, int n_grids, const MultiPlan &plan, int flip,
+                           int *err, cudaStream_t st)
+{
+    using C = CfgM<K, 0, SC>;
+    const Occupancy &occ = multi_occupancy<K, SC>();
+    if (occ.err != cudaSuccess) return occ.err;
+    const int blocks = (plan.warps + C::WPC - 1) / C::WPC;
+    launch_pdl(fused_multi_kernel<K, SC>, blocks, C::WPC * 32, C::SMEM, st, tab, n_grids,
+               plan.units, plan.warps, plan.aligned ? 1 : 0, flip, err);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
+#define TS_KERNEL(K, MODE, SC) \
+    template cudaError_t launch_k<K, MODE, SC>(const FusedLaunch &, cudaStream_t);
+#define TS_MULTI(K, SC)                                                                     \
+    template const Occupancy &multi_occupancy<K, SC>();                                     \
+    template cudaError_t launch_multi_k<K, SC>(const EpochEntry *, int, const MultiPlan &, \
+                                               int, int *, cudaStream_t);
+#define TS_KERNEL_3D(SC) \
+    template cudaError_t launch3_k<SC>(const FusedLaunch &, int, cudaStream_t);
+#if TS_FUSED_PART == 1
+TS_KERNEL(1, 0, true)
+TS_KERNEL(2, 0, true)
+TS_KERNEL(3, 0, true)
+#elif TS_FUSED_PART == 2
+TS_KERNEL(4, 0, true)
+TS_KERNEL(5, 0, true)
+#elif TS_FUSED_PART == 3
+TS_KERNEL(6, 0, true)
+TS_KERNEL(7, 0, true)
+#elif TS_FUSED_PART == 4
+TS_KERNEL(8, 0, true)
+TS_KERNEL(5, 4, true)
+#elif TS_FUSED_PART == 5
+TS_MULTI(1, true)
+TS_MULTI(2, true)
+TS_MULTI(3, true)
+#elif TS_FUSED_PART == 6
+TS_MULTI(4, true)
+TS_MULTI(5, true)
+#elif TS_FUSED_PART == 7
+TS_MULTI(6, true)
+TS_MULTI(7, true)
+#elif TS_FUSED_PART == 8
+TS_MULTI(8, true)
+TS_KERNEL_3D(true)
+#elif TS_FUSED_PART == 9
+TS_KERNEL(1, 3, true)
+TS_KERNEL(2, 3, true)
+TS_KERNEL(3, 3, true)
+#elif TS_FUSED_PART == 10
+TS_KERNEL(4, 3, true)
+TS_KERNEL(1, 5, true)
+TS_KERNEL(2, 5, true)
+#elif TS_FUSED_PART == 11
+TS_KERNEL(3, 5, true)
+TS_KERNEL(4, 5, true)
+#elif TS_FUSED_PART == 12   // the lifting form, to FUSED_LIFT_MAX_K
+TS_KERNEL(1, 0, false)
+TS_KERNEL(2, 0, false)
+TS_KERNEL(3, 0, false)
+TS_KERNEL(4, 0, false)
+#elif TS_FUSED_PART == 13
+TS_MULTI(1, false)
+TS_MULTI(2, false)
+TS_MULTI(3, false)
+TS_MULTI(4, false)
+#elif TS_FUSED_PART == 14
+TS_KERNEL(1, 3, false)
+TS_KERNEL(2, 3, false)
+TS_KERNEL(3, 3, false)
+TS_KERNEL(4, 3, false)
+#elif TS_FUSED_PART == 15
+TS_KERNEL(5, 4, false)
+TS_KERNEL_3D(false)
+TS_KERNEL(1, 5, false)
+TS_KERNEL(2, 5, false)
+TS_KERNEL(3, 5, false)
+TS_KERNEL(4, 5, false)
+#endif
+
+#else   // part 0
 
 }  // namespace
 
 cudaError_t launch_fused(int K, const FusedLaunch &a, cudaStream_t st)
 {
+    if (!a.sc) {
+        switch (K) {
+        case 1: return launch_k<1, 0, false>(a, st);
+        case 2: return launch_k<2, 0, false>(a, st);
+        case 3: return launch_k<3, 0, false>(a, st);
+        case 4: return launch_k<4, 0, false>(a, st);
+        default: return cudaErrorInvalidValue;
+        }
+    }
     switch (K) {
-    case 1: return launch_k<1, 0>(a, st);
-    case 2: return launch_k<2, 0>(a, st);
-    case 3: return launch_k<3, 0>(a, st);
-    case 4: return launch_k<4, 0>(a, st);
-    case 5: return launch_k<5, 0>(a, st);
-    case 6: return launch_k<6, 0>(a, st);
-    case 7: return launch_k<7, 0>(a, st);
-    case 8: return launch_k<8, 0>(a, st);
+    case 1: return launch_k<1, 0, true>(a, st);
+    case 2: return launch_k<2, 0, true>(a, st);
+    case 3: return launch_k<3, 0, true>(a, st);
+    case 4: return launch_k<4, 0, true>(a, st);
+    case 5: return launch_k<5, 0, true>(a, st);
+    case 6: return launch_k<6, 0, true>(a, st);
+    case 7: return launch_k<7, 0, true>(a, st);
+    case 8: return launch_k<8, 0, true>(a, st);
     default: return cudaErrorInvalidValue;
     }
 }
 
-template <int K>
-const Occupancy &multi_occupancy()
+// The multi-grid kernel's occupancy at depth K (nullptr: no such kernel).
+static const Occupancy *multi_occ(int K, bool scaled)
 {
-    using C = Cfg<K>;
-    static const Occupancy occ = occupancy_of(fused_multi_kernel<K>, C::WPC * 32, C::SMEM);
-    return occ;
-}
-
-template <int K>
-cudaError_t prepare_multi_k()
-{
-    return multi_occupancy<K>().err;
-}
-
-template <int K>
-cudaError_t launch_multi_k(const EpochEntry *tab, int n_grids, const MultiPlan &plan, int flip,
-                           int *err, cudaStream_t st)
-{
-    using C = Cfg<K>;
-    const Occupancy &occ = multi_occupancy<K>();
-    if (occ.err != cudaSuccess) return occ.err;
-    const int blocks = (plan.warps + C::WPC - 1) / C::WPC;
-    launch_pdl(fused_multi_kernel<K>, blocks, C::WPC * 32, C::SMEM, st, tab, n_grids, plan.units, plan.warps, plan.aligned ? 1 : 0, flip, err);
-    count_launches(1);
-    return cudaGetLastError();
-}
-
-// Resident warps of the multi-grid kernel at depth K (-1 on an error) and the SM count.
-template <int K>
-int64_t multi_capacity(int &num_sms)
-{
-    const Occupancy &occ = multi_occupancy<K>();
-    if (occ.err != cudaSuccess) return -1;
-    num_sms = occ.num_sms;
-    return (int64_t)occ.num_sms * occ.blocks_per_sm * Cfg<K>::WPC;
+    if (!scaled) {
+        switch (K) {
+        case 1: return &multi_occupancy<1, false>();
+        case 2: return &multi_occupancy<2, false>();
+        case 3: return &multi_occupancy<3, false>();
+        case 4: return &multi_occupancy<4, false>();
+        default: return nullptr;
+        }
+    }
+    switch (K) {
+    case 1: return &multi_occupancy<1, true>();
+    case 2: return &multi_occupancy<2, true>();
+    case 3: return &multi_occupancy<3, true>();
+    case 4: return &multi_occupancy<4, true>();
+    case 5: return &multi_occupancy<5, true>();
+    case 6: return &multi_occupancy<6, true>();
+    case 7: return &multi_occupancy<7, true>();
+    case 8: return &multi_occupancy<8, true>();
+    default: return nullptr;
+    }
 }
 
 cudaError_t fused_multi_prepare(int K)
 {
-    switch (K) {
-    case 1: return prepare_multi_k<1>();
-    case 2: return prepare_multi_k<2>();
-    case 3: return prepare_multi_k<3>();
-    case 4: return prepare_multi_k<4>();
-    case 5: return prepare_multi_k<5>();
-    case 6: return prepare_multi_k<6>();
-    case 7: return prepare_multi_k<7>();
-    case 8: return prepare_multi_k<8>();
-    default: return cudaErrorInvalidValue;
-    }
+    const Occupancy *o = multi_occ(K, true);
+    cudaError_t e = o ? o->err : cudaErrorInvalidValue;
+    if (e == cudaSuccess && K <= FUSED_LIFT_MAX_K) e = multi_occ(K, false)->err;
+    return e;
 }
 
-cudaError_t launch_fused_multi(int K, const EpochEntry *tab, int n_grids, const MultiPlan &plan,
-                               int flip, int *err, cudaStream_t st)
+cudaError_t launch_fused_multi(int K, bool scaled, const EpochEntry *tab, int n_grids,
+                               const MultiPlan &plan, int flip, int *err, cudaStream_t st)
 {
     if (n_grids < 1 || plan.warps < 1 || plan.units < 1) return cudaSuccess;
+    if (!scaled) {
+        switch (K) {
+        case 1: return launch_multi_k<1, false>(tab, n_grids, plan, flip, err, st);
+        case 2: return launch_multi_k<2, false>(tab, n_grids, plan, flip, err, st);
+        case 3: return launch_multi_k<3, false>(tab, n_grids, plan, flip, err, st);
+        case 4: return launch_multi_k<4, false>(tab, n_grids, plan, flip, err, st);
+        default: return cudaErrorInvalidValue;
+        }
+    }
     switch (K) {
-    case 1: return launch_multi_k<1>(tab, n_grids, plan, flip, err, st);
-    case 2: return launch_multi_k<2>(tab, n_grids, plan, flip, err, st);
-    case 3: return launch_multi_k<3>(tab, n_grids, plan, flip, err, st);
-    case 4: return launch_multi_k<4>(tab, n_grids, plan, flip, err, st);
-    case 5: return launch_multi_k<5>(tab, n_grids, plan, flip, err, st);
-    case 6: return launch_multi_k<6>(tab, n_grids, plan, flip, err, st);
-    case 7: return launch_multi_k<7>(tab, n_grids, plan, flip, err, st);
-    case 8: return launch_multi_k<8>(tab, n_grids, plan, flip, err, st);
+    case 1: return launch_multi_k<1, true>(tab, n_grids, plan, flip, err, st);
+    case 2: return launch_multi_k<2, true>(tab, n_grids, plan, flip, err, st);
+    case 3: return launch_multi_k<3, true>(tab, n_grids, plan, flip, err, st);
+    case 4: return launch_multi_k<4, true>(tab, n_grids, plan, flip, err, st);
+    case 5: return launch_multi_k<5, true>(tab, n_grids, plan, flip, err, st);
+    case 6: return launch_multi_k<6, true>(tab, n_grids, plan, flip, err, st);
+    case 7: return launch_multi_k<7, true>(tab, n_grids, plan, flip, err, st);
+    case 8: return launch_multi_k<8, true>(tab, n_grids, plan, flip, err, st);
     default: return cudaErrorInvalidValue;
     }
 }
 
-MultiPlan fused_multi_plan(int K, int n, const int *nx, const int *ny, EpochEntry *tab)
+MultiPlan fused_multi_plan(int K, bool scaled, int n, const int *nx, const int *ny,
+                           EpochEntry *tab)
 {
     MultiPlan plan = {0, 0, false};
-    int64_t cap;
-    int num_sms = 1;
-    switch (K) {
-    case 1: cap = multi_capacity<1>(num_sms); break;
-    case 2: cap = multi_capacity<2>(num_sms); break;
-    case 3: cap = multi_capacity<3>(num_sms); break;
-    case 4: cap = multi_capacity<4>(num_sms); break;
-    case 5: cap = multi_capacity<5>(num_sms); break;
-    case 6: cap = multi_capacity<6>(num_sms); break;
-    case 7: cap = multi_capacity<7>(num_sms); break;
-    case 8: cap = multi_capacity<8>(num_sms); break;
-    default: return plan;
-    }
-    if (cap < 1 || n < 1) return plan;
+    const Occupancy *occ = multi_occ(K, scaled);
+    if (!occ || occ->err != cudaSuccess || n < 1) return plan;
+    const int num_sms = occ->num_sms;
+    // resident warps
+    const int64_t cap = (int64_t)num_sms * occ->blocks_per_sm *
+                        (K <= 2 ? TS_FUSED_WPC_SHALLOW : TS_FUSED_WPC_DEEP);
     const int halo = ((2 * K + 3) / 4) * 4, valid = FUSED_BOX_COLS - 2 * halo;
     std::vector<int64_t> strips((size_t)n), pairs((size_t)n), w((size_t)n, 1);
     int64_t units = 0, all_strips = 0;
@@ -1808,28 +2326,31 @@ MultiPlan fused_multi_plan(int K, int n, const int *nx, const int *ny, EpochEntr
 cudaError_t launch_fused_drive(int K, const FusedLaunch &a, cudaStream_t st)
 {
     switch (K) {
-    case 1: return launch_k<1, 3>(a, st);
-    case 2: return launch_k<2, 3>(a, st);
-    case 3: return launch_k<3, 3>(a, st);
-    case 4: return launch_k<4, 3>(a, st);
+    case 1: return a.sc ? launch_k<1, 3, true>(a, st) : launch_k<1, 3, false>(a, st);
+    case 2: return a.sc ? launch_k<2, 3, true>(a, st) : launch_k<2, 3, false>(a, st);
+    case 3: return a.sc ? launch_k<3, 3, true>(a, st) : launch_k<3, 3, false>(a, st);
+    case 4: return a.sc ? launch_k<4, 3, true>(a, st) : launch_k<4, 3, false>(a, st);
     default: return cudaErrorInvalidValue;
     }
 }
 
-cudaError_t launch_fused_u4(const FusedLaunch &a, cudaStream_t st) { return launch_k<5, 4>(a, st); }
+cudaError_t launch_fused_u4(const FusedLaunch &a, cudaStream_t st)
+{
+    return a.sc ? launch_k<5, 4, true>(a, st) : launch_k<5, 4, false>(a, st);
+}
 
 cudaError_t launch_fused3d(const FusedLaunch &a, int nz, cudaStream_t st)
 {
-    return launch3_k(a, nz, st);
+    return a.sc ? launch3_k<true>(a, nz, st) : launch3_k<false>(a, nz, st);
 }
 
 cudaError_t launch_fused_adjoint(int K, const FusedLaunch &a, cudaStream_t st)
 {
     switch (K) {
-    case 1: return launch_k<1, 5>(a, st);
-    case 2: return launch_k<2, 5>(a, st);
-    case 3: return launch_k<3, 5>(a, st);
-    case 4: return launch_k<4, 5>(a, st);
+    case 1: return a.sc ? launch_k<1, 5, true>(a, st) : launch_k<1, 5, false>(a, st);
+    case 2: return a.sc ? launch_k<2, 5, true>(a, st) : launch_k<2, 5, false>(a, st);
+    case 3: return a.sc ? launch_k<3, 5, true>(a, st) : launch_k<3, 5, false>(a, st);
+    case 4: return a.sc ? launch_k<4, 5, true>(a, st) : launch_k<4, 5, false>(a, st);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -1874,5 +2395,7 @@ bool make_pair_tensor_map(CUtensorMap *tm, const void *base, int nx, int ny, int
     }
     return true;
 }
+
+#endif  // part 0
 
 }  // namespace ts

@@ -18,6 +18,15 @@ struct RotCoef {
     double g1, s1, t1, s2, t2;
 };
 RotCoef rot_coef(double theta);
+
+// Scaled rotations (fused.cu) serve |theta| <= this, per substep.  A launch
+// takes its scale out by a -= h a, and the rounding of h (ulp(h) / 2, the same
+// at every site) is what they add to the norm: under 1e-9 per step here, where
+// h < 1/8 at depth 4.  The tangents and the edge ratios stay far from their
+// poles.  Larger angles take the lifting form.
+constexpr double SCALED_MAX_THETA = 0.075;
+// Coefficients of a launch of K substeps with kinetic half angles sub[i].
+void scaled_coef(const double *sub, int K, int64_t nx, int64_t ny, int64_t nz, ScaledCoef &c);
 }  // namespace ts
 
 // One grid: a slab of seven planes (re, im of ping-pong pairs 0 and 1,
@@ -80,7 +89,8 @@ void grid_set_coefficients(ts_grid *g, double dt, double theta, cudaStream_t st)
 // Write the grid's multi-grid descriptor (tensor maps, planes, coefficients)
 // into its slab on stream st (api.cu).
 void grid_write_desc(ts_grid *g, cudaStream_t st);
-// Evolve n FP32 grids (|theta| <= pi/4) together with the multi-grid kernel
-// at depth K (api.cu).
-cudaError_t evolve_multi(ts_grid *const *gs, const int64_t *steps, int n, int K, cudaStream_t st);
+// Evolve n FP32 grids (|theta| <= pi/4, with `scaled` <= SCALED_MAX_THETA)
+// together with the multi-grid kernel at depth K (api.cu).
+cudaError_t evolve_multi(ts_grid *const *gs, const int64_t *steps, int n, int K, bool scaled,
+                         cudaStream_t st);
 }  // namespace ts

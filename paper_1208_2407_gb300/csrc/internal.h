@@ -83,6 +83,28 @@ cudaError_t launch_inner(const float *phi_re, const float *phi_im, const float *
                          double *result, cudaStream_t st);
 
 // --- fused temporally blocked path (fused.cu) -----------------------------
+constexpr int FUSED_MAX_K = 8;
+constexpr int FUSED_LIFT_MAX_K = 4;   // ... of the lifting form (deeper ones run slower)
+constexpr int FUSED_ADJ_MAX_K = 4;
+// Scaled rotations (see pair_s in fused.cu): what the pairs with a member on
+// an edge of the grid receive in even sweep k and odd sweep m (the edge member
+// lo, its partner hi), h = 1 - scale of a launch for a site at place (z, y, x),
+// entry 9 z + 3 y + x with 0 bulk, 1 the first site of the axis, 2 the last,
+// and (adjoint) the squared scale at phase k, entry 3 y + x.
+struct ScaledEdge {
+    float elo[FUSED_MAX_K + 1], ehi[FUSED_MAX_K + 1];
+    float olo[2 * FUSED_MAX_K], ohi[2 * FUSED_MAX_K];
+    float h[27];
+    float f[FUSED_ADJ_MAX_K][9];
+};
+// The bulk coefficients (tangents) of a launch: even sweeps 0 and K, the even
+// sweeps between, odd sweeps before and after a phase; fourth-order steps:
+// the even sweeps that join a and b substeps and the odd sweeps of b.
+struct ScaledCoef {
+    float te_end, te_mid, to_a, to_b, te_ab, to_sub;
+    ScaledEdge edge;
+};
+
 struct FusedLaunch {
     const CUtensorMap *tm_state;   // (re, im) planes of the input pair, 3-D map
     const CUtensorMap *tm_phase;   // (gamma_V, s_V) planes, 3-D map
@@ -104,8 +126,9 @@ struct FusedLaunch {
     // a substep's; the b substep's lifting (tb, sb) and versine (gb) forms,
     // and the merged angle a + b in lifting form (tab, sab)
     float tb = 0, sb = 0, gb = 0, tab = 0, sab = 0;
+    // not null: scaled rotations with these coefficients (the rest is unused)
+    const ScaledCoef *sc = nullptr;
 };
-constexpr int FUSED_MAX_K = 8;
 static_assert(sizeof(FusedLaunch::adt) / sizeof(float) == FUSED_MAX_K, "one a_n dt per step");
 constexpr int FUSED_BOX_COLS = 128;   // columns a warp strip loads (box width)
 constexpr int FUSED_BOX_ROWS = 2;     // rows per pipeline slot (box height)
@@ -115,7 +138,6 @@ cudaError_t launch_fused(int K, const FusedLaunch &a, cudaStream_t st);
 // (psi re, im, lambda re, im), psi goes to (out_re, out_im) and lambda to
 // (out2_re, out2_im).  At each step's phase point G += conj(lambda~) m, with
 // lambda~ = B^dagger lambda_s and m = B^dagger psi_s.
-constexpr int FUSED_ADJ_MAX_K = 4;
 cudaError_t launch_fused_adjoint(int K, const FusedLaunch &a, cudaStream_t st);
 // K (1..4) steps with the time-dependent potential V0 + a_n V1: tm_phase
 // maps three planes (gamma_V, s_V, V1) and adt[k] = a_n dt of step k.
@@ -140,6 +162,7 @@ struct GridDesc {
     int nx, ny;
     int64_t pitch;
     float t1, s1, g1, t2, s2;  // rotation coefficients (see FusedLaunch)
+    ScaledCoef sc[FUSED_MAX_K];   // scaled rotations, by depth - 1
 };
 
 // One grid of an epoch: its descriptor, where its work starts in the
@@ -168,11 +191,12 @@ cudaError_t fused_multi_prepare(int K);
 // ranges, so neighbouring strips share halo columns through L2) is taken
 // when its longest warp is within 10 % of the even split's; mixes of many
 // small grids get the even split.  warps == 0 on an error.
-MultiPlan fused_multi_plan(int K, int n, const int *nx, const int *ny, EpochEntry *tab);
+MultiPlan fused_multi_plan(int K, bool scaled, int n, const int *nx, const int *ny,
+                           EpochEntry *tab);
 // K steps for every grid of a device epoch table planned by
 // fused_multi_plan; the input pair of grid i is tab[i].cur0 ^ flip.
-cudaError_t launch_fused_multi(int K, const EpochEntry *tab, int n_grids, const MultiPlan &plan,
-                               int flip, int *err, cudaStream_t st);
+cudaError_t launch_fused_multi(int K, bool scaled, const EpochEntry *tab, int n_grids,
+                               const MultiPlan &plan, int flip, int *err, cudaStream_t st);
 
 // Build a 3-D FP32 tensor map over `planes` consecutive pitched planes
 // (nx x ny each, `plane_bytes` apart) for the fused path.  Its boxes span

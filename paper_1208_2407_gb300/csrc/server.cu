@@ -63,6 +63,7 @@ struct Req {
     void *slab = nullptr;
     cudaEvent_t ready = nullptr;    // inputs uploaded
     bool ready_seen = false;
+    bool scaled = false;            // evolves with scaled rotations (else the lifting form)
     int64_t full_left = 0, rem_left = 0;   // launches still to enqueue
     int64_t t_submit = 0, t_admit = 0, t_done = 0;
     bool cancel = false;
@@ -86,12 +87,13 @@ struct Epoch {
 
 struct GraphKey {
     int slot, n, L, K;
+    bool scaled;
     int warps;
     int64_t units;
     bool aligned;
     bool operator==(const GraphKey &o) const
     {
-        return slot == o.slot && n == o.n && L == o.L && K == o.K && warps == o.warps &&
+        return slot == o.slot && n == o.n && L == o.L && K == o.K && scaled == o.scaled && warps == o.warps &&
                units == o.units && aligned == o.aligned;
     }
 };
@@ -131,7 +133,10 @@ struct ts_server {
     void enqueue_epoch(std::unique_lock<std::mutex> &lk);
     void retire(Epoch &e, bool ok);
     int take_table();
-    cudaError_t launch_full(int slot, int n, const ts::MultiPlan &plan, int L);
+    // the depth of full launches for grids with scaled rotations or in the
+    // lifting form
+    int depth(bool scaled) const { return scaled ? K : std::min(K, (int)ts::FUSED_LIFT_MAX_K); }
+    cudaError_t launch_full(int slot, int n, bool scaled, const ts::MultiPlan &plan, int L);
 };
 
 int ts_server::take_table()
@@ -142,11 +147,12 @@ int ts_server::take_table()
     return s;
 }
 
-cudaError_t ts_server::launch_full(int slot, int n, const ts::MultiPlan &plan, int L)
+cudaError_t ts_server::launch_full(int slot, int n, bool scaled, const ts::MultiPlan &plan, int L)
 {
     const ts::EpochEntry *tab = tab_dev + (size_t)slot * cfg.max_slots;
-    if (L == 1) return ts::launch_fused_multi(K, tab, n, plan, 0, err_dev, compute);
-    const GraphKey key{slot, n, L, K, plan.warps, plan.units, plan.aligned};
+    const int K = depth(scaled);
+    if (L == 1) return ts::launch_fused_multi(K, scaled, tab, n, plan, 0, err_dev, compute);
+    const GraphKey key{slot, n, L, K, scaled, plan.warps, plan.units, plan.aligned};
     for (auto &kv : graphs)
         if (kv.first == key) {
             ++graph_launches;
@@ -156,7 +162,7 @@ cudaError_t ts_server::launch_full(int slot, int n, const ts::MultiPlan &plan, i
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamBeginCapture(compute, cudaStreamCaptureModeThreadLocal);
     for (int t = 0; t < L && e == cudaSuccess; ++t)
-        e = ts::launch_fused_multi(K, tab, n, plan, t & 1, err_dev, compute);
+        e = ts::launch_fused_multi(K, scaled, tab, n, plan, t & 1, err_dev, compute);
     cudaError_t e2 = cudaStreamEndCapture(compute, &graph);
     if (e == cudaSuccess) e = e2;
     cudaGraphExec_t exec = nullptr;
@@ -232,8 +238,9 @@ bool ts_server::admit_one(const ReqP &q)
         q->status = TS_ERR_CUDA;
         return false;
     }
-    q->full_left = r.steps / K;
-    q->rem_left = r.steps % K;
+    q->scaled = std::fabs(r.theta) <= ts::SCALED_MAX_THETA;
+    q->full_left = r.steps / depth(q->scaled);
+    q->rem_left = r.steps % depth(q->scaled);
     return true;
 }
 
@@ -301,7 +308,8 @@ void ts_server::enqueue_epoch(std::unique_lock<std::mutex> &lk)
     for (auto &q : run_full) L = std::min(L, q->full_left);
     lk.unlock();
     cudaError_t e = cudaSuccess;
-    auto upload = [&](const std::vector<ReqP> &set, int depth, ts::MultiPlan &plan) -> int {
+    auto upload = [&](const std::vector<ReqP> &set, int depth, bool scaled,
+                      ts::MultiPlan &plan) -> int {
         const int slot = take_table();
         ts::EpochEntry *h = tab_host + (size_t)slot * cfg.max_slots;
         std::vector<int> nx(set.size()), ny(set.size());
@@ -310,7 +318,7 @@ void ts_server::enqueue_epoch(std::unique_lock<std::mutex> &lk)
             nx[i] = (int)set[i]->r.nx;
             ny[i] = (int)set[i]->r.ny;
         }
-        plan = ts::fused_multi_plan(depth, (int)set.size(), nx.data(), ny.data(), h);
+        plan = ts::fused_multi_plan(depth, scaled, (int)set.size(), nx.data(), ny.data(), h);
         if (plan.warps < 1 && e == cudaSuccess) e = cudaErrorInvalidConfiguration;
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(tab_dev + (size_t)slot * cfg.max_slots, h,
@@ -318,26 +326,34 @@ void ts_server::enqueue_epoch(std::unique_lock<std::mutex> &lk)
         ep.tables.push_back(slot);
         return slot;
     };
-    if (!run_full.empty()) {
-        ts::MultiPlan plan{};
-        const int slot = upload(run_full, K, plan);
-        if (e != cudaSuccess) where = "epoch table upload";
-        if (e == cudaSuccess) {
-            e = launch_full(slot, (int)run_full.size(), plan, (int)L);
-            if (e != cudaSuccess) where = L > 1 ? "epoch graph" : "epoch launch";
+    // grids with scaled rotations, then those in the lifting form: each form
+    // has its full launches and its remainder launches (one per distinct
+    // depth r below the form's)
+    for (const bool scaled : {true, false}) {
+        std::vector<ReqP> full;
+        std::vector<std::vector<ReqP>> by_rem(K);
+        for (auto &q : run_full)
+            if (q->scaled == scaled) full.push_back(q);
+        for (auto &q : run_rem)
+            if (q->scaled == scaled) by_rem[q->rem_left].push_back(q);
+        if (!full.empty() && e == cudaSuccess) {
+            ts::MultiPlan plan{};
+            const int slot = upload(full, depth(scaled), scaled, plan);
+            if (e != cudaSuccess) where = "epoch table upload";
+            if (e == cudaSuccess) {
+                e = launch_full(slot, (int)full.size(), scaled, plan, (int)L);
+                if (e != cudaSuccess) where = L > 1 ? "epoch graph" : "epoch launch";
+            }
         }
-    }
-    // remainder launches (one per distinct depth r < K)
-    std::vector<std::vector<ReqP>> by_rem(K);
-    for (auto &q : run_rem) by_rem[q->rem_left].push_back(q);
-    for (int r = 1; r < K && e == cudaSuccess; ++r) {
-        if (by_rem[r].empty()) continue;
-        ts::MultiPlan plan{};
-        const int slot = upload(by_rem[r], r, plan);
-        if (e == cudaSuccess) {
-            e = ts::launch_fused_multi(r, tab_dev + (size_t)slot * cfg.max_slots,
-                                       (int)by_rem[r].size(), plan, 0, err_dev, compute);
-            if (e != cudaSuccess) where = "remainder launch";
+        for (int r = 1; r < K && e == cudaSuccess; ++r) {
+            if (by_rem[r].empty()) continue;
+            ts::MultiPlan plan{};
+            const int slot = upload(by_rem[r], r, scaled, plan);
+            if (e == cudaSuccess) {
+                e = ts::launch_fused_multi(r, scaled, tab_dev + (size_t)slot * cfg.max_slots,
+                                           (int)by_rem[r].size(), plan, 0, err_dev, compute);
+                if (e != cudaSuccess) where = "remainder launch";
+            }
         }
     }
     ep.err_copy = err_host + (epochs % kTables);

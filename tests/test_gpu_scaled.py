@@ -1,0 +1,85 @@
+"""Scaled rotations of the fused kernels (|theta| <= 0.075): the lanes and rows
+at the edges of the grid take coefficients of their own, by how the side ends in
+a lane's four columns (sides 1 .. 9, around a strip of 112 or 120 columns) and
+by its parity, at every depth; the largest angle of the form and the first one
+beyond it, which takes the lifting form.
+
+Tolerances.  A step rounds each component about 10 times (six sweeps, the phase
+and the scale) by at most 2^-24 relative, and 13 steps add up like a random
+walk: 2^-24 sqrt(130) = 7e-7, with a factor 3 for the tails and the rounding of
+the coefficients: 2e-6.  The scale's rounding adds at most 1e-9 to the norm per
+step, the random roundings 2^-24 sqrt(130 / sites), so 13 steps stay within
+1.3e-8 + 3 * 7e-7 / sqrt(sites); the input's rounding to FP32 adds up to 2^-23."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1208_2407_gb300 import trotter
+from gpu_helpers import random_state, rel_l2, run_gpu
+
+pytestmark = pytest.mark.gpu
+
+STEPS, TOL = 13, 2e-6
+SIDES = [(1, 9), (2, 8), (3, 7), (4, 6), (5, 5), (6, 4), (7, 3), (8, 2), (9, 1), (111, 12),
+         (112, 13), (113, 14), (114, 5), (115, 6), (116, 33), (119, 8), (120, 7), (121, 6),
+         (225, 40), (226, 41)]
+
+
+@pytest.mark.parametrize("nx,ny", SIDES)
+@pytest.mark.parametrize("theta", [0.075, -0.075, 0.0751])
+def test_edges_at_every_depth(nx, ny, theta):
+    rng = np.random.default_rng(nx * 1009 + ny)
+    re, im = random_state(rng, nx, ny)
+    V = rng.uniform(-0.5, 0.5, (ny, nx))
+    dt = 2.0 * theta
+    ore, oim = oracle.evolve(re, im, V, dt, theta, STEPS)
+    for K in range(0, 9):
+        (gre, gim), _ = run_gpu(re, im, V, dt, theta, STEPS, K=K)
+        assert rel_l2(gre, gim, ore, oim) < TOL, K
+        drift = abs(np.sum(gre * gre + gim * gim) - np.sum(ore * ore + oim * oim))
+        assert drift < 1.3e-8 + 3 * 7e-7 / np.sqrt(nx * ny) + 1.2e-7, (K, drift)
+
+
+@pytest.mark.parametrize("nx,ny,nz", [(1, 1, 2), (2, 3, 4), (3, 2, 5), (113, 4, 3), (5, 7, 22),
+                                      (9, 6, 23)])
+@pytest.mark.parametrize("theta", [0.075, 0.0751])
+def test_edges_3d(nx, ny, nz, theta):
+    rng = np.random.default_rng(nx + 31 * ny + 97 * nz)
+    re, im = rng.standard_normal((2, nz, ny, nx))
+    s = np.sqrt(np.sum(re * re + im * im))
+    re, im = re / s, im / s
+    V = rng.uniform(-0.5, 0.5, (nz, ny, nx))
+    g = trotter.Grid(nx, ny, "f32", nz=nz)
+    try:
+        g.set_state(re, im)
+        g.set_potential(V, 2.0 * theta, theta)
+        g.evolve(STEPS)
+        gre, gim = g.get_state(np.float64)
+    finally:
+        g.close()
+    ore, oim = oracle.evolve3(re, im, V, 2.0 * theta, theta, STEPS)
+    assert rel_l2(gre, gim, ore, oim) < TOL
+
+
+def test_batch_of_both_forms_equals_solo_runs():
+    """A batch of grids on either side of the largest scaled angle: each form
+    has its own launches, and each grid's result is its solo result."""
+    rng = np.random.default_rng(5)
+    cases = [(130, 66, 0.075, 9), (64, 40, 0.2, 11), (33, 57, 0.0751, 6), (250, 9, 0.01, 7)]
+    grids, want = [], []
+    try:
+        for nx, ny, theta, steps in cases:
+            re, im = random_state(rng, nx, ny)
+            V = rng.uniform(-0.5, 0.5, (ny, nx))
+            g = trotter.Grid(nx, ny, "f32")
+            g.set_state(re, im)
+            g.set_potential(V, 0.05, theta)
+            grids.append(g)
+            want.append(run_gpu(re, im, V, 0.05, theta, steps, K=0)[0])
+        trotter.evolve_batched(grids, [c[3] for c in cases])
+        for g, (wre, wim) in zip(grids, want):
+            gre, gim = g.get_state(np.float64)
+            assert np.array_equal(gre, wre) and np.array_equal(gim, wim)
+    finally:
+        for g in grids:
+            g.close()
