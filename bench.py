@@ -266,7 +266,7 @@ def kernel_source_hash() -> str:
     import hashlib
     import re
     h = hashlib.sha256()
-    for name in ("fused.cu", "common.cuh", "ffloat.cuh", "internal.h", "mbar.cuh"):
+    for name in ("fused.cu", "scaled.cuh", "common.cuh", "ffloat.cuh", "internal.h", "mbar.cuh"):
         with open(os.path.join(ROOT, "paper_1208_2407_gb300", "csrc", name)) as f:
             text = f.read()
         text = re.sub(r"/\*.*?\*/", " ", text, flags=re.S)   # block comments

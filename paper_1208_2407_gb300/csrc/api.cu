@@ -220,6 +220,8 @@ void grid_write_desc(ts_grid *g, cudaStream_t st)
     d.g1 = (float)g->g1;
     d.t2 = (float)g->t2;
     d.s2 = (float)g->s2;
+    d.pg = (const float *)g->pg();
+    d.ps = (const float *)g->ps();
     const double sub[FUSED_MAX_K] = {g->theta, g->theta, g->theta, g->theta,
                                      g->theta, g->theta, g->theta, g->theta};
     for (int K = 1; K <= FUSED_MAX_K; ++K)
@@ -824,9 +826,10 @@ ts_status merged_run(ts_grid *g, int64_t n, SubAt sub, cudaStream_t st)
 }  // extern "C++"
 
 // `steps` second-order steps on the fused path at depth K (a remainder runs
-// at a smaller depth), at kinetic half angle theta with the phase table map tm.
+// at a smaller depth), at kinetic half angle theta with the phase table map tm
+// and the table's planes at pg.
 ts_status fused_run(ts_grid *g, int64_t steps, int K, double theta, const CUtensorMap *tm,
-                    cudaStream_t st, const double *drive_adt = nullptr)
+                    const void *pg, cudaStream_t st, const double *drive_adt = nullptr)
 {
     if (!g->tmaps_ok) return fail(TS_ERR_STATE, "fused path: tensor maps missing");
     const bool scaled = std::fabs(theta) <= ts::SCALED_MAX_THETA;
@@ -858,7 +861,15 @@ ts_status fused_run(ts_grid *g, int64_t steps, int K, double theta, const CUtens
         a.s2 = (float)c.s2;
         a.err = g->err;
         cudaError_t e;
-        if (drive_adt) {
+        const int nx = a.nx, ny = a.ny;
+        const int shape = scaled && !drive_adt ? ts::tile_shape(k, 1, &nx, &ny) : -1;
+        if (shape >= 0) {
+            const ts::TileLaunch t = {(const float *)g->re(), (const float *)g->im(),
+                                      (const float *)pg,
+                                      (const float *)pg + g->L.plane_bytes / sizeof(float),
+                                      a.out_re, a.out_im, a.nx, a.ny, a.pitch, &sc};
+            e = ts::launch_tile(k, shape, t, st);
+        } else if (drive_adt) {
             for (int i = 0; i < k; ++i) a.adt[i] = (float)drive_adt[steps - left + i];
             e = ts::launch_fused_drive(k, a, st);
         } else {
@@ -880,7 +891,7 @@ ts_status plain_steps(ts_grid *g, int64_t steps, cudaStream_t st)
 
 ts_status fused_steps(ts_grid *g, int64_t steps, int K, cudaStream_t st)
 {
-    return fused_run(g, steps, K, g->theta, &g->tm_phase, st);
+    return fused_run(g, steps, K, g->theta, &g->tm_phase, g->pg(), st);
 }
 
 // Fourth-order steps (Eq. fourthorder): the substeps a = U2(p dt) and
@@ -945,7 +956,7 @@ ts_status evolve_driven(ts_grid *g, int64_t steps, int K, bool plain, cudaStream
         // site-steps/s against 3.8e11 at depth 3)
         int depth = K == 0 ? ts::FUSED_DRIVE_MAX_K : K;
         if (depth > ts::FUSED_DRIVE_MAX_K) depth = ts::FUSED_DRIVE_MAX_K;
-        s = fused_run(g, steps, depth, g->theta, &g->tm_drive, st, adt.data());
+        s = fused_run(g, steps, depth, g->theta, &g->tm_drive, nullptr, st, adt.data());
     }
     if (s == TS_OK) g->drive_pos += steps;
     return s;
@@ -1006,14 +1017,14 @@ ts_status evolve4(ts_grid *g, int64_t steps, int K, bool plain, cudaStream_t st)
         const int64_t n = (r + depth - 1) / depth;
         for (int64_t i = 0; i < n; ++i) {
             const int64_t k = r / n + (i < r % n ? 1 : 0);
-            ts_status s = fused_run(g, k, (int)k, w[0] * g->theta, &g->tm_phase, st);
+            ts_status s = fused_run(g, k, (int)k, w[0] * g->theta, &g->tm_phase, g->pg(), st);
             if (s != TS_OK) return s;
         }
         return TS_OK;
     };
     auto run_b = [&]() -> ts_status {
         if (plain) return plain_run(g, 1, g->sub[1], g->pg_b(), g->ps_b(), st);
-        return fused_run(g, 1, 1, w[1] * g->theta, &g->tm_phase_b, st);
+        return fused_run(g, 1, 1, w[1] * g->theta, &g->tm_phase_b, g->pg_b(), st);
     };
     ts_status s = run_a(2);
     for (int64_t n = 0; n < steps && s == TS_OK; ++n) {

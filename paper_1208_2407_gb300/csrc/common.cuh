@@ -163,6 +163,13 @@ __device__ __forceinline__ void grid_dep_sync()
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// Let the next kernel's blocks become resident: they run up to their own
+// grid_dep_sync while this kernel finishes.
+__device__ __forceinline__ void grid_dep_launch()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 __device__ __forceinline__ uint64_t globaltimer_ns()
 {
     uint64_t t;

@@ -152,6 +152,25 @@ cudaError_t launch_fused_u4(const FusedLaunch &a, cudaStream_t st);
 // the result.  Needs (nz + 32) * ny < 2^31.
 cudaError_t launch_fused3d(const FusedLaunch &a, int nz, cudaStream_t st);
 
+// --- fused steps on tiles held in registers (tile.cu) ---------------------
+constexpr int TILE_MAX_K = 4;
+struct TileLaunch {
+    const float *in_re, *in_im, *pg, *ps;   // state and phase table
+    float *out_re, *out_im;
+    int nx, ny;
+    int64_t pitch;
+    const ScaledCoef *sc;   // of depth K
+};
+// The tile shape for a launch of depth K over n grids with scaled rotations,
+// or -1 where the warp streams are faster (or K > TILE_MAX_K).
+constexpr int TILE_SHAPES = 3;
+int tile_shape(int K, int n, const int *nx, const int *ny);
+// Blocks of one grid at that shape.
+int tile_blocks(int K, int shape, int nx, int ny);
+// K steps (1..TILE_MAX_K): what launch_fused with scaled rotations gives at
+// that depth, bit for bit.
+cudaError_t launch_tile(int K, int shape, const TileLaunch &a, cudaStream_t st);
+
 // Device-resident description of one FP32 grid for the multi-grid launch
 // (written once per grid set-up; read by the kernel with generic loads, its
 // tensor maps by TMA).
@@ -163,6 +182,7 @@ struct GridDesc {
     int64_t pitch;
     float t1, s1, g1, t2, s2;  // rotation coefficients (see FusedLaunch)
     ScaledCoef sc[FUSED_MAX_K];   // scaled rotations, by depth - 1
+    const float *pg, *ps;      // the phase table's planes
 };
 
 // One grid of an epoch: its descriptor, where its work starts in the
@@ -181,6 +201,7 @@ struct MultiPlan {
     int warps;       // warps launched
     int64_t units;   // row-pair units of all grids (strips x row pairs)
     bool aligned;    // strip-aligned (per-grid warps per strip) or even split
+    int shape;       // >= 0: a launch of tiles of that shape instead (units: its blocks)
 };
 
 // Set the multi-grid kernel's attributes for depth K (call outside stream capture).
@@ -195,6 +216,10 @@ MultiPlan fused_multi_plan(int K, bool scaled, int n, const int *nx, const int *
                            EpochEntry *tab);
 // K steps for every grid of a device epoch table planned by
 // fused_multi_plan; the input pair of grid i is tab[i].cur0 ^ flip.
+// A plan with a tile shape runs as tiles (tile.cu), which report no error.
+cudaError_t tile_multi_prepare();
+cudaError_t launch_tile_multi(int K, int shape, const EpochEntry *tab, int n, int blocks, int flip,
+                              cudaStream_t st);
 cudaError_t launch_fused_multi(int K, bool scaled, const EpochEntry *tab, int n_grids,
                                const MultiPlan &plan, int flip, int *err, cudaStream_t st);
 

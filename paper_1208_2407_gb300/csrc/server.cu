@@ -91,10 +91,11 @@ struct GraphKey {
     int warps;
     int64_t units;
     bool aligned;
+    int shape;
     bool operator==(const GraphKey &o) const
     {
         return slot == o.slot && n == o.n && L == o.L && K == o.K && scaled == o.scaled && warps == o.warps &&
-               units == o.units && aligned == o.aligned;
+               units == o.units && aligned == o.aligned && shape == o.shape;
     }
 };
 
@@ -152,7 +153,7 @@ cudaError_t ts_server::launch_full(int slot, int n, bool scaled, const ts::Multi
     const ts::EpochEntry *tab = tab_dev + (size_t)slot * cfg.max_slots;
     const int K = depth(scaled);
     if (L == 1) return ts::launch_fused_multi(K, scaled, tab, n, plan, 0, err_dev, compute);
-    const GraphKey key{slot, n, L, K, scaled, plan.warps, plan.units, plan.aligned};
+    const GraphKey key{slot, n, L, K, scaled, plan.warps, plan.units, plan.aligned, plan.shape};
     for (auto &kv : graphs)
         if (kv.first == key) {
             ++graph_launches;
