@@ -152,6 +152,29 @@ cudaError_t launch_fused_u4(const FusedLaunch &a, cudaStream_t st);
 // the result.  Needs (nz + 32) * ny < 2^31.
 cudaError_t launch_fused3d(const FusedLaunch &a, int nz, cudaStream_t st);
 
+// --- fused FP64 steps (fused64.cu) -----------------------------------------
+// A scaled sweep: the bulk tangent, and what a pair with a member on an edge
+// receives (the edge member lo, its partner hi).
+struct Sweep64 {
+    double t, lo, hi;
+};
+// One launch Ye Yo P Yo (Xo Xe Xo), the last of a run without its second Xo;
+// or the tail: Ye and the scale (sx, sy by place: 0 bulk, 1 first, 2 last).
+struct Step64 {
+    const double *in_re, *in_im, *pg, *ps;
+    double *out_re, *out_im;
+    int nx, ny;
+    int64_t pitch;
+    Sweep64 ye, yo1, yo2, xo1, xe, xo2;
+    double sx[3], sy[3];
+    int last;
+    int n_strips, rows;   // set by plan_step64: strips, rows per range (even)
+};
+// Set the split; cols (columns per lane) and blocks go to launch_step64.
+void plan_step64(Step64 &p, int num_sms, int &cols, int &blocks);
+cudaError_t launch_step64(const Step64 &p, int cols, int blocks, cudaStream_t st);
+cudaError_t launch_tail64(const Step64 &p, cudaStream_t st);
+
 // --- fused steps on tiles held in registers (tile.cu) ---------------------
 constexpr int TILE_MAX_K = 4;
 struct TileLaunch {
@@ -164,6 +187,7 @@ struct TileLaunch {
 // The tile shape for a launch of depth K over n grids with scaled rotations,
 // or -1 where the warp streams are faster (or K > TILE_MAX_K).
 constexpr int TILE_SHAPES = 3;
+int num_sms();   // of the device current at the first call
 int tile_shape(int K, int n, const int *nx, const int *ny);
 // Blocks of one grid at that shape.
 int tile_blocks(int K, int shape, int nx, int ny);

@@ -305,18 +305,6 @@ cudaError_t launch_many(int K, const EpochEntry *tab, int n, int blocks, int fli
     return e;
 }
 
-int num_sms()
-{
-    static const int n = [] {
-        int dev = 0, v = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-            v = 1;
-        return v;
-    }();
-    return n;
-}
-
 // The tile shapes: rows per warp and warps per block.
 struct Shape {
     int r, w;
@@ -330,6 +318,18 @@ int64_t tiles_of(int K, const Shape &s, int nx, int ny)
 }
 
 }  // namespace
+
+int num_sms()
+{
+    static const int n = [] {
+        int dev = 0, v = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+            v = 1;
+        return v;
+    }();
+    return n;
+}
 
 int tile_blocks(int K, int shape, int nx, int ny) { return (int)tiles_of(K, shapes[shape], nx, ny); }
 
