@@ -1132,7 +1132,7 @@ ts_status fused64_run(ts_grid *g, int64_t n, SubAt sub, cudaStream_t st)
 // FP64 grids that take fused64_run: 2-D, no drive, every angle within tan <= 1
 // (the merged ones too), and 1024 sites or more: below that a step is nothing
 // but launches, and the sweeps' sequence stays as it is.  (256^2: 12.6 us per
-// step in sweeps, fused 6; 2047 x 1536: 160 and 100.)
+// step in sweeps, 7.9 fused; 2047 x 1536: 160 and 107.)
 bool fused64_ok(const ts_grid *g, double max_theta)
 {
     return !g->is3d() && !g->driven && g->L.nx * g->L.ny >= 1024 &&

@@ -246,9 +246,12 @@ tail64_kernel(const __grid_constant__ Step64 p)
 
 }  // namespace
 
-// Columns per lane and rows per range: the least time of an SM's share.  A
-// range of h rows takes (16 h + 24) C warp-wide DFMAs; up to 4 warps of an SM
-// run side by side (3 or fewer 1.19 times as fast), more share its units.
+// Columns per lane and rows per range.  A range of h rows takes (16 h + 24) C
+// warp-wide DFMAs per warp, one warp per scheduler in a block; an SM's blocks
+// share its units two at a time, and a block that runs alone takes 1.3 times as
+// long, since nothing covers its shuffles and loads (2047 x 1536, C = 4: h = 44,
+// one block per SM, 136 us per step; h = 22, two, 107 us; h = 16, three, 128 us;
+// h = 12, four, 123 us).  The FP64 units alone would need 97 us there.
 void plan_step64(Step64 &p, int num_sms, int &cols, int &blocks)
 {
     double best = 0.0;
@@ -259,8 +262,8 @@ void plan_step64(Step64 &p, int num_sms, int &cols, int &blocks)
         for (int hp = 1; hp <= pairs; hp = hp < 64 ? hp + 1 : hp * 9 / 8) {
             const int64_t items = (int64_t)strips * ((pairs + hp - 1) / hp);
             const int64_t nb = (items + kWarps - 1) / kWarps;
-            const double rounds = (double)((nb + num_sms - 1) / num_sms);
-            const double t = rounds * (32.0 * hp + 24.0) * C;
+            const int64_t rounds = (nb + num_sms - 1) / num_sms;
+            const double t = ((double)rounds + (rounds & 1 ? 0.3 : 0.0)) * (32.0 * hp + 24.0) * C;
             if (cols == 0 || t < best * 0.999) {
                 best = t;
                 cols = C;

@@ -11,6 +11,8 @@
 // FP64 grids: every term in FP64; each thread sums a run of 4 sites in
 // plain FP64 and adds the run into Neumaier-compensated per-thread sums.
 // Either way the block writes FP64 partials and a final block sums them.
+#include <algorithm>
+
 #include "common.cuh"
 #include "ffloat.cuh"
 #include "internal.h"
@@ -40,42 +42,51 @@ __device__ __forceinline__ void neu_merge(Neu &a, const Neu &b)
     a.c += b.c;
 }
 
-// Block-level Neumaier reduction of NQ per-thread sums into partials.
-template <int NQ>
-__device__ __forceinline__ void block_reduce_write(Neu (&acc)[NQ], double *__restrict__ partials)
+// Sum a quantity over the block: lane l of one warp adds the values of
+// threads l, l + 32, ... (a value is v.x + v.y, v.y its low part), then the
+// lanes' sums are merged.
+template <typename V2>
+__device__ __forceinline__ Neu warp_sum(const V2 *v, int lane)
 {
-    __shared__ double sh_s[kThreads / 32][NQ], sh_c[kThreads / 32][NQ];
+    Neu a = {0.0, 0.0};
+#pragma unroll
+    for (int i = 0; i < kThreads / 32; ++i) {
+        const V2 x = v[lane + 32 * i];
+        a.add((double)x.x);
+        a.c += (double)x.y;
+    }
+    return a;
+}
+
+__device__ __forceinline__ Neu warp_merge(Neu a)
+{
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        Neu b;
+        b.s = __shfl_down_sync(0xffffffffu, a.s, off);
+        b.c = __shfl_down_sync(0xffffffffu, a.c, off);
+        neu_merge(a, b);
+    }
+    return a;
+}
+
+// Block-level compensated reduction of NQ per-thread sums into partials, one
+// warp per quantity.  The FP64 units bound it (64 cycles per warp-wide
+// operation and scheduler): so shared, a block takes about 90 of them per
+// quantity; with every warp merging all quantities over its lanes first it took
+// 270 (a whole ts_observe at 128^2: 117 -> 42 us; 2048^2: 217 -> 79 us).
+template <int NQ, typename V2>
+__device__ __forceinline__ void block_reduce_write(const V2 (&acc)[NQ], double *__restrict__ partials)
+{
+    __shared__ V2 sh[NQ][kThreads];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        Neu a = acc[q];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            Neu b;
-            b.s = __shfl_down_sync(0xffffffffu, a.s, off);
-            b.c = __shfl_down_sync(0xffffffffu, a.c, off);
-            neu_merge(a, b);
-        }
-        if (lane == 0) {
-            sh_s[warp][q] = a.s;
-            sh_c[warp][q] = a.c;
-        }
-    }
+    for (int q = 0; q < NQ; ++q) sh[q][threadIdx.x] = acc[q];
     __syncthreads();
-    if (warp == 0) {
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-            Neu a = {0.0, 0.0};
-            if (lane < kThreads / 32) a = {sh_s[lane][q], sh_c[lane][q]};
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                Neu b;
-                b.s = __shfl_down_sync(0xffffffffu, a.s, off);
-                b.c = __shfl_down_sync(0xffffffffu, a.c, off);
-                neu_merge(a, b);
-            }
-            if (lane == 0) partials[(int64_t)blockIdx.x * OBS_Q + q] = a.val();
-        }
+    constexpr int stride = NQ > OBS_Q ? NQ : OBS_Q;
+    for (int q = warp; q < NQ; q += kThreads / 32) {
+        const Neu a = warp_merge(warp_sum(sh[q], lane));
+        if (lane == 0) partials[(int64_t)blockIdx.x * stride + q] = a.val();
     }
 }
 
@@ -86,8 +97,8 @@ __device__ __forceinline__ void block_reduce_write(Neu (&acc)[NQ], double *__res
 template <bool NORM_ONLY>
 __global__ void __launch_bounds__(kThreads)
 observe_f32_kernel(const float *__restrict__ re, const float *__restrict__ im,
-                   const float *__restrict__ vp, int nx, int ny, int64_t pitch, float J_hi,
-                   float J_lo, double *__restrict__ partials)
+                   const float *__restrict__ vp, int nx, int ny, int64_t pitch,
+                   double *__restrict__ partials)
 {
     grid_dep_sync();
     constexpr int NQ = NORM_ONLY ? 1 : OBS_Q;
@@ -158,20 +169,10 @@ observe_f32_kernel(const float *__restrict__ re, const float *__restrict__ im,
             acc[6] = ff_add(acc[6], VP);
         }
     }
-    Neu nacc[NQ];
+    float2 sums[NQ];
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        nacc[q] = {0.0, 0.0};
-        nacc[q].add((double)acc[q].hi);
-        nacc[q].add((double)acc[q].lo);
-    }
-    if constexpr (!NORM_ONLY) {
-        // kinetic: -2 J * sum Re(conj(psi_j) psi_k), J = J_hi + J_lo
-        const double k = nacc[5].val();
-        nacc[5] = {0.0, 0.0};
-        nacc[5].add(-2.0 * ((double)J_hi + (double)J_lo) * k);
-    }
-    block_reduce_write<NQ>(nacc, partials);
+    for (int q = 0; q < NQ; ++q) sums[q] = make_float2(acc[q].hi, acc[q].lo);
+    block_reduce_write<NQ>(sums, partials);
 }
 
 // <phi|psi>: exact products, double-float per-thread sums, FP64 combine.
@@ -204,112 +205,26 @@ inner_f32_kernel(const float *__restrict__ ar, const float *__restrict__ ai,
             si = ff_add(si, ff_add(two_prod(pr[u], qi[u]), two_prod(-pi[u], qr[u])));
         }
     }
-    Neu acc[2];
-    acc[0] = {0.0, 0.0};
-    acc[1] = {0.0, 0.0};
-    acc[0].add((double)sr.hi);
-    acc[0].add((double)sr.lo);
-    acc[1].add((double)si.hi);
-    acc[1].add((double)si.lo);
-    block_reduce_write<2>(acc, partials);
+    const float2 sums[2] = {make_float2(sr.hi, sr.lo), make_float2(si.hi, si.lo)};
+    block_reduce_write<2>(sums, partials);
 }
 
-template <typename T, bool NORM_ONLY>
+// Observables in FP64 (2-D or 3-D grids; slab z = rows z*ny .. z*ny + ny - 1):
+// runs of 4 sites are summed plainly and added into Neumaier-compensated
+// per-thread sums.  The FP64 units bound it, so a run sums p, u p and u^2 p
+// (u = 0 .. 3) and expands x = x0 + u, y and z once per run, and the kinetic
+// sum takes its factor -2 J in the final pass (a whole ts_observe at 2047 x 1536: 355 -> 190 us, at 256^3 1856 -> 1215 us).
+template <typename T, bool NORM_ONLY, bool THREE>
 __global__ void __launch_bounds__(kThreads)
 observe_kernel(const T *__restrict__ re, const T *__restrict__ im, const T *__restrict__ vp,
-               int nx, int ny, int64_t pitch, double J, double *__restrict__ partials)
+               int nx, int ny, int nz, int64_t pitch, double *__restrict__ partials)
 {
     grid_dep_sync();
-    constexpr int NQ = NORM_ONLY ? 1 : OBS_Q;
+    constexpr int NQ = NORM_ONLY ? 1 : THREE ? OBS_Q3 : OBS_Q;
     Neu acc[NQ];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) acc[q] = {0.0, 0.0};
 
-    const int chunks_per_row = (nx + 3) / 4;
-    const int64_t nchunks = (int64_t)chunks_per_row * ny;
-    for (Walk w(chunks_per_row, blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
-                (int64_t)gridDim.x * blockDim.x);
-         w.i < nchunks; w.next()) {
-        const int y = (int)w.y;
-        const int x0 = (int)w.x * 4;
-        const int64_t o = (int64_t)y * pitch;
-        double run[NQ];
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) run[q] = 0.0;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int x = x0 + u;
-            if (x >= nx) break;
-            const double r = (double)re[o + x], m = (double)im[o + x];
-            const double p = r * r + m * m;
-            run[0] += p;
-            if constexpr (!NORM_ONLY) {
-                run[1] += (double)x * p;
-                run[2] += (double)y * p;
-                run[3] += (double)x * (double)x * p;
-                run[4] += (double)y * (double)y * p;
-                double kin = 0.0;
-                if (x + 1 < nx)
-                    kin += r * (double)re[o + x + 1] + m * (double)im[o + x + 1];
-                if (y + 1 < ny)
-                    kin += r * (double)re[o + pitch + x] + m * (double)im[o + pitch + x];
-                run[5] += -2.0 * J * kin;
-                run[6] += (double)vp[o + x] * p;
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) acc[q].add(run[q]);
-    }
-
-    // block reduction: warp shuffles, then one warp over the warp results
-    __shared__ double sh_s[kThreads / 32][NQ], sh_c[kThreads / 32][NQ];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        Neu a = acc[q];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            Neu b;
-            b.s = __shfl_down_sync(0xffffffffu, a.s, off);
-            b.c = __shfl_down_sync(0xffffffffu, a.c, off);
-            neu_merge(a, b);
-        }
-        if (lane == 0) {
-            sh_s[warp][q] = a.s;
-            sh_c[warp][q] = a.c;
-        }
-    }
-    __syncthreads();
-    if (warp == 0) {
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-            Neu a = {0.0, 0.0};
-            if (lane < kThreads / 32) a = {sh_s[lane][q], sh_c[lane][q]};
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                Neu b;
-                b.s = __shfl_down_sync(0xffffffffu, a.s, off);
-                b.c = __shfl_down_sync(0xffffffffu, a.c, off);
-                neu_merge(a, b);
-            }
-            if (lane == 0) partials[(int64_t)blockIdx.x * OBS_Q + q] = a.val();
-        }
-    }
-}
-
-// Observables of a 3-D grid (slab z = rows z*ny .. z*ny + ny - 1): every
-// term in FP64 (it is called at report points only), runs of 4 sites summed
-// plainly and added into Neumaier-compensated per-thread sums.
-template <typename T>
-__global__ void __launch_bounds__(kThreads)
-observe3_kernel(const T *__restrict__ re, const T *__restrict__ im, const T *__restrict__ vp,
-                int nx, int ny, int nz, int64_t pitch, double J, double *__restrict__ partials)
-{
-    grid_dep_sync();
-    constexpr int NQ = OBS_Q3;
-    Neu acc[NQ];
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) acc[q] = {0.0, 0.0};
     const int64_t rows = (int64_t)ny * nz;
     const int64_t slab = (int64_t)ny * pitch;
     const int chunks_per_row = (nx + 3) / 4;
@@ -317,108 +232,88 @@ observe3_kernel(const T *__restrict__ re, const T *__restrict__ im, const T *__r
     for (Walk w(chunks_per_row, blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
                 (int64_t)gridDim.x * blockDim.x);
          w.i < nchunks; w.next()) {
-        const int64_t r = w.y;
+        const int64_t row = w.y;
         const int x0 = (int)w.x * 4;
-        const int z = (int)(r / ny), y = (int)(r - (int64_t)z * ny);
-        const int64_t o = r * pitch;
-        double run[NQ];
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) run[q] = 0.0;
+        const int z = THREE ? (int)(row / ny) : 0, y = (int)(row - (int64_t)z * ny);
+        const int64_t o = row * pitch + x0;
+        const bool down = y + 1 < ny, below = THREE && z + 1 < nz;
+        double P = 0.0, XP = 0.0, X2P = 0.0, KIN = 0.0, VP = 0.0;
+        double r = (double)re[o], m = (double)im[o];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const int x = x0 + u;
-            if (x >= nx) break;
-            const double a = (double)re[o + x], b = (double)im[o + x];
-            const double p = a * a + b * b;
-            run[0] += p;
-            run[1] += (double)x * p;
-            run[2] += (double)y * p;
-            run[3] += (double)x * (double)x * p;
-            run[4] += (double)y * (double)y * p;
-            double kin = 0.0;
-            if (x + 1 < nx) kin += a * (double)re[o + x + 1] + b * (double)im[o + x + 1];
-            if (y + 1 < ny) kin += a * (double)re[o + pitch + x] + b * (double)im[o + pitch + x];
-            if (z + 1 < nz) kin += a * (double)re[o + slab + x] + b * (double)im[o + slab + x];
-            run[5] += -2.0 * J * kin;
-            run[6] += (double)vp[o + x] * p;
-            run[7] += (double)z * p;
-            run[8] += (double)z * (double)z * p;
-        }
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) acc[q].add(run[q]);
-    }
-    __shared__ double sh_s[kThreads / 32][NQ], sh_c[kThreads / 32][NQ];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        Neu a = acc[q];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            Neu b;
-            b.s = __shfl_down_sync(0xffffffffu, a.s, off);
-            b.c = __shfl_down_sync(0xffffffffu, a.c, off);
-            neu_merge(a, b);
-        }
-        if (lane == 0) {
-            sh_s[warp][q] = a.s;
-            sh_c[warp][q] = a.c;
-        }
-    }
-    __syncthreads();
-    if (warp == 0) {
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-            Neu a = {0.0, 0.0};
-            if (lane < kThreads / 32) a = {sh_s[lane][q], sh_c[lane][q]};
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                Neu b;
-                b.s = __shfl_down_sync(0xffffffffu, a.s, off);
-                b.c = __shfl_down_sync(0xffffffffu, a.c, off);
-                neu_merge(a, b);
+            if (x0 + u >= nx) break;
+            const double p = fma(r, r, m * m);
+            P += p;
+            if constexpr (!NORM_ONLY) {
+                if (u == 1) {
+                    XP += p;
+                    X2P += p;
+                } else if (u > 1) {
+                    XP = fma((double)u, p, XP);
+                    X2P = fma((double)(u * u), p, X2P);
+                }
+                VP = fma((double)vp[o + u], p, VP);
+                if (down)
+                    KIN = fma(r, (double)re[o + pitch + u], fma(m, (double)im[o + pitch + u], KIN));
+                if (below)
+                    KIN = fma(r, (double)re[o + slab + u], fma(m, (double)im[o + slab + u], KIN));
             }
-            if (lane == 0) partials[(int64_t)blockIdx.x * OBS_Q3 + q] = a.val();
+            if (x0 + u + 1 < nx) {
+                const double rn = (double)re[o + u + 1], mn = (double)im[o + u + 1];
+                if constexpr (!NORM_ONLY) KIN = fma(r, rn, fma(m, mn, KIN));
+                r = rn;
+                m = mn;
+            }
         }
+        acc[0].add(P);
+        if constexpr (!NORM_ONLY) {
+            const double fx = (double)x0, fy = (double)y;
+            acc[1].add(fma(fx, P, XP));
+            acc[2].add(fy * P);
+            acc[3].add(fma(fx, fma(fx, P, 2.0 * XP), X2P));
+            acc[4].add(fy * fy * P);
+            acc[5].add(KIN);
+            acc[6].add(VP);
+            if constexpr (THREE) {
+                const double fz = (double)z;
+                acc[7].add(fz * P);
+                acc[8].add(fz * fz * P);
+            }
+        }
+    }
+    double2 sums[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) sums[q] = make_double2(acc[q].s, acc[q].c);
+    block_reduce_write<NQ>(sums, partials);
+}
+
+// The blocks' partials: one warp per quantity.  Quantity 5 is the kinetic sum,
+// which takes its factor here.
+__global__ void __launch_bounds__(kThreads)
+observe_finalize_kernel(const double *__restrict__ partials, int nblocks, int nq, int stride,
+                        double kin_factor, double *__restrict__ result)
+{
+    grid_dep_sync();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int q = warp; q < nq; q += kThreads / 32) {
+        Neu a = {0.0, 0.0};
+        for (int b = lane; b < nblocks; b += 32) a.add(partials[(int64_t)b * stride + q]);
+        a = warp_merge(a);
+        if (lane == 0) result[q] = q == 5 ? kin_factor * a.val() : a.val();
     }
 }
 
-__global__ void __launch_bounds__(kThreads)
-observe_finalize_kernel(const double *__restrict__ partials, int nblocks, int nq, int stride,
-                        double *__restrict__ result)
+// Blocks of a reduction over nchunks runs of 4 sites.  More blocks per SM hide
+// the loads but add block reductions, which the FP64 units take one after the
+// other: FP32 grids get 1, 2 from 8 and 4 from 64 runs per thread and SM-filling
+// block (observables at 1001 x 777: 54, 58, 80 us with 1, 2, 4; at 8192^2: 636,
+// 436, 428 us; norm at 8192^2: 372, 217, 153 us), FP64 kernels, bound by those
+// units in any case, 1 (2047 x 1536: 189, 191, 213 us).
+int reduce_blocks(int64_t nchunks, bool fp64)
 {
-    grid_dep_sync();
-    __shared__ double sh_s[kThreads / 32], sh_c[kThreads / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int q = 0; q < nq; ++q) {
-        Neu a = {0.0, 0.0};
-        for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
-            a.add(partials[(int64_t)b * stride + q]);
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            Neu o;
-            o.s = __shfl_down_sync(0xffffffffu, a.s, off);
-            o.c = __shfl_down_sync(0xffffffffu, a.c, off);
-            neu_merge(a, o);
-        }
-        if (lane == 0) {
-            sh_s[warp] = a.s;
-            sh_c[warp] = a.c;
-        }
-        __syncthreads();
-        if (warp == 0) {
-            Neu t = {0.0, 0.0};
-            if (lane < kThreads / 32) t = {sh_s[lane], sh_c[lane]};
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                Neu o;
-                o.s = __shfl_down_sync(0xffffffffu, t.s, off);
-                o.c = __shfl_down_sync(0xffffffffu, t.c, off);
-                neu_merge(t, o);
-            }
-            if (lane == 0) result[q] = t.val();
-        }
-        __syncthreads();
-    }
+    const int64_t per = (nchunks + kThreads - 1) / kThreads, sms = num_sms();
+    const int64_t most = fp64 ? sms : per >= 64 * sms ? 4 * sms : per >= 8 * sms ? 2 * sms : sms;
+    return (int)std::max<int64_t>(1, std::min({per, most, (int64_t)OBS_MAX_BLOCKS}));
 }
 
 }  // namespace
@@ -427,23 +322,26 @@ cudaError_t launch_observe(const void *re, const void *im, const void *vplane, b
                            int ny, int64_t pitch, double J, bool norm_only, double *partials,
                            double *result, cudaStream_t st)
 {
-    const int64_t nchunks = (int64_t)((nx + 3) / 4) * ny;
-    int64_t b = (nchunks + kThreads * 8 - 1) / (kThreads * 8);
-    int nblocks = (int)(b < 1 ? 1 : (b > OBS_MAX_BLOCKS ? OBS_MAX_BLOCKS : b));
+    const int nblocks = reduce_blocks((int64_t)((nx + 3) / 4) * ny, f64);
     if (f64) {
+        const double *r = (const double *)re, *m = (const double *)im, *v = (const double *)vplane;
         if (norm_only)
-            launch_pdl(observe_kernel<double, true>, nblocks, kThreads, 0, st, (const double *)re, (const double *)im, (const double *)vplane, nx, ny, pitch, J, partials);
+            launch_pdl(observe_kernel<double, true, false>, nblocks, kThreads, 0, st, r, m, v, nx,
+                       ny, 1, pitch, partials);
         else
-            launch_pdl(observe_kernel<double, false>, nblocks, kThreads, 0, st, (const double *)re, (const double *)im, (const double *)vplane, nx, ny, pitch, J, partials);
+            launch_pdl(observe_kernel<double, false, false>, nblocks, kThreads, 0, st, r, m, v, nx,
+                       ny, 1, pitch, partials);
     } else {
-        const float J_hi = (float)J, J_lo = (float)(J - (double)J_hi);
+        const float *r = (const float *)re, *m = (const float *)im, *v = (const float *)vplane;
         if (norm_only)
-            launch_pdl(observe_f32_kernel<true>, nblocks, kThreads, 0, st, (const float *)re, (const float *)im, (const float *)vplane, nx, ny, pitch, J_hi, J_lo, partials);
+            launch_pdl(observe_f32_kernel<true>, nblocks, kThreads, 0, st, r, m, v, nx, ny, pitch,
+                       partials);
         else
-            launch_pdl(observe_f32_kernel<false>, nblocks, kThreads, 0, st, (const float *)re, (const float *)im, (const float *)vplane, nx, ny, pitch, J_hi, J_lo, partials);
+            launch_pdl(observe_f32_kernel<false>, nblocks, kThreads, 0, st, r, m, v, nx, ny, pitch,
+                       partials);
     }
-    launch_pdl(observe_finalize_kernel, 1, kThreads, 0, st, partials, nblocks, norm_only ? 1 : OBS_Q, OBS_Q,
-                                                    result);
+    launch_pdl(observe_finalize_kernel, 1, kThreads, 0, st, partials, nblocks,
+               norm_only ? 1 : OBS_Q, OBS_Q, -2.0 * J, result);
     count_launches(2);
     return cudaGetLastError();
 }
@@ -452,14 +350,15 @@ cudaError_t launch_observe3(const void *re, const void *im, const void *vplane, 
                             int ny, int nz, int64_t pitch, double J, double *partials,
                             double *result, cudaStream_t st)
 {
-    const int64_t nchunks = (int64_t)((nx + 3) / 4) * ny * nz;
-    int64_t b = (nchunks + kThreads * 8 - 1) / (kThreads * 8);
-    int nblocks = (int)(b < 1 ? 1 : (b > OBS_MAX_BLOCKS ? OBS_MAX_BLOCKS : b));
+    const int nblocks = reduce_blocks((int64_t)((nx + 3) / 4) * ny * nz, true);
     if (f64)
-        launch_pdl(observe3_kernel<double>, nblocks, kThreads, 0, st, (const double *)re, (const double *)im, (const double *)vplane, nx, ny, nz, pitch, J, partials);
+        launch_pdl(observe_kernel<double, false, true>, nblocks, kThreads, 0, st, (const double *)re,
+                   (const double *)im, (const double *)vplane, nx, ny, nz, pitch, partials);
     else
-        launch_pdl(observe3_kernel<float>, nblocks, kThreads, 0, st, (const float *)re, (const float *)im, (const float *)vplane, nx, ny, nz, pitch, J, partials);
-    launch_pdl(observe_finalize_kernel, 1, kThreads, 0, st, partials, nblocks, OBS_Q3, OBS_Q3, result);
+        launch_pdl(observe_kernel<float, false, true>, nblocks, kThreads, 0, st, (const float *)re,
+                   (const float *)im, (const float *)vplane, nx, ny, nz, pitch, partials);
+    launch_pdl(observe_finalize_kernel, 1, kThreads, 0, st, partials, nblocks, OBS_Q3, OBS_Q3,
+               -2.0 * J, result);
     count_launches(2);
     return cudaGetLastError();
 }
@@ -468,12 +367,11 @@ cudaError_t launch_inner(const float *phi_re, const float *phi_im, const float *
                          const float *psi_im, int nx, int ny, int64_t pitch, double *partials,
                          double *result, cudaStream_t st)
 {
-    const int64_t nchunks = (int64_t)((nx + 3) / 4) * ny;
-    int64_t b = (nchunks + kThreads * 8 - 1) / (kThreads * 8);
-    int nblocks = (int)(b < 1 ? 1 : (b > OBS_MAX_BLOCKS ? OBS_MAX_BLOCKS : b));
-    launch_pdl(inner_f32_kernel, nblocks, kThreads, 0, st, phi_re, phi_im, psi_re, psi_im, nx, ny, pitch,
-                                                   partials);
-    launch_pdl(observe_finalize_kernel, 1, kThreads, 0, st, partials, nblocks, 2, OBS_Q, result);
+    const int nblocks = reduce_blocks((int64_t)((nx + 3) / 4) * ny, false);
+    launch_pdl(inner_f32_kernel, nblocks, kThreads, 0, st, phi_re, phi_im, psi_re, psi_im, nx, ny,
+               pitch, partials);
+    launch_pdl(observe_finalize_kernel, 1, kThreads, 0, st, partials, nblocks, 2, OBS_Q, 1.0,
+               result);
     count_launches(2);
     return cudaGetLastError();
 }
