@@ -8,6 +8,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -55,6 +56,52 @@ size_t scratch_bytes()
            round_up(sizeof(ts::GridDesc), 256);
 }
 
+// Pinned slots that read-backs land in, one per grid that reads back.  Blocks of
+// 64 slots; a block whose slots have all been returned is freed, unless it is
+// the only one.
+constexpr size_t kSlotBytes = 512;
+constexpr int kBlockSlots = 64;
+struct SlotBlock {
+    unsigned char *base;
+    uint64_t used;
+};
+std::mutex g_slot_mu;
+std::vector<SlotBlock> g_slots;
+
+unsigned char *readback_get()   // nullptr if no pinned memory is to be had
+{
+    std::lock_guard<std::mutex> lk(g_slot_mu);
+    for (SlotBlock &b : g_slots)
+        for (int i = 0; i < kBlockSlots; ++i)
+            if (!(b.used >> i & 1)) {
+                b.used |= uint64_t(1) << i;
+                return b.base + i * kSlotBytes;
+            }
+    void *p = nullptr;
+    if (cudaHostAlloc(&p, kSlotBytes * kBlockSlots, cudaHostAllocPortable) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    g_slots.push_back({(unsigned char *)p, 1});
+    return (unsigned char *)p;
+}
+
+void readback_put(unsigned char *slot)
+{
+    if (!slot) return;
+    std::lock_guard<std::mutex> lk(g_slot_mu);
+    for (size_t k = 0; k < g_slots.size(); ++k) {
+        SlotBlock &b = g_slots[k];
+        if (slot < b.base || slot >= b.base + kSlotBytes * kBlockSlots) continue;
+        b.used &= ~(uint64_t(1) << (slot - b.base) / kSlotBytes);
+        if (b.used == 0 && g_slots.size() > 1) {
+            cudaFreeHost(b.base);
+            g_slots.erase(g_slots.begin() + (ptrdiff_t)k);
+        }
+        return;
+    }
+}
+
 }  // namespace
 
 namespace ts {
@@ -75,6 +122,7 @@ ts_status grid_setup(const ts_layout &L, void *slab, bool owns_slab, ts_grid **o
     scr += round_up(sizeof(double) * OBS_Q3, 256);
     g->err = (int *)scr;
     g->host_copied = nullptr;
+    g->readback = nullptr;
     scr += 256;
     g->desc_dev = (GridDesc *)scr;
     g->cur = 0;
@@ -419,6 +467,7 @@ ts_status ts_destroy_grid(ts_grid *g)
         if (e == cudaSuccess) e = f;
     }
     if (g->host_copied) cudaEventDestroy(g->host_copied);
+    readback_put(g->readback);
     delete g;
     if (e != cudaSuccess) return cuda_fail(e, "ts_destroy_grid: cudaFree");
     return TS_OK;
@@ -476,18 +525,31 @@ ts_status stage_in(ts_grid *g, const void *host, ts_dtype src_dtype, void *dst, 
     return TS_OK;
 }
 
-ts_status check_errword(ts_grid *g, cudaStream_t st)
+// Wait for the stream, and report what the kernels before reported.  With nq > 0
+// the first nq results of the reductions come back too: they lie beside the
+// error word, so it is one copy and one wait (into pinned memory: a copy into
+// pageable memory is staged and took 10 us more).
+ts_status read_back(ts_grid *g, cudaStream_t st, int nq = 0, double *res = nullptr)
 {
-    int h = 0;
-    cudaError_t e = cudaMemcpyAsync(&h, g->err, sizeof(int), cudaMemcpyDeviceToHost, st);
+    if (!g->readback) g->readback = readback_get();
+    unsigned char local[kSlotBytes];
+    unsigned char *h = g->readback ? g->readback : local;
+    const size_t off = (size_t)((unsigned char *)g->err - (unsigned char *)g->result);
+    const void *src = nq ? (const void *)g->result : (const void *)g->err;
+    const size_t word = nq ? off : 0;
+    cudaError_t e = cudaMemcpyAsync(h, src, word + sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(e, "kernel error (reported at sync)");
-    if (h != 0) {
+    if (nq) std::memcpy(res, h, sizeof(double) * (size_t)nq);
+    int bits;
+    std::memcpy(&bits, h + word, sizeof(int));
+    if (bits != 0) {
         cudaMemsetAsync(g->err, 0, sizeof(int), st);
         cudaStreamSynchronize(st);
-        if (h & ts::ERRBIT_WAIT_TIMEOUT)
-            return fail(TS_ERR_TIMEOUT, "a bounded wait in a fused kernel gave up (error word %d)", h);
-        return fail(TS_ERR_CUDA, "a kernel reported error word %d", h);
+        if (bits & ts::ERRBIT_WAIT_TIMEOUT)
+            return fail(TS_ERR_TIMEOUT, "a bounded wait in a fused kernel gave up (error word %d)",
+                        bits);
+        return fail(TS_ERR_CUDA, "a kernel reported error word %d", bits);
     }
     return TS_OK;
 }
@@ -505,9 +567,8 @@ ts_status ts_set_state(ts_grid *g, const void *re, const void *im, ts_dtype src_
     const bool sf = src_dtype == TS_F64;
     const int nx = (int)g->L.nx, ny = (int)g->rows();   // rows: all slabs
     if (where == TS_DEVICE) {
-        cudaError_t e = ts::launch_convert_in(re, sf, g->re(), g->f64(), nx, ny, g->L.pitch, st);
-        if (e == cudaSuccess)
-            e = ts::launch_convert_in(im, sf, g->im(), g->f64(), nx, ny, g->L.pitch, st);
+        cudaError_t e = ts::launch_convert_in2(re, im, sf, g->re(), g->im(), g->f64(), nx, ny,
+                                               g->L.pitch, st);
         if (e != cudaSuccess) return cuda_fail(e, "ts_set_state: convert kernel");
         return TS_OK;
     }
@@ -537,19 +598,14 @@ ts_status ts_get_state(ts_grid *g, void *re, void *im, ts_dtype dst_dtype, ts_me
     if (dst_dtype != TS_F32 && dst_dtype != TS_F64)
         return fail(TS_ERR_ARG, "ts_get_state: unknown dtype");
     cudaStream_t st = (cudaStream_t)stream;
-    ts_status s = check_errword(g, st);
-    if (s != TS_OK) return s;
     const bool df = dst_dtype == TS_F64;
     const int nx = (int)g->L.nx, ny = (int)g->rows();   // rows: all slabs
     const size_t n = (size_t)nx * ny;
     cudaError_t e;
     if (where == TS_DEVICE) {
-        e = ts::launch_convert_out(g->re(), g->f64(), re, df, nx, ny, g->L.pitch, st);
-        if (e == cudaSuccess)
-            e = ts::launch_convert_out(g->im(), g->f64(), im, df, nx, ny, g->L.pitch, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        e = ts::launch_convert_out2(g->re(), g->im(), g->f64(), re, im, df, nx, ny, g->L.pitch, st);
         if (e != cudaSuccess) return cuda_fail(e, "ts_get_state");
-        return TS_OK;
+        return read_back(g, st);
     }
     if (where != TS_HOST) return fail(TS_ERR_ARG, "ts_get_state: unknown memory kind");
     if (df == g->f64()) {
@@ -559,9 +615,8 @@ ts_status ts_get_state(ts_grid *g, void *re, void *im, ts_dtype dst_dtype, ts_me
         if (e == cudaSuccess)
             e = cudaMemcpy2DAsync(im, nx * es, g->im(), g->L.pitch * es, nx * es, ny,
                                   cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) return cuda_fail(e, "ts_get_state: device-to-host copy");
-        return TS_OK;
+        return read_back(g, st);
     }
     // convert on the device into the staging region, then copy out
     const size_t es = df ? 8 : 4;
@@ -572,10 +627,9 @@ ts_status ts_get_state(ts_grid *g, void *re, void *im, ts_dtype dst_dtype, ts_me
         e = ts::launch_convert_out(srcs[c], g->f64(), stage, df, nx, ny, g->L.pitch, st);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(dsts[c], stage, n * es, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) return cuda_fail(e, "ts_get_state");
     }
-    return TS_OK;
+    return read_back(g, st);
 }
 
 ts_status ts_set_potential(ts_grid *g, const double *V, ts_mem where, double dt, double theta,
@@ -1285,9 +1339,7 @@ ts_status observe(ts_grid *g, bool norm_only, double *res, cudaStream_t st)
                                g->result, st);
     }
     if (e != cudaSuccess) return cuda_fail(e, "observables kernel");
-    e = cudaMemcpyAsync(res, g->result, sizeof(double) * nq, cudaMemcpyDeviceToHost, st);
-    if (e != cudaSuccess) return cuda_fail(e, "observables copy");
-    return check_errword(g, st);
+    return read_back(g, st, norm_only ? 1 : nq, res);
 }
 
 }  // namespace

@@ -62,12 +62,16 @@ __device__ __forceinline__ void store4(T *p, const T (&v)[4])
     }
 }
 
-// IN: dense src -> pitched dst; otherwise pitched src -> dense dst
+// IN: dense src -> pitched dst; otherwise pitched src -> dense dst.  A launch
+// takes one array or two (gridDim.z).
 template <bool IN, typename Ts, typename Td>
-__global__ void convert_kernel(const Ts *__restrict__ src, Td *__restrict__ dst, int nx, int ny,
+__global__ void convert_kernel(const Ts *__restrict__ src0, Td *__restrict__ dst0,
+                               const Ts *__restrict__ src1, Td *__restrict__ dst1, int nx, int ny,
                                int64_t pitch, bool vec4)
 {
     grid_dep_sync();
+    const Ts *src = blockIdx.z ? src1 : src0;
+    Td *dst = blockIdx.z ? dst1 : dst0;
     for (int64_t y = blockIdx.y; y < ny; y += gridDim.y) {
         const Ts *s = src + y * (IN ? (int64_t)nx : pitch);
         Td *d = dst + y * (IN ? pitch : (int64_t)nx);
@@ -342,19 +346,29 @@ inline dim3 grid2d(int64_t per_row, int rows)
 }  // namespace
 
 template <bool IN>
-cudaError_t launch_convert(const void *src, bool src_f64, void *dst, bool dst_f64, int nx, int ny,
-                           int64_t pitch, cudaStream_t st)
+cudaError_t launch_convert(const void *src0, const void *src1, bool src_f64, void *dst0,
+                           void *dst1, bool dst_f64, int nx, int ny, int64_t pitch,
+                           cudaStream_t st)
 {
-    const bool vec4 = (nx % 4) == 0 && ((uintptr_t)src % 16) == 0 && ((uintptr_t)dst % 16) == 0;
+    auto aligned = [](const void *q) { return ((uintptr_t)q % 16) == 0; };
+    const bool vec4 = (nx % 4) == 0 && aligned(src0) && aligned(dst0) &&
+                      (!dst1 || (aligned(src1) && aligned(dst1)));
     dim3 grid = grid2d(vec4 ? nx / 4 : nx, ny);
+    grid.z = dst1 ? 2 : 1;
+    auto run = [&](auto s, auto d) {
+        using Ts = decltype(s);
+        using Td = decltype(d);
+        launch_pdl(convert_kernel<IN, Ts, Td>, grid, kThreads, 0, st, (const Ts *)src0, (Td *)dst0,
+                   (const Ts *)src1, (Td *)dst1, nx, ny, pitch, vec4);
+    };
     if (src_f64 && dst_f64)
-        launch_pdl(convert_kernel<IN, double, double>, grid, kThreads, 0, st, (const double *)src, (double *)dst, nx, ny, pitch, vec4);
+        run(double(), double());
     else if (src_f64)
-        launch_pdl(convert_kernel<IN, double, float>, grid, kThreads, 0, st, (const double *)src, (float *)dst, nx, ny, pitch, vec4);
+        run(double(), float());
     else if (dst_f64)
-        launch_pdl(convert_kernel<IN, float, double>, grid, kThreads, 0, st, (const float *)src, (double *)dst, nx, ny, pitch, vec4);
+        run(float(), double());
     else
-        launch_pdl(convert_kernel<IN, float, float>, grid, kThreads, 0, st, (const float *)src, (float *)dst, nx, ny, pitch, vec4);
+        run(float(), float());
     count_launches(1);
     return cudaGetLastError();
 }
@@ -362,13 +376,27 @@ cudaError_t launch_convert(const void *src, bool src_f64, void *dst, bool dst_f6
 cudaError_t launch_convert_in(const void *src, bool src_f64, void *dst, bool dst_f64, int nx,
                               int ny, int64_t pitch, cudaStream_t st)
 {
-    return launch_convert<true>(src, src_f64, dst, dst_f64, nx, ny, pitch, st);
+    return launch_convert<true>(src, nullptr, src_f64, dst, nullptr, dst_f64, nx, ny, pitch, st);
 }
 
 cudaError_t launch_convert_out(const void *src, bool src_f64, void *dst, bool dst_f64, int nx,
                                int ny, int64_t pitch, cudaStream_t st)
 {
-    return launch_convert<false>(src, src_f64, dst, dst_f64, nx, ny, pitch, st);
+    return launch_convert<false>(src, nullptr, src_f64, dst, nullptr, dst_f64, nx, ny, pitch, st);
+}
+
+cudaError_t launch_convert_in2(const void *src0, const void *src1, bool src_f64, void *dst0,
+                               void *dst1, bool dst_f64, int nx, int ny, int64_t pitch,
+                               cudaStream_t st)
+{
+    return launch_convert<true>(src0, src1, src_f64, dst0, dst1, dst_f64, nx, ny, pitch, st);
+}
+
+cudaError_t launch_convert_out2(const void *src0, const void *src1, bool src_f64, void *dst0,
+                                void *dst1, bool dst_f64, int nx, int ny, int64_t pitch,
+                                cudaStream_t st)
+{
+    return launch_convert<false>(src0, src1, src_f64, dst0, dst1, dst_f64, nx, ny, pitch, st);
 }
 
 cudaError_t launch_phase_table(const double *V, void *pg, void *ps, void *vplane, bool f64, int nx,
