@@ -40,7 +40,7 @@
 // Work split: a persistent launch gives each strip the same number of warps,
 // each on one row range, the same ranges in every strip, so that warps of
 // neighbouring strips walk the same rows together and share their halo
-// columns through L2 (min_pairs_per_warp sets how short a range may be).  The
+// columns through L2 (strip_warps_for chooses how many).  The
 // multi-grid kernel picks between that split and an even split of all its
 // grids' (strip, row-pair) units (fused_multi_plan).
 //
@@ -120,29 +120,20 @@ namespace {
 #ifndef TS_FUSED_SC_MIN_BLOCKS_K4     // ... and with scaled rotations: 168 registers
 #define TS_FUSED_SC_MIN_BLOCKS_K4 12
 #endif
+#ifndef TS_FUSED_SC_MULTI_MIN_BLOCKS  // multi-grid kernel with scaled rotations, K = 3 and 4
+#define TS_FUSED_SC_MULTI_MIN_BLOCKS 12
+#endif
 #ifndef TS_FUSED_MULTI_MIN_BLOCKS_K3   // multi-grid kernel, K = 3
 #define TS_FUSED_MULTI_MIN_BLOCKS_K3 1
 #endif
 #ifndef TS_FUSED_MULTI_MIN_BLOCKS_K4   // multi-grid kernel, K = 4
 #define TS_FUSED_MULTI_MIN_BLOCKS_K4 1
 #endif
-#ifndef TS_FUSED_MIN_PAIRS       // row pairs per warp: at least this many ...
-#define TS_FUSED_MIN_PAIRS 4
-#endif
-#ifndef TS_FUSED_MAX_MIN_PAIRS   // ... and at most this many as the floor
-#define TS_FUSED_MAX_MIN_PAIRS 16
-#endif
-#ifndef TS_FUSED_FILL_WARPS_PER_SM   // warps per SM that keep HBM busy
-#define TS_FUSED_FILL_WARPS_PER_SM 8
-#endif
 #ifndef TS_FUSED_PINGPONG_MIN_K  // interior row pairs alternate two carry sets for K in
 #define TS_FUSED_PINGPONG_MIN_K 3    // [MIN_K, MAX_K] (beyond MAX_K the second set spills)
 #endif
 #ifndef TS_FUSED_PINGPONG_MAX_K
 #define TS_FUSED_PINGPONG_MAX_K 6
-#endif
-#ifndef TS_FUSED_ALIGNED         // 1: strip-aligned work split when strips <= warps
-#define TS_FUSED_ALIGNED 1
 #endif
 #ifndef TS_FUSED_FFMA2           // packed FP32 FMAs (__ffma2_rn): see Cfg<K>::PACKED
 #define TS_FUSED_FFMA2 1
@@ -193,10 +184,10 @@ __host__ __device__ constexpr int min_blocks(int K, int MODE, bool SC)
 }
 
 // ... and of the multi-grid kernel
-__host__ __device__ constexpr int multi_min_blocks(int K)
+__host__ __device__ constexpr int multi_min_blocks(int K, bool SC)
 {
-    return K == 3   ? TS_FUSED_MULTI_MIN_BLOCKS_K3
-           : K == 4 ? TS_FUSED_MULTI_MIN_BLOCKS_K4
+    return K == 3   ? (SC ? TS_FUSED_SC_MULTI_MIN_BLOCKS : TS_FUSED_MULTI_MIN_BLOCKS_K3)
+           : K == 4 ? (SC ? TS_FUSED_SC_MULTI_MIN_BLOCKS : TS_FUSED_MULTI_MIN_BLOCKS_K4)
                     : TS_FUSED_MIN_BLOCKS;
 }
 
@@ -716,8 +707,9 @@ __device__ __forceinline__ float4 neg4(float4 v) { return make_float4(-v.x, -v.y
 // -theta; the phase is conjugated here) that accumulate G at each step's
 // phase point, with the running sums of the rows in flight in shared memory
 // (updated in place).
-// SC: scaled rotations (see pair_s); INTERIOR then also means that none of the
-// strip's columns lies on an edge of the grid.  The rows leave scaled.
+// SC: scaled rotations (see pair_s); the rows leave scaled.  MODE 7 is MODE 0 of
+// the multi-grid kernel, whose coefficients are no kernel parameters: it reads
+// them from shared memory at each sweep, which keeps 16 registers free.
 template <int K, bool INTERIOR, int MODE, bool SC, typename S = StateT<MODE>>
 __device__ __forceinline__ void pipeline_step(const S (&cin)[2 * K], S (&cout)[2 * K],
                                               S a, S b, int yin, int j,
@@ -769,7 +761,9 @@ __device__ __forceinline__ void pipeline_step(const S (&cin)[2 * K], S (&cout)[2
     };
     // Y sweeps of the rows (y, y + 1)
     auto YE = [&](S &f0, S &f1, int y, int k) {
-        if constexpr (SC) {
+        if constexpr (SC && INTERIOR && MODE == 7) {
+            y_pair_bulk(f0, f1, et->bulk[k]);
+        } else if constexpr (SC) {
             float ta = te(k), tb = ta;
             if constexpr (!INTERIOR) {
                 const float2 lh = et->lohi[k];
@@ -784,7 +778,9 @@ __device__ __forceinline__ void pipeline_step(const S (&cin)[2 * K], S (&cout)[2
         }
     };
     auto YO = [&](S &f0, S &f1, int y, int m) {
-        if constexpr (SC) {
+        if constexpr (SC && INTERIOR && MODE == 7) {
+            y_pair_bulk(f0, f1, et->bulk[K + 1 + m]);
+        } else if constexpr (SC) {
             float ta = to(m), tb = ta;
             if constexpr (!INTERIOR) {
                 const float2 lh = et->lohi[K + 1 + m];
@@ -1409,21 +1405,22 @@ __device__ __forceinline__ bool run_segment(WarpRings &r, const CUtensorMap *tm_
         for (int i = 0; i < 3 * K + 1; ++i) {
             const float2 lh = et->lohi[i];
             float4 c;
-            float other;
+            float other, t;
             if (i < NE) {
-                const float t = MODE == 4 && (i == 2 || i == 3) ? p.te_ab
+                t = MODE == 4 && (i == 2 || i == 3) ? p.te_ab
                                 : i == 0 || i == K              ? p.te_end
                                                                 : p.te_mid;
                 pair_coef(pair_kind(xg, p.nx), t, lh.x, lh.y, c.x, c.y);
                 pair_coef(pair_kind(xg + 2, p.nx), t, lh.x, lh.y, c.z, c.w);
             } else {
                 const int m = i - NE;
-                const float t = MODE == 4 && m / 2 == 2 ? p.to_sub : (m & 1) ? p.to_b : p.to_a;
+                t = MODE == 4 && m / 2 == 2 ? p.to_sub : (m & 1) ? p.to_b : p.to_a;
                 pair_coef(pair_kind(xg + 1, p.nx), t, lh.x, lh.y, c.y, c.z);
                 pair_coef(pair_kind(xg + 3, p.nx), t, lh.x, lh.y, c.w, other);
                 pair_coef(pair_kind(xg - 1, p.nx), t, lh.x, lh.y, other, c.x);
             }
             et->recv[i][cls] = c;
+            if constexpr (MODE == 7) et->bulk[i] = make_float4(-t, -t, t, t);
         }
         __syncwarp();
     }
@@ -1638,13 +1635,16 @@ __device__ __forceinline__ void multi_params(KParams &p, const GridDesc *d, int 
 }
 
 template <int K, bool SC>
-__global__ void __launch_bounds__(Cfg<K>::WPC * 32, multi_min_blocks(K))
+__global__ void __launch_bounds__(Cfg<K>::WPC * 32, multi_min_blocks(K, SC))
 fused_multi_kernel(const EpochEntry *__restrict__ tab, int n_grids, int64_t total_units,
                    int total_warps, int aligned, int flip, int *err)
 {
     using C = CfgM<K, 0, SC>;
     extern __shared__ unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // the grid's parameters, per warp: in shared memory, not in registers
+    __shared__ KParams params[C::WPC];
+    KParams &p = params[warp];
     const int gw = blockIdx.x * C::WPC + warp;
     if (gw >= total_warps) return;
     WarpRings r = carve_rings<K, 0, SC>(smem_raw, warp, lane);
@@ -1665,16 +1665,15 @@ fused_multi_kernel(const EpochEntry *__restrict__ tab, int n_grids, int64_t tota
         if (lane == 0) {
             tensormap_acquire(&d->tm_state[cur]);
             tensormap_acquire(&d->tm_phase);
+            multi_params<K, SC>(p, d, cur, err);
         }
         __syncwarp();
-        KParams p;
-        multi_params<K, SC>(p, d, cur, err);
         const int w = e.strip_warps, l = gw - (int)e.begin;
         const int sx = l / w, i = l - sx * w;
         const int q0 = (int)((int64_t)i * p.n_pairs / w);
         const int q1 = (int)((int64_t)(i + 1) * p.n_pairs / w);
         if (q1 > q0)
-            run_segment<K, 0, SC>(r, &d->tm_state[cur], &d->tm_phase, nullptr, p, sx, q0, q1, lane);
+            run_segment<K, SC ? 7 : 0, SC>(r, &d->tm_state[cur], &d->tm_phase, nullptr, p, sx, q0, q1, lane);
         return;
     }
     const int64_t u_begin = (int64_t)gw * total_units / total_warps;
@@ -1686,15 +1685,15 @@ fused_multi_kernel(const EpochEntry *__restrict__ tab, int n_grids, int64_t tota
         const GridDesc *d = e.desc;
         const int cur = e.cur0 ^ flip;
         if (fenced != gi) {
+            __syncwarp();   // every lane is done with the grid before
             if (lane == 0) {
                 tensormap_acquire(&d->tm_state[cur]);
                 tensormap_acquire(&d->tm_phase);
+                multi_params<K, SC>(p, d, cur, err);
             }
             __syncwarp();
             fenced = gi;
         }
-        KParams p;
-        multi_params<K, SC>(p, d, cur, err);
         const int64_t local = u - e.begin;
         const int64_t g_units = (gi + 1 < n_grids ? tab[gi + 1].begin : total_units) - e.begin;
         const int sx = (int)(local / p.n_pairs);
@@ -1704,21 +1703,44 @@ fused_multi_kernel(const EpochEntry *__restrict__ tab, int n_grids, int64_t tota
         if (q1_want > q0 + left_in_grid) q1_want = q0 + left_in_grid;
         const int q1 = (int)(q1_want < p.n_pairs ? q1_want : (int64_t)p.n_pairs);
         u += q1 - q0;
-        if (!run_segment<K, 0, SC>(r, &d->tm_state[cur], &d->tm_phase, nullptr, p, sx, q0, q1, lane)) return;
+        if (!run_segment<K, SC ? 7 : 0, SC>(r, &d->tm_state[cur], &d->tm_phase, nullptr, p, sx, q0, q1, lane)) return;
     }
 }
 
-// Fewest row pairs a warp takes.  Each warp runs a chain of dependent
-// iterations, and each of its segments first fills a pipeline of 2K row
-// pairs.  On small grids the chains set the launch time, so many warps with
-// short ranges win (down to TS_FUSED_MIN_PAIRS).  Once a grid has enough
-// work for TS_FUSED_FILL_WARPS_PER_SM warps per SM at that length, more
-// warps only add fills, so the floor grows with the work (up to
-// TS_FUSED_MAX_MIN_PAIRS).
-inline int64_t min_pairs_per_warp(int64_t units, int num_sms)
+// What a row pair costs a warp that shares its scheduler with n - 1 others,
+// relative: 1.06, 1.27 and 1.6 us at depth 4 for n = 1, 2, 3 (512^2 with 96
+// warps, 2048^2 with 1216, 8192^2 with 1776).
+inline double pair_cost(int64_t warps, int num_sms)
 {
-    const int64_t by_work = units / ((int64_t)TS_FUSED_FILL_WARPS_PER_SM * num_sms);
-    return std::min<int64_t>(TS_FUSED_MAX_MIN_PAIRS, std::max<int64_t>(TS_FUSED_MIN_PAIRS, by_work));
+    const int64_t n = (warps + 4 * num_sms - 1) / (4 * num_sms);
+    return 0.62 + 0.36 * (double)n;
+}
+
+// Warps per strip.  A warp's row range of q row pairs takes q + 2K iterations
+// (the pipeline fills over 2K), so few long ranges save fills and many short
+// ones shorten the chain; the schedulers should get equal numbers of warps.
+// Take the least (q + 2K) pair_cost over whole numbers of warps per scheduler.
+// (A floor of units / (8 SMs) row pairs, before, gave 2013 x 1986 1278 warps, 3
+// on some schedulers and 2 on the others: 38.6 us per launch of depth 4,
+// against 32.0 at 2048^2.)
+inline int64_t strip_warps_for(int64_t strips, int64_t pairs, int K, int64_t cap, int num_sms)
+{
+    int64_t best = 0;
+    double best_cost = 0.0;
+    const int64_t per = 4 * (int64_t)num_sms;
+    for (int64_t total = per;; total += per) {
+        const int64_t w = std::min(std::min(total, cap) / strips, pairs);
+        if (w >= 1) {
+            const double q = (double)((pairs + w - 1) / w);
+            const double cost = (q + 2.0 * K) * pair_cost(w * strips, num_sms);
+            if (best == 0 || cost < best_cost) {
+                best = w;
+                best_cost = cost;
+            }
+        }
+        if (total >= cap) break;
+    }
+    return best;
 }
 
 #if TS_FUSED_PART != 0
@@ -1829,19 +1851,12 @@ cudaError_t launch_k(const FusedLaunch &a, cudaStream_t st)
     p.n_strips = (a.nx + C::VALID - 1) / C::VALID;
     p.n_pairs = (a.ny + 1) / 2;
     p.units = (int64_t)p.n_strips * p.n_pairs;
-    // at most the resident warps, each with at least min_pairs_per_warp row pairs
-    const int64_t mp = min_pairs_per_warp(p.units, num_sms);
-    int64_t want = (p.units + mp - 1) / mp;
-    int64_t cap = (int64_t)num_sms * blocks_per_sm * C::WPC;
-    p.total_warps = (int)(want < cap ? (want < 1 ? 1 : want) : cap);
+    const int64_t cap = (int64_t)num_sms * blocks_per_sm * C::WPC;
+    p.total_warps = (int)std::min(p.units, cap);
     p.strip_warps = 0;
-    if (TS_FUSED_ALIGNED && p.n_strips <= cap) {
-        int64_t w = cap / p.n_strips;
-        const int64_t rows_cap = (p.n_pairs + mp - 1) / mp;
-        if (w > rows_cap) w = rows_cap;
-        if (w < 1) w = 1;
-        p.strip_warps = (int)w;
-        p.total_warps = (int)(w * p.n_strips);
+    if (p.n_strips <= cap) {
+        p.strip_warps = (int)strip_warps_for(p.n_strips, p.n_pairs, K, cap, num_sms);
+        p.total_warps = p.strip_warps * p.n_strips;
     }
     p.t1 = a.t1;
     p.s1 = a.s1;
@@ -2079,32 +2094,47 @@ MultiPlan fused_multi_plan(int K, bool scaled, int n, const int *nx, const int *
         units += strips[(size_t)i] * pairs[(size_t)i];
         all_strips += strips[(size_t)i];
     }
-    // even split: at most the resident warps, each with at least
-    // min_pairs_per_warp row pairs
-    const int64_t mp = min_pairs_per_warp(units, num_sms);
-    const int64_t lin_warps = std::min(cap, std::max<int64_t>(1, (units + mp - 1) / mp));
-    const int64_t lin_span = (units + lin_warps - 1) / lin_warps;
+    // even split: the warps that cost least (as in strip_warps_for; a range that
+    // crosses from one strip into the next fills twice, which 2K per range and
+    // strip counts on average)
+    const int64_t per = 4 * (int64_t)num_sms;
+    int64_t lin_warps = 0;
+    double lin_cost = 0.0;
+    for (int64_t total = per;; total += per) {
+        const int64_t w = std::min(std::min(total, cap), units);
+        const double q = (double)((units + w - 1) / w);
+        const double cost = (q + 2.0 * K * (1.0 + (double)all_strips / (double)w)) *
+                            pair_cost(w, num_sms);
+        if (lin_warps == 0 || cost < lin_cost) {
+            lin_warps = w;
+            lin_cost = cost;
+        }
+        if (total >= cap || w == units) break;
+    }
     // aligned split: one warp per strip to start with, then more warps (on
     // every strip of a grid at once) to the grid with the most row pairs per
-    // warp while they fit; it is taken when its longest warp is within 10 %
-    // of the even split's
-    int64_t al_warps = all_strips, al_span = 0;
+    // warp while they fit the warps of the even split's count or the next full
+    // one; it is taken when it costs no more than 1.1 times the even split
+    int64_t al_warps = all_strips;
+    double al_cost = 0.0;
     if (all_strips <= cap) {
+        const int64_t most = std::min(cap, std::max((all_strips + per - 1) / per * per, lin_warps));
         auto work = [&](int i) { return (pairs[(size_t)i] + w[(size_t)i] - 1) / w[(size_t)i]; };
         std::priority_queue<std::pair<int64_t, int>> heap;
         for (int i = 0; i < n; ++i) heap.push({work(i), i});
         while (!heap.empty()) {
             const int i = heap.top().second;
-            if (al_warps + strips[(size_t)i] > cap || pairs[(size_t)i] / (w[(size_t)i] + 1) < mp)
-                break;
+            if (al_warps + strips[(size_t)i] > most || w[(size_t)i] >= pairs[(size_t)i]) break;
             heap.pop();
             ++w[(size_t)i];
             al_warps += strips[(size_t)i];
             heap.push({work(i), i});
         }
-        for (int i = 0; i < n; ++i) al_span = std::max(al_span, work(i));
+        int64_t span = 0;
+        for (int i = 0; i < n; ++i) span = std::max(span, work(i));
+        al_cost = ((double)span + 2.0 * K) * pair_cost(al_warps, num_sms);
     }
-    plan.aligned = all_strips <= cap && al_span * 10 <= lin_span * 11;
+    plan.aligned = all_strips <= cap && al_cost <= 1.1 * lin_cost;
     plan.units = units;
     int64_t begin = 0;
     for (int i = 0; i < n; ++i) {

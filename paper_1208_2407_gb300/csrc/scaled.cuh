@@ -26,6 +26,7 @@ template <int K, bool ADJ>
 struct EdgeTab {
     static constexpr int SWEEPS = 3 * K + 1, CLASSES = 8;
     float4 recv[SWEEPS][CLASSES];
+    float4 bulk[SWEEPS];        // (-t, -t, t, t) of the sweep's bulk pairs
     float4 hrow[2][CLASSES];    // h and f of the columns of a lane, bulk rows
     float4 frow[ADJ ? K : 1][CLASSES];
     float2 lohi[SWEEPS];
@@ -167,6 +168,27 @@ __device__ __forceinline__ void y_pair_s(Frag &a, Frag &b, float ta, float tb)
         pair_s(a.re.z, a.im.z, b.re.z, b.im.z, ta, tb);
         pair_s(a.re.w, a.im.w, b.re.w, b.im.w, ta, tb);
     }
+}
+
+// The same for a bulk pair with t = (-t, -t, t, t), packed.
+__device__ __forceinline__ void y_pair_bulk(Frag &a, Frag &b, float4 t)
+{
+    const float2 n = make_float2(t.x, t.y), p = make_float2(t.z, t.w);
+    auto half = [&](float2 &ar, float2 &ai, float2 &br, float2 &bi) {
+        const float2 r = ar, m = ai;
+        ar = __ffma2_rn(n, bi, ar);
+        ai = __ffma2_rn(p, br, ai);
+        br = __ffma2_rn(n, m, br);
+        bi = __ffma2_rn(p, r, bi);
+    };
+    float2 ar = lo2(a.re), ai = lo2(a.im), br = lo2(b.re), bi = lo2(b.im);
+    float2 cr = hi2(a.re), ci = hi2(a.im), dr = hi2(b.re), di = hi2(b.im);
+    half(ar, ai, br, bi);
+    half(cr, ci, dr, di);
+    a.re = join2(ar, cr);
+    a.im = join2(ai, ci);
+    b.re = join2(br, dr);
+    b.im = join2(bi, di);
 }
 
 // a -= h a, h per column
