@@ -1851,7 +1851,14 @@ cudaError_t launch_k(const FusedLaunch &a, cudaStream_t st)
     p.n_strips = (a.nx + C::VALID - 1) / C::VALID;
     p.n_pairs = (a.ny + 1) / 2;
     p.units = (int64_t)p.n_strips * p.n_pairs;
-    const int64_t cap = (int64_t)num_sms * blocks_per_sm * C::WPC;
+    int64_t cap = (int64_t)num_sms * blocks_per_sm * C::WPC;
+    // Depths 1 and 2 wait for HBM, and with every warp in flight neighbouring
+    // strips drift apart: the halo columns they share leave L2 before the second
+    // strip reads them.  On grids larger than L2 (24 B per site) fewer warps keep
+    // pace (8192^2, depth 1: 290 us with 8 warps per SM, 272 with 4; depth 2: 281
+    // with 8, 264 with 7).
+    if (SC && MODE == 0 && K <= 2 && 24.0 * a.nx * a.ny > 128e6)
+        cap = std::min<int64_t>(cap, (int64_t)num_sms * (K == 1 ? 4 : 7));
     p.total_warps = (int)std::min(p.units, cap);
     p.strip_warps = 0;
     if (p.n_strips <= cap) {
