@@ -244,7 +244,7 @@ struct Cfg {
     // four planes, [row][plane][lane] as float4)
     static constexpr int GST_BYTES = M == 5 ? 4096 : 0;
     // scaled rotations: the warp's edge values (EdgeTab)
-    static constexpr int EDGE_BYTES = SC ? (sizeof(EdgeTab<K, M == 5>) + 127) / 128 * 128 : 0;
+    static constexpr int EDGE_BYTES = SC ? (sizeof(EdgeTab<K, M>) + 127) / 128 * 128 : 0;
     static constexpr int WARP_SMEM = NSS * SSLOT + NSP * PSLOT + NSB * SLOT_BYTES + SUMS_BYTES +
                                      GST_BYTES + EDGE_BYTES;
     static constexpr int SMEM = 1024 + WPC * (WARP_SMEM + NBAR * 8);
@@ -253,6 +253,10 @@ struct Cfg {
 // The configuration of a mode's kernel at depth K.
 template <int K, int MODE, bool SC>
 using CfgM = Cfg<K, phase_planes(MODE), MODE == 4, state_planes(MODE), MODE, SC>;
+
+// The multi-grid kernel's mode.
+template <bool SC>
+constexpr int MULTI_MODE = SC ? 7 : 0;
 
 // The same columns of two states that take the same factors: the forward
 // state psi (a) and the costate lambda (b) of a backward adjoint step, or
@@ -571,17 +575,21 @@ __device__ __forceinline__ bool owns_row(const Owned &w, const KParams &p, int r
 // Adjoint hooks.  At the phase point of a backward step the lane's rows of
 // the costate, lt = B^dagger lambda_s, meet the mid-step state of the same
 // step, m = B^dagger psi_s: the term conj(lt) m = (lr mr + li mi) + i (lr mi - li mr).
+// Packed, two columns per instruction (the kernel is bound by issue up to 2048^2).
 __device__ __forceinline__ Frag adj_term(const Frag &lt, const Frag &m)
 {
+    auto neg = [](float2 v) { return make_float2(-v.x, -v.y); };
+    auto re = [](float2 lr, float2 li, float2 mr, float2 mi) {
+        return __ffma2_rn(lr, mr, __fmul2_rn(li, mi));
+    };
+    auto im = [&](float2 lr, float2 li, float2 mr, float2 mi) {
+        return __ffma2_rn(lr, mi, __fmul2_rn(neg(li), mr));
+    };
     Frag t;
-    t.re = make_float4(fmaf(lt.re.x, m.re.x, lt.im.x * m.im.x),
-                       fmaf(lt.re.y, m.re.y, lt.im.y * m.im.y),
-                       fmaf(lt.re.z, m.re.z, lt.im.z * m.im.z),
-                       fmaf(lt.re.w, m.re.w, lt.im.w * m.im.w));
-    t.im = make_float4(fmaf(lt.re.x, m.im.x, -lt.im.x * m.re.x),
-                       fmaf(lt.re.y, m.im.y, -lt.im.y * m.re.y),
-                       fmaf(lt.re.z, m.im.z, -lt.im.z * m.re.z),
-                       fmaf(lt.re.w, m.im.w, -lt.im.w * m.re.w));
+    t.re = join2(re(lo2(lt.re), lo2(lt.im), lo2(m.re), lo2(m.im)),
+                 re(hi2(lt.re), hi2(lt.im), hi2(m.re), hi2(m.im)));
+    t.im = join2(im(lo2(lt.re), lo2(lt.im), lo2(m.re), lo2(m.im)),
+                 im(hi2(lt.re), hi2(lt.im), hi2(m.re), hi2(m.im)));
     return t;
 }
 
@@ -589,10 +597,8 @@ __device__ __forceinline__ Frag adj_term(const Frag &lt, const Frag &m)
 __device__ __forceinline__ Frag frag_fma(const Frag &a, float4 f, const Frag &b)
 {
     Frag r;
-    r.re = make_float4(fmaf(f.x, b.re.x, a.re.x), fmaf(f.y, b.re.y, a.re.y),
-                       fmaf(f.z, b.re.z, a.re.z), fmaf(f.w, b.re.w, a.re.w));
-    r.im = make_float4(fmaf(f.x, b.im.x, a.im.x), fmaf(f.y, b.im.y, a.im.y),
-                       fmaf(f.z, b.im.z, a.im.z), fmaf(f.w, b.im.w, a.im.w));
+    r.re = join2(__ffma2_rn(lo2(f), lo2(b.re), lo2(a.re)), __ffma2_rn(hi2(f), hi2(b.re), hi2(a.re)));
+    r.im = join2(__ffma2_rn(lo2(f), lo2(b.im), lo2(a.im)), __ffma2_rn(hi2(f), hi2(b.im), hi2(a.im)));
     return r;
 }
 
@@ -742,7 +748,7 @@ __device__ __forceinline__ void pipeline_step(const S (&cin)[2 * K], S (&cout)[2
     auto mixed = [&](int k) { return k > 0 && k < K && is_b(k - 1) != is_b(k); };
     auto te = [&](int k) { return mixed(k) ? p.te_ab : k == 0 || k == K ? p.te_end : p.te_mid; };
     auto to = [&](int m) { return is_b(m / 2) ? p.to_sub : (m & 1) ? p.to_b : p.to_a; };
-    const EdgeTab<K, MODE == 5> *et = reinterpret_cast<const EdgeTab<K, MODE == 5> *>(w.edge);
+    const EdgeTab<K, MODE> *et = reinterpret_cast<const EdgeTab<K, MODE> *>(w.edge);
     auto XE = [&](S &f, int k) {
         if constexpr (SC) {
             const float4 r = et->recv[k][w.lane_class];
@@ -1027,7 +1033,7 @@ __device__ __forceinline__ void z_even(Frag2 &r0, Frag2 &r1, const Seg &s, const
 {
     if constexpr (SC) {
         float ta, tb;
-        const float2 lh = reinterpret_cast<const EdgeTab<1, false> *>(s.own.edge)->lohi[k];
+        const float2 lh = reinterpret_cast<const EdgeTab<1, 6> *>(s.own.edge)->lohi[k];
         pair_coef(pair_kind(s.z, p.nz), p.te_end, lh.x, lh.y, ta, tb);
         y_pair_s<PACKED>(r0.a, r0.b, ta, tb);
         y_pair_s<PACKED>(r1.a, r1.b, ta, tb);
@@ -1070,7 +1076,7 @@ __device__ __forceinline__ bool z_odd(Frag2 &r0, Frag2 &r1, const Seg &s, const 
             f.im = join2(__ffma2_rn(u, lo2(qr), lo2(f.im)), __ffma2_rn(u, hi2(qr), hi2(f.im)));
         };
         const float t = m == 0 ? p.to_a : p.to_b;
-        const float2 lh = reinterpret_cast<const EdgeTab<1, false> *>(s.own.edge)->lohi[2 + m];
+        const float2 lh = reinterpret_cast<const EdgeTab<1, 6> *>(s.own.edge)->lohi[2 + m];
         float mine_t, other;
         if (s.w + 1 < NW && on_grid(s.z + 1, p) && on_grid(s.z + 2, p)) {
             pair_coef(pair_kind(s.z + 1, p.nz), t, lh.x, lh.y, mine_t, other);
@@ -1240,13 +1246,14 @@ __device__ __forceinline__ bool row_pair(WarpRings &r, const Seg &s, const KPara
     }
     const int yo = yin - 2 * K;
     if constexpr (SC) {   // take the launch's scale out
-        const EdgeTab<K, MODE == 5> *et = reinterpret_cast<const EdgeTab<K, MODE == 5> *>(s.own.edge);
+        const EdgeTab<K, MODE> *et = reinterpret_cast<const EdgeTab<K, MODE> *>(s.own.edge);
         auto edge = [&](int slab, int row) {
             return edge4(et->h + 9 * slab, row, p.ny, s.own.cols);
         };
         if constexpr (MODE == 6) {
             if constexpr (INTERIOR) {
-                const float4 ha = et->hrow[0][s.own.lane_class], hb = et->hrow[1][s.own.lane_class];
+                const float4 ha = et->hrow[0][s.own.lane_class];
+                const float4 hb = et->hrow[MODE == 6][s.own.lane_class];
                 unscale(O0.a, ha);
                 unscale(O1.a, ha);
                 unscale(O0.b, hb);
@@ -1383,12 +1390,12 @@ __device__ __forceinline__ bool run_segment(WarpRings &r, const CUtensorMap *tm_
     }
     Issued iss = {n_pro_s, n_pro_p, n_pro_b};
     if constexpr (SC) {   // the edge values (while the first copies are under way)
-        EdgeTab<K, MODE == 5> *et = reinterpret_cast<EdgeTab<K, MODE == 5> *>(r.edge);
+        EdgeTab<K, MODE> *et = reinterpret_cast<EdgeTab<K, MODE> *>(r.edge);
         constexpr int NE = K + 1;
         for (int i = lane; i < 3 * K + 1; i += 32)
             et->lohi[i] = i < NE ? make_float2(p.ed->elo[i], p.ed->ehi[i])
                                  : make_float2(p.ed->olo[i - NE], p.ed->ohi[i - NE]);
-        if (lane < 18) {
+        if (lane < 9 * EdgeTab<K, MODE>::SLABS) {
             const int z = s.z + (lane >= 9);
             et->h[lane] = p.ed->h[(MODE == 6 ? 9 * edge_kind(z, p.nz) : 0) + lane % 9];
         }
@@ -1397,7 +1404,8 @@ __device__ __forceinline__ bool run_segment(WarpRings &r, const CUtensorMap *tm_
         }
         __syncwarp();
         const int cls = s.own.lane_class;   // (all lanes of a class write the same values)
-        for (int i = 0; i < 2; ++i) et->hrow[i][cls] = edge4(et->h + 9 * i, -1, p.ny, s.own.cols);
+        for (int i = 0; i < EdgeTab<K, MODE>::SLABS; ++i)
+            et->hrow[i][cls] = edge4(et->h + 9 * i, -1, p.ny, s.own.cols);
         if constexpr (MODE == 5) {
             for (int i = 0; i < K; ++i) et->frow[i][cls] = edge4(et->f + 9 * i, -1, p.ny, s.own.cols);
         }
@@ -1639,7 +1647,7 @@ __global__ void __launch_bounds__(Cfg<K>::WPC * 32, multi_min_blocks(K, SC))
 fused_multi_kernel(const EpochEntry *__restrict__ tab, int n_grids, int64_t total_units,
                    int total_warps, int aligned, int flip, int *err)
 {
-    using C = CfgM<K, 0, SC>;
+    using C = CfgM<K, MULTI_MODE<SC>, SC>;
     extern __shared__ unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // the grid's parameters, per warp: in shared memory, not in registers
@@ -1647,7 +1655,7 @@ fused_multi_kernel(const EpochEntry *__restrict__ tab, int n_grids, int64_t tota
     KParams &p = params[warp];
     const int gw = blockIdx.x * C::WPC + warp;
     if (gw >= total_warps) return;
-    WarpRings r = carve_rings<K, 0, SC>(smem_raw, warp, lane);
+    WarpRings r = carve_rings<K, MULTI_MODE<SC>, SC>(smem_raw, warp, lane);
     grid_dep_sync();
     if (aligned) {
         // the grid of warp gw: the last entry whose first warp is <= gw
@@ -1673,7 +1681,7 @@ fused_multi_kernel(const EpochEntry *__restrict__ tab, int n_grids, int64_t tota
         const int q0 = (int)((int64_t)i * p.n_pairs / w);
         const int q1 = (int)((int64_t)(i + 1) * p.n_pairs / w);
         if (q1 > q0)
-            run_segment<K, SC ? 7 : 0, SC>(r, &d->tm_state[cur], &d->tm_phase, nullptr, p, sx, q0, q1, lane);
+            run_segment<K, MULTI_MODE<SC>, SC>(r, &d->tm_state[cur], &d->tm_phase, nullptr, p, sx, q0, q1, lane);
         return;
     }
     const int64_t u_begin = (int64_t)gw * total_units / total_warps;
@@ -1703,7 +1711,7 @@ fused_multi_kernel(const EpochEntry *__restrict__ tab, int n_grids, int64_t tota
         if (q1_want > q0 + left_in_grid) q1_want = q0 + left_in_grid;
         const int q1 = (int)(q1_want < p.n_pairs ? q1_want : (int64_t)p.n_pairs);
         u += q1 - q0;
-        if (!run_segment<K, SC ? 7 : 0, SC>(r, &d->tm_state[cur], &d->tm_phase, nullptr, p, sx, q0, q1, lane)) return;
+        if (!run_segment<K, MULTI_MODE<SC>, SC>(r, &d->tm_state[cur], &d->tm_phase, nullptr, p, sx, q0, q1, lane)) return;
     }
 }
 
@@ -1854,10 +1862,11 @@ cudaError_t launch_k(const FusedLaunch &a, cudaStream_t st)
     int64_t cap = (int64_t)num_sms * blocks_per_sm * C::WPC;
     // Depths 1 and 2 wait for HBM, and with every warp in flight neighbouring
     // strips drift apart: the halo columns they share leave L2 before the second
-    // strip reads them.  On grids larger than L2 (24 B per site) fewer warps keep
-    // pace (8192^2, depth 1: 290 us with 8 warps per SM, 272 with 4; depth 2: 281
-    // with 8, 264 with 7).
-    if (SC && MODE == 0 && K <= 2 && 24.0 * a.nx * a.ny > 128e6)
+    // strip reads them.  On grids far larger than L2 fewer warps keep pace (depth
+    // 1, 8 or 4 warps per SM: 3000 x 2048, 147 MB at 24 B per site, 23.3 and 27.1
+    // us, 4096^2 73.2 and 67.6, 8192^2 290 and 272; depth 2, 8 or 7: 4096^2 64.6
+    // and 71.9, 8192^2 281 and 264).
+    if (SC && MODE == 0 && K <= 2 && 24.0 * a.nx * a.ny > (K == 1 ? 256e6 : 1e9))
         cap = std::min<int64_t>(cap, (int64_t)num_sms * (K == 1 ? 4 : 7));
     p.total_warps = (int)std::min(p.units, cap);
     p.strip_warps = 0;
@@ -1894,7 +1903,7 @@ cudaError_t launch_k(const FusedLaunch &a, cudaStream_t st)
 template <int K, bool SC>
 const Occupancy &multi_occupancy()
 {
-    using C = CfgM<K, 0, SC>;
+    using C = CfgM<K, MULTI_MODE<SC>, SC>;
     static const Occupancy occ = occupancy_of(fused_multi_kernel<K, SC>, C::WPC * 32, C::SMEM);
     return occ;
 }
@@ -1903,7 +1912,7 @@ template <int K, bool SC>
 cudaError_t launch_multi_k(const EpochEntry *tab, int n_grids, const MultiPlan &plan, int flip,
                            int *err, cudaStream_t st)
 {
-    using C = CfgM<K, 0, SC>;
+    using C = CfgM<K, MULTI_MODE<SC>, SC>;
     const Occupancy &occ = multi_occupancy<K, SC>();
     if (occ.err != cudaSuccess) return occ.err;
     const int blocks = (plan.warps + C::WPC - 1) / C::WPC;

@@ -22,16 +22,20 @@ constexpr uint32_t FULL = 0xffffffffu;
 // of the table, for edge strips alone, those strips took 1.4 times as long and
 // held up the launch.)  lohi, h and f serve the rows at the edges.  Sweep
 // k < K + 1 is even sweep k, sweep K + 1 + m odd sweep m.
-template <int K, bool ADJ>
+// Kept small: 2.4 KB is what the fourth-order and the adjoint kernels have
+// beside their rings for 8 blocks per SM.  The modes are those of fused.cu.
+constexpr int LANE_CLASSES = 7;   // see lane_class
+template <int K, int MODE>
 struct EdgeTab {
-    static constexpr int SWEEPS = 3 * K + 1, CLASSES = 8;
+    static constexpr int SWEEPS = 3 * K + 1, CLASSES = LANE_CLASSES;
+    static constexpr int SLABS = MODE == 6 ? 2 : 1;   // slabs z and z + 1
     float4 recv[SWEEPS][CLASSES];
-    float4 bulk[SWEEPS];        // (-t, -t, t, t) of the sweep's bulk pairs
-    float4 hrow[2][CLASSES];    // h and f of the columns of a lane, bulk rows
-    float4 frow[ADJ ? K : 1][CLASSES];
+    float4 bulk[MODE == 7 ? SWEEPS : 1];   // (-t, -t, t, t) of the sweep's bulk pairs
+    float4 hrow[SLABS][CLASSES];   // h and f of the columns of a lane, bulk rows
+    float4 frow[MODE == 5 ? K : 1][CLASSES];
     float2 lohi[SWEEPS];
-    float h[18];     // 3 x 3 (rows by columns); MODE 6: of slab z, then of slab z + 1
-    float f[ADJ ? 9 * K : 1];
+    float h[9 * SLABS];            // 3 x 3 (rows by columns) per slab
+    float f[MODE == 5 ? 9 * K : 1];
 };
 
 // Four columns of one row of one state, held by one lane.

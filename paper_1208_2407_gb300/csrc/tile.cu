@@ -36,7 +36,7 @@ namespace ts {
 
 namespace {
 
-constexpr int SWEEPS = 3 * TILE_MAX_K + 1, CLASSES = 8;
+constexpr int SWEEPS = 3 * TILE_MAX_K + 1, CLASSES = LANE_CLASSES;
 
 // One grid of a launch.
 struct TileGrid {
