@@ -22,7 +22,8 @@
 //  - X sweeps are row-local: pairs inside a lane's float4 rotate in
 //    registers, the pair that straddles two lanes uses warp shuffles.  The
 //    strip reads h = roundup(2K, 4) halo columns per side (the valid region
-//    shrinks by 2 columns per side per step) and stores the inner 128 - 2h.
+//    shrinks by 2 columns per side per step) and stores the inner 128 - 2h (the
+//    first and the last strip up to the grid's edge).
 //  - Y sweeps couple consecutive rows held by the same lane.  The K steps form
 //    a software pipeline down the rows: an even-family sweep on a row pair
 //    that starts at an even row, or an odd-family one on a pair that starts
@@ -228,8 +229,8 @@ struct Cfg {
     // their halo columns are shared through L2 by warps that keep pace).
     static constexpr bool PSHIFT = M == 6 || (M != 4 && K >= 2);
     static constexpr int NSP = PF + K + (PSHIFT ? 0 : 1);
-    static constexpr int HALO = ((2 * K + 3) / 4) * 4;
-    static constexpr int VALID = FUSED_BOX_COLS - 2 * HALO;
+    static constexpr int HALO = depth_halo(K);
+    static constexpr int VALID = strip_valid(HALO);
     // a phase slot holds (gamma_V, s_V) and, with a drive, the V1 rows too
     static constexpr int PSLOT = PP * PLANE_SLOT_BYTES;
     // b ring (MODE 4): row pair r is read at iterations r + 2 and r + 3 and
@@ -1348,7 +1349,7 @@ __device__ __forceinline__ bool run_segment(WarpRings &r, const CUtensorMap *tm_
     s.store_a = sl.store_a;
     s.store_b = sl.store_b;
     s.lane = lane;
-    s.XL = sx * VALID - HALO;            // first loaded column (multiple of 4)
+    s.XL = sx * VALID;                   // first loaded column (multiple of 4)
     s.xg = s.XL + 4 * lane;              // this lane's first column
     s.Y0 = 2 * q0;                       // output rows [Y0, Y1)
     s.Y1 = 2 * q1;
@@ -1371,7 +1372,8 @@ __device__ __forceinline__ bool run_segment(WarpRings &r, const CUtensorMap *tm_
         s.c.Eab = {e0 ? p.tab : 0.f, e0 ? p.sab : 0.f, e1 ? p.tab : 0.f, e1 ? p.sab : 0.f};
     }
     }
-    s.store_lane = lane >= HALO / 4 && lane < 32 - HALO / 4 && xg < p.nx;
+    s.store_lane = (lane >= HALO / 4 || sx == 0) &&
+                   (lane < 32 - HALO / 4 || s.XL + FUSED_BOX_COLS >= p.nx) && xg < p.nx;
     s.own = {s.Y0, s.Y1, xg, s.store_lane, SC ? col_places(xg, p.nx) : 0u, r.edge,
              SC ? lane_class(xg, p.nx) : 0, r.sums, r.gst};
 
@@ -1805,7 +1807,7 @@ cudaError_t launch3_k(const FusedLaunch &a, int nz, cudaStream_t st)
     p.ny = a.ny;
     p.nz = nz;
     p.pitch = a.pitch;
-    p.n_strips = (a.nx + C::VALID - 1) / C::VALID;
+    p.n_strips = strip_count(a.nx, C::HALO);
     p.n_pairs = (a.ny + 1) / 2;
     p.n_zblocks = (nz + VZ - 1) / VZ;
     // Row ranges per slab: the resident CTAs take the units round robin, so
@@ -1856,7 +1858,7 @@ cudaError_t launch_k(const FusedLaunch &a, cudaStream_t st)
     p.nx = a.nx;
     p.ny = a.ny;
     p.pitch = a.pitch;
-    p.n_strips = (a.nx + C::VALID - 1) / C::VALID;
+    p.n_strips = strip_count(a.nx, C::HALO);
     p.n_pairs = (a.ny + 1) / 2;
     p.units = (int64_t)p.n_strips * p.n_pairs;
     int64_t cap = (int64_t)num_sms * blocks_per_sm * C::WPC;
@@ -2101,11 +2103,10 @@ MultiPlan fused_multi_plan(int K, bool scaled, int n, const int *nx, const int *
     // resident warps
     const int64_t cap = (int64_t)num_sms * occ->blocks_per_sm *
                         (K <= 2 ? TS_FUSED_WPC_SHALLOW : TS_FUSED_WPC_DEEP);
-    const int halo = ((2 * K + 3) / 4) * 4, valid = FUSED_BOX_COLS - 2 * halo;
     std::vector<int64_t> strips((size_t)n), pairs((size_t)n), w((size_t)n, 1);
     int64_t units = 0, all_strips = 0;
     for (int i = 0; i < n; ++i) {
-        strips[(size_t)i] = (nx[i] + valid - 1) / valid;
+        strips[(size_t)i] = strip_count(nx[i], depth_halo(K));
         pairs[(size_t)i] = (ny[i] + 1) / 2;
         units += strips[(size_t)i] * pairs[(size_t)i];
         all_strips += strips[(size_t)i];

@@ -23,8 +23,8 @@
 // pairs: each warp takes a copy of the neighbouring rows (through shared
 // memory, one barrier per step) and applies the three to them as well.
 //
-// A tile reads 2K halo rows and roundup(2K, 4) halo columns per side and
-// stores the rest.  Rows and columns off the grid are zeros whose pairs have
+// A tile reads 2K halo rows and roundup(2K, 4) halo columns per side, where the
+// grid goes on, and stores the rest.  Rows and columns off the grid are zeros whose pairs have
 // coefficient zero.
 #include <algorithm>
 
@@ -147,10 +147,10 @@ __device__ __forceinline__ void run_tile(const TileGrid &g, const ScaledEdge *ed
                                          int ty, TileShared<W> &sh)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int halo = (2 * K + 3) / 4 * 4, valid = FUSED_BOX_COLS - 2 * halo;
+    const int halo = depth_halo(K);
     const int rows = R * W - 4 * K;              // rows stored per tile
-    const int y0 = ty * rows - 2 * K;            // the tile's first row (even)
-    const int xg = sx * valid - halo + 4 * lane; // the lane's first column
+    const int y0 = ty * rows;                    // the tile's first row (even)
+    const int XL = sx * strip_valid(halo), xg = XL + 4 * lane;   // the lane's first column
     TileCtx c = {K, y0 + R * warp, g.ny, warp, lane, lane_class(xg, g.nx),
                  g.te_end, g.te_mid, g.to_a, g.to_b};
 
@@ -220,13 +220,15 @@ __device__ __forceinline__ void run_tile(const TileGrid &g, const ScaledEdge *ed
         tile_steps<R, W, false>(st, tg, tv, c, sh);
 
     grid_dep_launch();
-    const bool store = col && 4 * lane >= halo && 4 * lane < FUSED_BOX_COLS - halo;
+    const bool store = col && (4 * lane >= halo || sx == 0) &&
+                       (4 * lane < FUSED_BOX_COLS - halo || XL + FUSED_BOX_COLS >= g.nx);
+    const bool first = ty == 0, last = y0 + R * W >= g.ny;   // tiles at the grid's top and bottom
     const float4 hb = sh.hrow[c.cls];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int t = R * warp + r, y = y0 + t;
         unscale(st[r], edge ? edge4(sh.h, y, g.ny, cols) : hb);
-        if (store && t >= 2 * K && t < R * W - 2 * K && y < g.ny) {
+        if (store && (t >= 2 * K || first) && (t < R * W - 2 * K || last) && y < g.ny) {
             const int64_t o = (int64_t)y * g.pitch + xg;
             *reinterpret_cast<float4 *>(g.out_re + o) = st[r].re;
             *reinterpret_cast<float4 *>(g.out_im + o) = st[r].im;
@@ -265,8 +267,7 @@ tile_multi_kernel(const EpochEntry *__restrict__ tab, int n_grids, int K, int fl
     const ScaledCoef &c = d->sc[K - 1];
     const TileGrid g = {d->re[cur], d->im[cur], d->pg, d->ps, d->re[cur ^ 1], d->im[cur ^ 1],
                         d->nx, d->ny, d->pitch, c.te_end, c.te_mid, c.to_a, c.to_b};
-    const int valid = FUSED_BOX_COLS - 2 * ((2 * K + 3) / 4 * 4);
-    const int strips = (d->nx + valid - 1) / valid, b = (int)(blockIdx.x - e.begin);
+    const int strips = strip_count(d->nx, depth_halo(K)), b = (int)(blockIdx.x - e.begin);
     run_tile<R, W>(g, &c.edge, K, b % strips, b / strips, *reinterpret_cast<TileShared<W> *>(smem));
 }
 
@@ -313,8 +314,11 @@ constexpr Shape shapes[TILE_SHAPES] = {{4, 8}, {4, 10}, {8, 8}};
 
 int64_t tiles_of(int K, const Shape &s, int nx, int ny)
 {
-    const int valid = FUSED_BOX_COLS - 2 * ((2 * K + 3) / 4 * 4), rows = s.r * s.w - 4 * K;
-    return (int64_t)((nx + valid - 1) / valid) * ((ny + rows - 1) / rows);
+    // rows of tiles as strips of columns: the first and the last store their
+    // halo at the grid's edge
+    const int rows = s.r * s.w - 4 * K;
+    const int64_t down = ny <= s.r * s.w ? 1 : (ny - 4 * K + rows - 1) / rows;
+    return strip_count(nx, depth_halo(K)) * down;
 }
 
 }  // namespace
@@ -335,7 +339,7 @@ int tile_blocks(int K, int shape, int nx, int ny) { return (int)tiles_of(K, shap
 
 // Tiles or warp streams?  Tiles of 64 rows in at most K rounds of one block
 // per SM.  Measured, one launch at depth 4 (us), tiles against streams: 256^2
-// 6.0 / 14.9, 512^2 6.8 / 14.7, 1001 x 777 12.4 / 19.4, 1024^2 14.4 / 22.2 (2
+// 6.0 / 14.9, 512^2 6.7 / 14.7, 1001 x 777 8.3 / 19.4, 1024^2 14.4 / 22.2 (2
 // rounds), 1500^2 22.4 / 28.6 (3), 2048^2 43 / 31.9 (6).  A tile recomputes its
 // halo (at depth 4 three quarters of its rows and 7/8 of its columns are
 // stored), so once the SMs are full the streams win; at a smaller depth sooner,
@@ -371,7 +375,7 @@ int tile_shape(int K, int n, const int *nx, const int *ny)
 cudaError_t launch_tile(int K, int shape, const TileLaunch &a, cudaStream_t st)
 {
     if (K < 1 || K > TILE_MAX_K || !a.sc) return cudaErrorInvalidValue;
-    const int valid = FUSED_BOX_COLS - 2 * ((2 * K + 3) / 4 * 4), strips = (a.nx + valid - 1) / valid;
+    const int strips = strip_count(a.nx, depth_halo(K));
     const int blocks = tile_blocks(K, shape, a.nx, a.ny);
     switch (shape) {
     case 0: return launch_one<4, 8>(K, a, blocks, strips, st);

@@ -20,7 +20,7 @@ from gpu_helpers import random_state, rel_l2, run_gpu
 pytestmark = pytest.mark.gpu
 
 STEPS, TOL = 13, 2e-6
-SIDES = [(1, 9), (2, 8), (3, 7), (4, 6), (5, 5), (6, 4), (7, 3), (8, 2), (9, 1), (111, 12),
+SIDES = [(124, 5), (125, 6), (126, 4), (127, 9), (128, 3), (129, 8), (240, 10), (241, 9), (1, 9), (2, 8), (3, 7), (4, 6), (5, 5), (6, 4), (7, 3), (8, 2), (9, 1), (111, 12),
          (112, 13), (113, 14), (114, 5), (115, 6), (116, 33), (119, 8), (120, 7), (121, 6),
          (225, 40), (226, 41)]
 

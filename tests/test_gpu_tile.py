@@ -13,7 +13,7 @@ from gpu_helpers import random_state, rel_l2
 
 pytestmark = pytest.mark.gpu
 
-SIDES = [(1, 1), (2, 5), (3, 9), (4, 17), (5, 24), (9, 25), (111, 48), (112, 49), (113, 16),
+SIDES = [(128, 30), (240, 32), (241, 65), (1, 1), (2, 5), (3, 9), (4, 17), (5, 24), (9, 25), (111, 48), (112, 49), (113, 16),
          (225, 33), (300, 47), (130, 97), (7, 200), (500, 301)]
 
 
