@@ -19,7 +19,7 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(ROOT, "_build")
 LIB = os.path.join(PKG, "libtrotter.so")
-SOURCES = ["api.cu", "tile.cu", "fused64.cu", "plain.cu", "reduce.cu", "adjoint.cu", "server.cu", "noalloc.cu",
+SOURCES = ["api.cu", "tile.cu", "tile_adjoint.cu", "fused64.cu", "plain.cu", "reduce.cu", "adjoint.cu", "server.cu", "noalloc.cu",
            "lattice3d.cu", "selftest.cu"]
 FUSED_PARTS = 16   # fused.cu is compiled in parts (-DTS_FUSED_PART=n), in parallel
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

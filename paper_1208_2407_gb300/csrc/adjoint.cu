@@ -225,7 +225,6 @@ ts_status ts_adjoint_backward_depth(ts_grid *g, void *ws, size_t ws_bytes, int K
     if (K < 0 || K > ts::FUSED_ADJ_MAX_K)
         return err(TS_ERR_ARG, "ts_adjoint_backward: depth K must be in [0, %d]",
                    ts::FUSED_ADJ_MAX_K);
-    const int KA = K > 0 ? K : TS_ADJ_DEFAULT_K;
     AdjointState a;
     {
         std::lock_guard<std::mutex> lk(g_adj_mu);
@@ -277,6 +276,12 @@ ts_status ts_adjoint_backward_depth(ts_grid *g, void *ws, size_t ws_bytes, int K
     const double sub[ts::FUSED_ADJ_MAX_K] = {th, th, th, th};
     ts::ScaledCoef sc;
     int sc_k = 0;
+    // Depth 4 on tiles where they serve, else depth 3 on streams (us per step,
+    // tiles and streams at those depths: 300 x 400 4.3 and 5.6, 512^2 4.4 and
+    // 6.8, 1024^2 7.9 and 9.2, 1500^2 20.6 and 13.5).
+    const int KA = K > 0 ? K
+                   : scaled && ts::tile_adjoint_serves(4, nx, ny) ? 4
+                                                                  : TS_ADJ_DEFAULT_K;
 
     int q = 0;   // psi and lambda in quad q (0: QA, 1: QB)
     auto quad = [&](int i) { return i ? WS_QB : WS_QA; };
@@ -293,6 +298,24 @@ ts_status ts_adjoint_backward_depth(ts_grid *g, void *ws, size_t ws_bytes, int K
                 sc_k = kk;
             }
             bw.sc = scaled ? &sc : nullptr;
+            if (scaled && ts::tile_adjoint_serves(kk, nx, ny)) {
+                ts::TileAdjoint t;
+                for (int i = 0; i < 4; ++i) {
+                    t.in[i] = (const float *)plane(quad(q) + i);
+                    t.out[i] = (float *)plane(quad(q ^ 1) + i);
+                    t.g[i] = (float *)plane(WS_G + i);
+                }
+                t.pg = (const float *)g->pg();
+                t.ps = (const float *)g->ps();
+                t.nx = nx;
+                t.ny = ny;
+                t.pitch = pitch;
+                e = ts::launch_tile_adjoint(kk, t, sc, st);
+                if (e != cudaSuccess) return cuda_err(e, "ts_adjoint_backward: backward launch");
+                q ^= 1;
+                i -= kk;
+                continue;
+            }
             bw.tm_state = &tmQ[q];
             bw.out_re = (float *)plane(quad(q ^ 1));
             bw.out_im = (float *)plane(quad(q ^ 1) + 1);

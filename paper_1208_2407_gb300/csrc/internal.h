@@ -220,6 +220,21 @@ int tile_blocks(int K, int shape, int nx, int ny);
 // that depth, bit for bit.
 cudaError_t launch_tile(int K, int shape, const TileLaunch &a, cudaStream_t st);
 
+// --- backward adjoint steps on tiles (tile_adjoint.cu) --------------------
+struct TileAdjoint {
+    const float *in[4];   // psi re, im, lambda re, im
+    float *out[4];
+    float *g[4];          // G: re hi, re lo, im hi, im lo
+    const float *pg, *ps;
+    int nx, ny;
+    int64_t pitch;
+};
+// whether a launch of depth K is faster on tiles than on warp streams
+bool tile_adjoint_serves(int K, int nx, int ny);
+// What launch_fused_adjoint does at depth K (1..FUSED_ADJ_MAX_K) with scaled
+// rotations (c: coefficients at -theta).
+cudaError_t launch_tile_adjoint(int K, const TileAdjoint &p, const ScaledCoef &c, cudaStream_t st);
+
 // Device-resident description of one FP32 grid for the multi-grid launch
 // (written once per grid set-up; read by the kernel with generic loads, its
 // tensor maps by TMA).
