@@ -127,6 +127,9 @@ ts_status grid_setup(const ts_layout &L, void *slab, bool owns_slab, ts_grid **o
     g->desc_dev = (GridDesc *)scr;
     g->cur = 0;
     g->dt = g->theta = g->J = 0.0;
+    g->desc_written = false;
+    g->sc_theta = 0.0;   // at theta = 0 every coefficient is 0
+    std::memset(g->desc_host.sc, 0, sizeof(g->desc_host.sc));
     g->g1 = g->s1 = g->t1 = g->s2 = g->t2 = 0.0;
     g->order = 2;
     g->sub[0] = g->sub[1] = RotCoef{0.0, 0.0, 0.0, 0.0, 0.0};
@@ -247,7 +250,8 @@ void grid_set_coefficients(ts_grid *g, double dt, double theta, cudaStream_t st)
     g->t1 = c.t1;
     g->s2 = c.s2;
     g->t2 = c.t2;
-    if (!g->f64()) grid_write_desc(g, st);
+    // the descriptor holds no dt: it stands while the angle does
+    if (!g->f64() && !(g->desc_written && g->sc_theta == g->theta)) grid_write_desc(g, st);
 }
 
 void grid_write_desc(ts_grid *g, cudaStream_t st)
@@ -272,8 +276,13 @@ void grid_write_desc(ts_grid *g, cudaStream_t st)
     d.ps = (const float *)g->ps();
     const double sub[FUSED_MAX_K] = {g->theta, g->theta, g->theta, g->theta,
                                      g->theta, g->theta, g->theta, g->theta};
-    for (int K = 1; K <= FUSED_MAX_K; ++K)
-        scaled_coef(sub, K, g->L.nx, g->L.ny, g->L.nz, d.sc[K - 1]);
+    // (some 500 tangents: only when the angle changes)
+    if (g->sc_theta != g->theta) {
+        for (int K = 1; K <= FUSED_MAX_K; ++K)
+            scaled_coef(sub, K, g->L.nx, g->L.ny, g->L.nz, d.sc[K - 1]);
+        g->sc_theta = g->theta;
+    }
+    g->desc_written = true;
     // pageable source: the call returns once the host struct is staged, and
     // the device copy lands in stream order before later kernels read it
     cudaMemcpyAsync(g->desc_dev, &d, sizeof(GridDesc), cudaMemcpyHostToDevice, st);

@@ -60,6 +60,8 @@ struct ts_grid {
     CUtensorMap tm_state[2], tm_phase;   // (re, im) of pair 0 / 1; (gamma_V, s_V)
     ts::GridDesc *desc_dev;              // the same, for multi-grid launches (in the slab)
     ts::GridDesc desc_host;
+    double sc_theta;                     // the angle of desc_host.sc
+    bool desc_written;                   // desc_dev holds desc_host
 
     void *plane(int i) const { return slab + (size_t)i * L.plane_bytes; }
     void *re() const { return plane(2 * cur); }
