@@ -282,10 +282,14 @@ void grid_write_desc(ts_grid *g, cudaStream_t st)
             scaled_coef(sub, K, g->L.nx, g->L.ny, g->L.nz, d.sc[K - 1]);
         g->sc_theta = g->theta;
     }
-    g->desc_written = true;
     // pageable source: the call returns once the host struct is staged, and
-    // the device copy lands in stream order before later kernels read it
-    cudaMemcpyAsync(g->desc_dev, &d, sizeof(GridDesc), cudaMemcpyHostToDevice, st);
+    // the device copy lands in stream order before later kernels read it; a
+    // captured copy only does when its graph runs
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const cudaError_t q = cudaStreamIsCapturing(st, &cap);
+    const cudaError_t e =
+        cudaMemcpyAsync(g->desc_dev, &d, sizeof(GridDesc), cudaMemcpyHostToDevice, st);
+    g->desc_written = e == cudaSuccess && q == cudaSuccess && cap == cudaStreamCaptureStatusNone;
 }
 
 cudaError_t evolve_multi(ts_grid *const *gs, const int64_t *steps, int n, int K, bool scaled,

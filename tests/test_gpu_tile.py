@@ -69,3 +69,30 @@ def test_captured_evolution():
         finally:
             g.close()
     assert np.array_equal(outs[0][0], outs[1][0]) and np.array_equal(outs[0][1], outs[1][1])
+
+
+def test_potential_set_under_capture_then_again():
+    """A captured set_potential has not run: the next one at the same angle still
+    writes what a multi-grid launch reads."""
+    import torch
+
+    n, theta = 200, 0.03
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    V = torch.rand(n, n, dtype=torch.float64, device="cuda", generator=gen)
+    re, im = torch.randn(2, n, n, device="cuda", generator=gen)
+    grids = [trotter.Grid(n, n, "f32") for _ in range(2)]
+    try:
+        for g in grids:
+            g.set_state(re, im)
+        torch.cuda.synchronize()
+        with torch.cuda.graph(torch.cuda.CUDAGraph()):
+            grids[0].set_potential(V, 2.0 * theta, theta)
+        for g in grids:
+            g.set_potential(V, 2.0 * theta, theta)
+        trotter.evolve_batched(grids[:1], [8], 4)
+        grids[1].evolve(8, 4)
+        a, b = (g.get_state(np.float32) for g in grids)
+    finally:
+        for g in grids:
+            g.close()
+    assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
