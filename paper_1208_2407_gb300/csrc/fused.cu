@@ -1249,7 +1249,7 @@ __device__ __forceinline__ bool row_pair(WarpRings &r, const Seg &s, const KPara
     if constexpr (SC) {   // take the launch's scale out
         const EdgeTab<K, MODE> *et = reinterpret_cast<const EdgeTab<K, MODE> *>(s.own.edge);
         auto edge = [&](int slab, int row) {
-            return edge4(et->h + 9 * slab, row, p.ny, s.own.cols);
+            return edge_h(et->h + 13 * slab, row, p.ny, s.own.cols);
         };
         if constexpr (MODE == 6) {
             if constexpr (INTERIOR) {
@@ -1397,9 +1397,9 @@ __device__ __forceinline__ bool run_segment(WarpRings &r, const CUtensorMap *tm_
         for (int i = lane; i < 3 * K + 1; i += 32)
             et->lohi[i] = i < NE ? make_float2(p.ed->elo[i], p.ed->ehi[i])
                                  : make_float2(p.ed->olo[i - NE], p.ed->ohi[i - NE]);
-        if (lane < 9 * EdgeTab<K, MODE>::SLABS) {
-            const int z = s.z + (lane >= 9);
-            et->h[lane] = p.ed->h[(MODE == 6 ? 9 * edge_kind(z, p.nz) : 0) + lane % 9];
+        if (lane < 13 * EdgeTab<K, MODE>::SLABS) {
+            const int i = lane % 13, z = MODE == 6 ? edge_kind(s.z + (lane >= 13), p.nz) : 0;
+            et->h[lane] = i < 9 ? p.ed->h[9 * z + i] : p.ed->hb[z][i - 9];
         }
         if constexpr (MODE == 5) {
             for (int i = lane; i < 9 * K; i += 32) et->f[i] = p.ed->f[i / 9][i % 9];
@@ -1407,7 +1407,7 @@ __device__ __forceinline__ bool run_segment(WarpRings &r, const CUtensorMap *tm_
         __syncwarp();
         const int cls = s.own.lane_class;   // (all lanes of a class write the same values)
         for (int i = 0; i < EdgeTab<K, MODE>::SLABS; ++i)
-            et->hrow[i][cls] = edge4(et->h + 9 * i, -1, p.ny, s.own.cols);
+            et->hrow[i][cls] = edge_h(et->h + 13 * i, -1, p.ny, s.own.cols);
         if constexpr (MODE == 5) {
             for (int i = 0; i < K; ++i) et->frow[i][cls] = edge4(et->f + 9 * i, -1, p.ny, s.own.cols);
         }

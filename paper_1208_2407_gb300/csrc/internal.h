@@ -103,11 +103,15 @@ constexpr int FUSED_ADJ_MAX_K = 4;
 // an edge of the grid receive in even sweep k and odd sweep m (the edge member
 // lo, its partner hi), h = 1 - scale of a launch for a site at place (z, y, x),
 // entry 9 z + 3 y + x with 0 bulk, 1 the first site of the axis, 2 the last,
-// and (adjoint) the squared scale at phase k, entry 3 y + x.
+// and (adjoint) the squared scale at phase k, entry 3 y + x.  In the bulk of x
+// and y, column i mod 4 takes hb[z][i] instead of h[9 z]: the two floats around
+// h, mixed so that their mean is nearer to it than one float is (the rounding of
+// h is the same at every site and launch, and would show in the norm).
 struct ScaledEdge {
     float elo[FUSED_MAX_K + 1], ehi[FUSED_MAX_K + 1];
     float olo[2 * FUSED_MAX_K], ohi[2 * FUSED_MAX_K];
     float h[27];
+    float hb[3][4];
     float f[FUSED_ADJ_MAX_K][9];
 };
 // The bulk coefficients (tangents) of a launch: even sweeps 0 and K, the even

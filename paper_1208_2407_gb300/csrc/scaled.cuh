@@ -34,7 +34,7 @@ struct EdgeTab {
     float4 hrow[SLABS][CLASSES];   // h and f of the columns of a lane, bulk rows
     float4 frow[MODE == 5 ? K : 1][CLASSES];
     float2 lohi[SWEEPS];
-    float h[9 * SLABS];            // 3 x 3 (rows by columns) per slab
+    float h[13 * SLABS];           // per slab: 3 x 3 (rows by columns), the 4 of the bulk
     float f[MODE == 5 ? 9 * K : 1];
 };
 
@@ -243,6 +243,18 @@ __device__ __forceinline__ float4 edge4(const float *tab, int row, int ny, unsig
 {
     const float *t = tab + 3 * edge_kind(row, ny);
     return make_float4(t[cols & 3], t[cols >> 2 & 3], t[cols >> 4 & 3], t[cols >> 6 & 3]);
+}
+
+// h of one row of the lane: as edge4, and in the bulk each column's own (entries
+// 9 .. 12 of the table)
+__device__ __forceinline__ float4 edge_h(const float *tab, int row, int ny, unsigned cols)
+{
+    const float *t = tab + 3 * edge_kind(row, ny);
+    auto at = [&](int i) {
+        const int k = cols >> 2 * i & 3;
+        return t[k == 0 && t == tab ? 9 + i : k];
+    };
+    return make_float4(at(0), at(1), at(2), at(3));
 }
 
 // asynchronous 16-byte copies to shared memory (zfill: zeros unless `in`)

@@ -52,7 +52,7 @@ struct TileShared {
     float4 recv[SWEEPS][CLASSES];   // as EdgeTab in scaled.cuh
     float4 hrow[CLASSES];
     float2 lohi[SWEEPS];
-    float h[9];
+    float h[13];
     // first and last row of each warp (re, im), two buffers
     float4 ex[2][W][2][2][32];
 };
@@ -161,7 +161,8 @@ __device__ __forceinline__ void run_tile(const TileGrid &g, const ScaledEdge *ed
     for (int i = threadIdx.x; i < 3 * K + 1; i += 32 * W)
         sh.lohi[i] = i <= K ? make_float2(ed->elo[i], ed->ehi[i])
                             : make_float2(ed->olo[i - K - 1], ed->ohi[i - K - 1]);
-    if (threadIdx.x < 9) sh.h[threadIdx.x] = ed->h[threadIdx.x];
+    if (threadIdx.x < 13)
+        sh.h[threadIdx.x] = threadIdx.x < 9 ? ed->h[threadIdx.x] : ed->hb[0][threadIdx.x - 9];
     __syncthreads();
     for (int i = warp; i < 3 * K + 1; i += W) {
         const float2 lh = sh.lohi[i];
@@ -179,7 +180,7 @@ __device__ __forceinline__ void run_tile(const TileGrid &g, const ScaledEdge *ed
         }
         sh.recv[i][c.cls] = v;   // the same value from every lane of the class
     }
-    if (warp == 0) sh.hrow[c.cls] = edge4(sh.h, -1, g.ny, cols);
+    if (warp == 0) sh.hrow[c.cls] = edge_h(sh.h, -1, g.ny, cols);
     __syncthreads();
     grid_dep_sync();
 
@@ -227,7 +228,7 @@ __device__ __forceinline__ void run_tile(const TileGrid &g, const ScaledEdge *ed
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int t = R * warp + r, y = y0 + t;
-        unscale(st[r], edge ? edge4(sh.h, y, g.ny, cols) : hb);
+        unscale(st[r], edge ? edge_h(sh.h, y, g.ny, cols) : hb);
         if (store && (t >= 2 * K || first) && (t < R * W - 2 * K || last) && y < g.ny) {
             const int64_t o = (int64_t)y * g.pitch + xg;
             *reinterpret_cast<float4 *>(g.out_re + o) = st[r].re;

@@ -28,7 +28,7 @@ struct Shared {
     float4 recv[SWEEPS][CLASSES];   // as EdgeTab in scaled.cuh
     float4 hrow[CLASSES], frow[MAX_K][CLASSES];
     float2 lohi[SWEEPS];
-    float h[9], f[MAX_K][9];
+    float h[13], f[MAX_K][9];
     // first and last row of each warp (psi re, im, lambda re, im), two buffers
     float4 ex[2][W][2][4][32];
     float4 tab[ROWS][2][32];   // gamma_V, s_V
@@ -193,7 +193,8 @@ tile_adjoint_kernel(const TileAdjoint p, const __grid_constant__ ScaledEdge ed,
     for (int i = threadIdx.x; i < 3 * K + 1; i += 32 * W)
         sh.lohi[i] = i <= K ? make_float2(ed.elo[i], ed.ehi[i])
                             : make_float2(ed.olo[i - K - 1], ed.ohi[i - K - 1]);
-    if (threadIdx.x < 9) sh.h[threadIdx.x] = ed.h[threadIdx.x];
+    if (threadIdx.x < 13)
+        sh.h[threadIdx.x] = threadIdx.x < 9 ? ed.h[threadIdx.x] : ed.hb[0][threadIdx.x - 9];
     if (threadIdx.x < 9 * K) sh.f[threadIdx.x / 9][threadIdx.x % 9] = ed.f[threadIdx.x / 9][threadIdx.x % 9];
     __syncthreads();
     for (int i = warp; i < 3 * K + 1; i += W) {
@@ -212,7 +213,7 @@ tile_adjoint_kernel(const TileAdjoint p, const __grid_constant__ ScaledEdge ed,
         }
         sh.recv[i][c.cls] = v;   // the same value from every lane of the class
     }
-    if (warp == 0) sh.hrow[c.cls] = edge4(sh.h, -1, p.ny, cols);
+    if (warp == 0) sh.hrow[c.cls] = edge_h(sh.h, -1, p.ny, cols);
     if (warp >= 1 && warp <= K) sh.frow[warp - 1][c.cls] = edge4(sh.f[warp - 1], -1, p.ny, cols);
     __syncthreads();
     grid_dep_sync();
@@ -271,7 +272,7 @@ tile_adjoint_kernel(const TileAdjoint p, const __grid_constant__ ScaledEdge ed,
     const float4 hb = sh.hrow[c.cls];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const float4 h = edge ? edge4(sh.h, c.yw + r, p.ny, cols) : hb;
+        const float4 h = edge ? edge_h(sh.h, c.yw + r, p.ny, cols) : hb;
         unscale(st[r].a, h);
         unscale(st[r].b, h);
         if (!mine[r]) continue;
