@@ -121,7 +121,8 @@ ts_status ts_set_state(ts_grid *g, const void *re, const void *im,
 
 /* Read the state into dense arrays of `dst_dtype` (host or device).  Syncs
  * `stream`; reports TS_ERR_TIMEOUT if a bounded wait inside an earlier fused
- * launch gave up, TS_ERR_CUDA for a failed earlier launch. */
+ * launch gave up, TS_ERR_CUDA for a failed earlier launch.  On either error
+ * what the arrays hold is undefined. */
 ts_status ts_get_state(ts_grid *g, void *re, void *im, ts_dtype dst_dtype,
                        ts_mem where, void *stream);
 
@@ -189,13 +190,19 @@ ts_status ts_clear_drive(ts_grid *g);
 /* Evolve `steps` second-order steps (Eq. secondorder) on the grid's current
  * state.  FP32 grids run the fused kernel: K whole steps per HBM round trip
  * on TMA-staged shared-memory tiles (temporal blocking; K = 0 picks the
- * depth automatically, 1 <= K <= 8 forces it; a remainder of steps % K runs
- * at a smaller depth).  FP64 grids run one sweep per launch (K must be 0,
- * else TS_ERR_UNSUPPORTED), with the sweeps of one axis merged where two
+ * depth automatically: 4, or 3 when |theta| > 0.075 and the grid has fewer
+ * than 2^21 sites; 1 <= K <= 8 asks for a
+ * depth, of which at most 4 is used when |theta| > 0.075; a remainder of
+ * steps % K runs at a smaller depth).  |theta| > pi/4 takes the plain path.
+ * Small and middle grids run the same steps on tiles held in registers, with
+ * the same results bit for bit.  FP64 grids (K must be 0, else
+ * TS_ERR_UNSUPPORTED) run one step per launch and pass over memory when they
+ * are 2-D, have no drive, at least 1024 sites and |theta| <= pi/8; others run
+ * one sweep per launch, with the sweeps of one axis merged where two
  * steps or substeps meet (X, Y and Z factors commute; two factors of one
  * family add their angles: n second-order steps take 6n + 2 sweeps in 2-D,
- * 9n + 3 in 3-D) and the lifting form for angles up to pi/2; the results
- * agree with ts_evolve_plain to FP64 rounding.  On a grid set to order 4
+ * 9n + 3 in 3-D) and the lifting form for angles up to pi/2.  Either way the
+ * results agree with ts_evolve_plain to FP64 rounding.  On a grid set to order 4
  * (ts_set_potential_order) each step is U4(dt): on FP32 grids with K = 0
  * each step is one launch that applies all five
  * substeps; with K >= 1 the p dt substeps of neighbouring steps run as
@@ -269,7 +276,7 @@ ts_status ts_evolve_batched(ts_grid *const *g, int n, const int64_t *steps, int 
  *   dense nx*ny FP32 device array `grad`.  Syncs.  One forward/backward pair
  *   per grid at a time; TS_ERR_STATE without a matching forward.
  *   psi and lambda step back together, K steps per fused launch (K = 3, or 4 on
- *   small grids).
+ *   grids small enough for the register tiles).
  * ts_adjoint_backward_depth: the same with the depth K of those launches
  *   given (1..4; 0 = the default); other K return TS_ERR_ARG.  K changes only
  *   the order in which G's terms are summed, not the gradient it defines.
@@ -390,7 +397,7 @@ ts_status ts_norm_noalloc(const void *re, const void *im, ts_dtype dtype, int64_
                           int64_t ny, int64_t pitch, double *out, void *stream);
 size_t ts_norm_noalloc_scratch_bytes(void);
 
-/* The fused depth ts_evolve uses when K = 0. */
+/* The fused depth ts_evolve uses when K = 0 (for |theta| <= 0.075). */
 int ts_fused_default_depth(void);
 
 /* Number of kernels this thread's calls enqueued since the last reset. */

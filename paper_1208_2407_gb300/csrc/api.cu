@@ -41,9 +41,15 @@ constexpr int64_t kMaxSide = int64_t(1) << 20;
 // Depth of the fused path when the caller passes K = 0.  On one GB300 at
 // 8192^2 (site-steps/s) with scaled rotations: K=2 4.6e11, K=3 8.0e11, K=4
 // 9.4e11, K=5 8.9e11, K=6 9.1e11; at 2048^2 K=3 4.7e11, K=4 4.8e11, K=5 4.6e11.
-// In the lifting form (larger angles): K=2 5.2e11, K=3 7.5e11 (88 % of the HBM
-// copy bandwidth), K=4 7.8e11, but K=4 is slower than K=3 at 2048^2.
-int auto_depth(bool scaled = true) { return scaled ? 4 : 3; }
+// In the lifting form (larger angles) the smaller grids are faster at K=3 (us per
+// step, K=3 and K=4: 1024^2 4.1 and 4.6, 1200^2 4.8 and 5.3), those from 2 M sites
+// on at K=4 (1500^2 6.1 and 6.0, 2048^2 9.2 and 8.1, 8192 x 512 9.2 and 8.2,
+// 8192^2 92 and 84).
+int auto_depth(const ts_grid *g)
+{
+    const bool scaled = std::fabs(g->theta) <= ts::SCALED_MAX_THETA;
+    return scaled || g->L.nx * g->L.ny >= (1 << 21) ? 4 : 3;
+}
 constexpr int kPlanes = 7;   // re_a, im_a, re_b, im_b, gamma_V, s_V, V
 
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -422,7 +428,7 @@ extern "C" {
 
 const char *ts_last_error(void) { return g_err; }
 
-int ts_fused_default_depth(void) { return auto_depth(); }
+int ts_fused_default_depth(void) { return 4; }
 
 int64_t ts_launch_count(int reset)
 {
@@ -1333,8 +1339,7 @@ ts_status ts_evolve(ts_grid *g, int64_t steps, int K, void *stream)
     // (|2 theta| <= pi/2).  Larger angles -- far beyond any useful Trotter
     // step -- run the one-sweep-per-kernel path.
     if (std::fabs(g->theta) > 0.25 * M_PI) return plain_steps(g, steps, st);
-    const bool scaled = std::fabs(g->theta) <= ts::SCALED_MAX_THETA;
-    return fused_steps(g, steps, K == 0 ? auto_depth(scaled) : K, st);
+    return fused_steps(g, steps, K == 0 ? auto_depth(g) : K, st);
 }
 
 ts_status ts_check_wait_timeout(ts_grid *g, int64_t limit_ns, void *stream)
@@ -1367,9 +1372,10 @@ ts_status ts_evolve_batched(ts_grid *const *gs, int n, const int64_t *steps, int
     cudaStream_t st = (cudaStream_t)stream;
     // grids the multi-grid kernel can take: 2-D, FP32, second order, no
     // drive, |theta| <= pi/4; the rest evolve one by one
-    // (those with scaled rotations, then those in the lifting form)
-    std::vector<ts_grid *> multi[2];
-    std::vector<int64_t> msteps[2];
+    // (those with scaled rotations, then those in the lifting form by depth)
+    std::vector<ts_grid *> multi[3];
+    std::vector<int64_t> msteps[3];
+    int depth[3] = {};
     for (int i = 0; i < n; ++i) {
         if (!gs[i] || steps[i] < 0) return fail(TS_ERR_ARG, "ts_evolve_batched: grid %d", i);
         if (steps[i] == 0) continue;
@@ -1379,15 +1385,16 @@ ts_status ts_evolve_batched(ts_grid *const *gs, int n, const int64_t *steps, int
             ts_status s = ts_evolve(gs[i], steps[i], gs[i]->f64() ? 0 : K, stream);
             if (s != TS_OK) return s;
         } else {
-            const int form = std::fabs(gs[i]->theta) <= ts::SCALED_MAX_THETA ? 0 : 1;
+            const int k = K == 0 ? auto_depth(gs[i]) : K;
+            const int form = std::fabs(gs[i]->theta) <= ts::SCALED_MAX_THETA ? 0 : k == 3 ? 1 : 2;
+            depth[form] = k;
             multi[form].push_back(gs[i]);
             msteps[form].push_back(steps[i]);
         }
     }
-    for (int form = 0; form < 2; ++form) {
-        const int depth = K == 0 ? auto_depth(form == 0) : K;
+    for (int form = 0; form < 3; ++form) {
         cudaError_t e = ts::evolve_multi(multi[form].data(), msteps[form].data(),
-                                         (int)multi[form].size(), depth, form == 0, st);
+                                         (int)multi[form].size(), depth[form], form == 0, st);
         if (e != cudaSuccess) return cuda_fail(e, "ts_evolve_batched: multi-grid launch");
     }
     return TS_OK;

@@ -83,3 +83,24 @@ def test_batch_of_both_forms_equals_solo_runs():
     finally:
         for g in grids:
             g.close()
+
+
+@pytest.mark.parametrize("nx,ny,depth", [(1448, 1448, 3), (1449, 1448, 4)])
+def test_default_depth_of_the_lifting_form(nx, ny, depth):
+    """Around 2^21 sites, alone and batched: bit for bit the launches of `depth`."""
+    rng = np.random.default_rng(nx)
+    re, im = random_state(rng, nx, ny)
+    V = rng.uniform(-0.5, 0.5, (ny, nx))
+    out = []
+    for run in (lambda g: g.evolve(13), lambda g: g.evolve(13, depth),
+                lambda g: trotter.evolve_batched([g], [13])):
+        g = trotter.Grid(nx, ny, "f32")
+        try:
+            g.set_state(re, im)
+            g.set_potential(V, 0.2, 0.1)
+            run(g)
+            out.append(g.get_state(np.float32))
+        finally:
+            g.close()
+    for r, i in out[1:]:
+        assert np.array_equal(r, out[0][0]) and np.array_equal(i, out[0][1])
