@@ -1317,7 +1317,7 @@ ts_status ts_evolve(ts_grid *g, int64_t steps, int K, void *stream)
     if (g->f64()) {
         if (K != 0)
             return fail(TS_ERR_UNSUPPORTED,
-                        "ts_evolve: FP64 grids run one sweep per launch (K must be 0)");
+                        "ts_evolve: FP64 grids take no depth (K must be 0)");
         return evolve_f64(g, steps, st);
     }
     if (g->is3d()) {

@@ -2087,7 +2087,7 @@ MultiPlan fused_multi_plan(int K, bool scaled, int n, const int *nx, const int *
                            EpochEntry *tab)
 {
     MultiPlan plan = {0, 0, false, -1};
-    if (scaled && n >= 1) plan.shape = tile_shape(K, n, nx, ny);
+    if (scaled && n >= 1) plan.shape = tile_shape(K, n, nx, ny, true);
     if (plan.shape >= 0) {
         for (int i = 0; i < n; ++i) {
             tab[i].begin = plan.units;

@@ -214,10 +214,11 @@ struct TileLaunch {
     const ScaledCoef *sc;   // of depth K
 };
 // The tile shape for a launch of depth K over n grids with scaled rotations,
-// or -1 where the warp streams are faster (or K > TILE_MAX_K).
-constexpr int TILE_SHAPES = 3;
+// or -1 where the warp streams are faster (or K > TILE_MAX_K).  multi: for
+// launch_tile_multi.
+constexpr int TILE_SHAPES = 4;
 int num_sms();   // of the device current at the first call
-int tile_shape(int K, int n, const int *nx, const int *ny);
+int tile_shape(int K, int n, const int *nx, const int *ny, bool multi);
 // Blocks of one grid at that shape.
 int tile_blocks(int K, int shape, int nx, int ny);
 // K steps (1..TILE_MAX_K): what launch_fused with scaled rotations gives at

@@ -47,14 +47,18 @@ struct TileGrid {
     float te_end, te_mid, to_a, to_b;
 };
 
-template <int W>
+template <int R, int W>
 struct TileShared {
+    // tables of the rows above and below a warp: in registers, but for the shapes
+    // of 8 rows and more than 8 warps (168 registers: they would spill)
+    static constexpr bool TABS = R == 8 && W > 8;
     float4 recv[SWEEPS][CLASSES];   // as EdgeTab in scaled.cuh
     float4 hrow[CLASSES];
     float2 lohi[SWEEPS];
     float h[13];
     // first and last row of each warp (re, im), two buffers
     float4 ex[2][W][2][2][32];
+    float4 tab[TABS ? W : 1][2][2][32];
 };
 
 // What every step of a tile needs besides the rows.
@@ -66,7 +70,7 @@ struct TileCtx {
 template <int R, int W, bool EDGE>
 __device__ __forceinline__ void tile_steps(Frag (&st)[R], const float4 (&tg)[R + 2],
                                            const float4 (&tv)[R + 2], const TileCtx &c,
-                                           TileShared<W> &sh)
+                                           TileShared<R, W> &sh)
 {
     const int K = c.K;
     auto even_x = [&](int k) {
@@ -124,10 +128,16 @@ __device__ __forceinline__ void tile_steps(Frag (&st)[R], const float4 (&tg)[R +
             bot.im = ex[c.warp + 1][0][1][c.lane];
         }
         odd_y(2 * k, c.to_a);
-        phase4<true>(top, tg[0], tv[0]);
+        auto phase_out = [&](Frag &f, int i) {   // the row above (0) or below (1)
+            if constexpr (TileShared<R, W>::TABS)
+                phase4<true>(f, sh.tab[c.warp][i][0][c.lane], sh.tab[c.warp][i][1][c.lane]);
+            else
+                phase4<true>(f, tg[i * (R + 1)], tv[i * (R + 1)]);
+        };
+        phase_out(top, 0);
 #pragma unroll
         for (int r = 0; r < R; ++r) phase4<true>(st[r], tg[r + 1], tv[r + 1]);
-        phase4<true>(bot, tg[R + 1], tv[R + 1]);
+        phase_out(bot, 1);
         odd_y(2 * k + 1, c.to_b);
         if (k < K - 1) {
             odd_x(2 * k + 1);
@@ -144,7 +154,7 @@ __device__ __forceinline__ void tile_steps(Frag (&st)[R], const float4 (&tg)[R +
 // K steps of the tile (sx, ty) of grid g: ed has the edge values at depth K.
 template <int R, int W>
 __device__ __forceinline__ void run_tile(const TileGrid &g, const ScaledEdge *ed, int K, int sx,
-                                         int ty, TileShared<W> &sh)
+                                         int ty, TileShared<R, W> &sh)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int halo = depth_halo(K);
@@ -200,6 +210,12 @@ __device__ __forceinline__ void run_tile(const TileGrid &g, const ScaledEdge *ed
         }
         tg[r + 1] = in ? *reinterpret_cast<const float4 *>(g.pg + o) : z;
         tv[r + 1] = in ? *reinterpret_cast<const float4 *>(g.ps + o) : z;
+        if constexpr (TileShared<R, W>::TABS) {   // (read by the lane that writes it)
+            if (r < 0 || r == R) {
+                sh.tab[warp][r == R][0][lane] = tg[r + 1];
+                sh.tab[warp][r == R][1][lane] = tv[r + 1];
+            }
+        }
     }
     // a lane across the grid's last column: its further columns are padding
     if (xg < g.nx && xg + 4 > g.nx) {
@@ -244,7 +260,7 @@ tile_kernel(const TileGrid g, const __grid_constant__ ScaledEdge ed, int K, int 
 {
     extern __shared__ __align__(16) unsigned char smem[];
     run_tile<R, W>(g, &ed, K, blockIdx.x % n_strips, blockIdx.x / n_strips,
-                   *reinterpret_cast<TileShared<W> *>(smem));
+                   *reinterpret_cast<TileShared<R, W> *>(smem));
 }
 
 // Many grids in one launch: tab[i].begin is grid i's first block.
@@ -269,7 +285,7 @@ tile_multi_kernel(const EpochEntry *__restrict__ tab, int n_grids, int K, int fl
     const TileGrid g = {d->re[cur], d->im[cur], d->pg, d->ps, d->re[cur ^ 1], d->im[cur ^ 1],
                         d->nx, d->ny, d->pitch, c.te_end, c.te_mid, c.to_a, c.to_b};
     const int strips = strip_count(d->nx, depth_halo(K)), b = (int)(blockIdx.x - e.begin);
-    run_tile<R, W>(g, &c.edge, K, b % strips, b / strips, *reinterpret_cast<TileShared<W> *>(smem));
+    run_tile<R, W>(g, &c.edge, K, b % strips, b / strips, *reinterpret_cast<TileShared<R, W> *>(smem));
 }
 
 template <int R, int W>
@@ -278,7 +294,7 @@ cudaError_t launch_one(int K, const TileLaunch &a, int blocks, int strips, cudaS
     const ScaledCoef &c = *a.sc;
     const TileGrid g = {a.in_re, a.in_im, a.pg, a.ps, a.out_re, a.out_im, a.nx, a.ny, a.pitch,
                         c.te_end, c.te_mid, c.to_a, c.to_b};
-    constexpr int smem = (int)sizeof(TileShared<W>);
+    constexpr int smem = (int)sizeof(TileShared<R, W>);
     static const cudaError_t attr = cudaFuncSetAttribute(
         tile_kernel<R, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (attr != cudaSuccess) return attr;
@@ -292,7 +308,7 @@ cudaError_t prepare_multi()
 {
     static const cudaError_t attr =
         cudaFuncSetAttribute(tile_multi_kernel<R, W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(TileShared<W>));
+                             (int)sizeof(TileShared<R, W>));
     return attr;
 }
 
@@ -301,7 +317,7 @@ cudaError_t launch_many(int K, const EpochEntry *tab, int n, int blocks, int fli
 {
     cudaError_t e = prepare_multi<R, W>();
     if (e == cudaSuccess)
-        e = launch_pdl(tile_multi_kernel<R, W>, blocks, 32 * W, sizeof(TileShared<W>), st, tab, n,
+        e = launch_pdl(tile_multi_kernel<R, W>, blocks, 32 * W, sizeof(TileShared<R, W>), st, tab, n,
                        K, flip);
     count_launches(1);
     return e;
@@ -311,7 +327,7 @@ cudaError_t launch_many(int K, const EpochEntry *tab, int n, int blocks, int fli
 struct Shape {
     int r, w;
 };
-constexpr Shape shapes[TILE_SHAPES] = {{4, 8}, {4, 10}, {8, 8}};
+constexpr Shape shapes[TILE_SHAPES] = {{4, 8}, {4, 10}, {8, 8}, {8, 10}};
 
 int64_t tiles_of(int K, const Shape &s, int nx, int ny)
 {
@@ -340,8 +356,8 @@ int tile_blocks(int K, int shape, int nx, int ny) { return (int)tiles_of(K, shap
 
 // Tiles or warp streams?  Tiles of 64 rows in at most K rounds of one block
 // per SM.  Measured, one launch at depth 4 (us), tiles against streams: 256^2
-// 6.0 / 14.9, 512^2 6.7 / 14.7, 1001 x 777 8.3 / 19.4, 1024^2 14.4 / 22.2 (2
-// rounds), 1500^2 22.4 / 28.6 (3), 2048^2 43 / 31.9 (6).  A tile recomputes its
+// 6.0 / 14.9, 512^2 6.7 / 14.7, 1001 x 777 8.3 / 19.4, 1024^2 12.2 / 22.2 (1
+// round of 80 rows), 1500^2 22.4 / 28.6 (3), 2048^2 43 / 31.9 (6).  A tile recomputes its
 // halo (at depth 4 three quarters of its rows and 7/8 of its columns are
 // stored), so once the SMs are full the streams win; at a smaller depth sooner,
 // since a launch has less work to set against its loads (depth 1: 1024^2 7.4 /
@@ -350,18 +366,22 @@ int tile_blocks(int K, int shape, int nx, int ny) { return (int)tiles_of(K, shap
 //
 // Which shape?  The least of time = 1.3 + rounds (g + s K) us, fitted to
 // launches from 128^2 to 1500^2 at depths 1 to 4; two blocks of the first shape
-// share an SM, a second round costs it half.
-int tile_shape(int K, int n, const int *nx, const int *ny)
+// share an SM, a second round costs it half.  The last shape, 80 rows, has three
+// warps on two of the schedulers and is worth it where it makes one round of what
+// tiles of 64 rows make two: 1024^2 at depth 4 14.9 -> 12.2 us (13.2 with 12
+// warps), 1000^2 14.4 -> 12.1, 1024^2 at depth 3 12.3 -> 10.4.
+int tile_shape(int K, int n, const int *nx, const int *ny, bool multi)
 {
     if (K < 1 || K > TILE_MAX_K) return -1;
-    static const double g[TILE_SHAPES] = {1.1, 1.1, 1.8}, s[TILE_SHAPES] = {0.9, 1.06, 1.28};
+    static const double g[TILE_SHAPES] = {1.1, 1.1, 1.8, 3.65}, s[TILE_SHAPES] = {0.9, 1.06, 1.28, 1.8};
     const int64_t sms = num_sms();
     int best = -1;
     double best_us = 0.0;
-    for (int i = TILE_SHAPES - 1; i >= 0; --i) {   // the largest tile first: it decides
+    for (int i : {2, 3, 1, 0}) {   // tiles of 64 rows first: they decide
+        if (i == 3 && multi) continue;   // (spills in that kernel)
         int64_t tiles = 0;
         for (int k = 0; k < n; ++k) tiles += tiles_of(K, shapes[i], nx[k], ny[k]);
-        if (i == TILE_SHAPES - 1 && tiles > K * sms) return -1;
+        if (i == 2 && tiles > K * sms) return -1;
         double rounds = (double)((tiles + sms - 1) / sms);
         if (i == 0 && rounds > 1.0) rounds *= 0.75;
         const double us = rounds * (g[i] + s[i] * K);
@@ -382,6 +402,7 @@ cudaError_t launch_tile(int K, int shape, const TileLaunch &a, cudaStream_t st)
     case 0: return launch_one<4, 8>(K, a, blocks, strips, st);
     case 1: return launch_one<4, 10>(K, a, blocks, strips, st);
     case 2: return launch_one<8, 8>(K, a, blocks, strips, st);
+    case 3: return launch_one<8, 10>(K, a, blocks, strips, st);
     default: return cudaErrorInvalidValue;
     }
 }

@@ -41,6 +41,14 @@ def test_tiles_equal_streams(nx, ny, K):
     assert rel_l2(*out[0], ore, oim) < 2e-6     # as derived in test_gpu_scaled.py
 
 
+# grids that tiles of 80 rows cover in one round of one block per SM where tiles
+# of 64 rows take two: the fewest and the most rows of that range, ragged sides
+@pytest.mark.parametrize("nx,ny", [(1024, 785), (1023, 1039), (1017, 1040), (897, 911)])
+@pytest.mark.parametrize("K", [3, 4])
+def test_tall_tiles_equal_streams(nx, ny, K):
+    test_tiles_equal_streams(nx, ny, K)
+
+
 def test_captured_evolution():
     """Dependent launches inside a CUDA graph keep their order: three replays
     of a captured evolution equal three evolutions."""
