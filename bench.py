@@ -494,9 +494,16 @@ PLAIN_BYTES = {"f32": 8 * 16 + 24, "f64": 16 * 16 + 48}   # 8 sweeps + the phase
 
 
 def fp64_merged_bytes(T: int) -> float:
-    """ts_evolve on an FP64 grid: 6 T + 2 sweeps (32 B/site each) and T phases
+    """ts_evolve on an FP64 grid in merged sweeps (3-D, drive, |theta| > pi/8,
+    fewer than 1024 sites): 6 T + 2 sweeps (32 B/site each) and T phases
     (48 B/site) for T steps, per site-step."""
     return ((6 * T + 2) * 32 + T * 48) / T
+
+
+def fp64_fused_bytes(T: int) -> float:
+    """ts_evolve on every other FP64 grid: two sweeps, T fused steps (48 B/site
+    each) and the closing sweep, per site-step."""
+    return (3 * 32 + T * 48) / T
 
 
 def k_sweep(args, hbm_peak, sizes=(8192, 16384), depths=range(1, 9), reps=3):
@@ -543,7 +550,7 @@ def k_sweep(args, hbm_peak, sizes=(8192, 16384), depths=range(1, 9), reps=3):
                     paths.append(("plain", None, g.evolve_plain, 1, PLAIN_BYTES["f32"]))
                 else:
                     paths.append(("plain", None, g.evolve_plain, 1, PLAIN_BYTES["f64"]))
-                    paths.append(("evolve", None, g.evolve, 1, fp64_merged_bytes(T)))
+                    paths.append(("evolve", None, g.evolve, 1, fp64_fused_bytes(T)))
                 for path, K, fn, count, bps in paths:
                     ms = timed(fn, count)
                     rate = sites * T / (ms / 1e3)

@@ -884,8 +884,8 @@ ts_status plain_run(ts_grid *g, int64_t steps, const ts::RotCoef &c, const void 
 
 
 
-// FP64 grids (ts_evolve): second-order substeps one sweep per launch, with
-// the sweeps merged where two substeps meet.  X, Y (and Z) factors act on
+// FP64 grids that fused64_ok leaves out: second-order substeps one sweep per
+// launch, with the sweeps merged where two substeps meet.  X, Y (and Z) factors act on
 // different coordinates and commute, and two factors of one family add
 // their angles, so the mirror half of substep i and the first half of
 // substep i + 1,
@@ -989,7 +989,7 @@ ts_status fused_run(ts_grid *g, int64_t steps, int K, double theta, const CUtens
         a.err = g->err;
         cudaError_t e;
         const int nx = a.nx, ny = a.ny;
-        const int shape = scaled && !drive_adt ? ts::tile_shape(k, 1, &nx, &ny) : -1;
+        const int shape = scaled && !drive_adt ? ts::tile_shape(k, 1, &nx, &ny, false) : -1;
         if (shape >= 0) {
             const ts::TileLaunch t = {(const float *)g->re(), (const float *)g->im(),
                                       (const float *)pg,

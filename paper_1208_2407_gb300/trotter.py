@@ -449,8 +449,9 @@ class Grid:
 
     def evolve(self, steps: int, K: int = 0, stream=None):
         """`steps` steps (ts_evolve).  FP32 grids: the fused kernel at depth K
-        (0: the library's default).  FP64 grids: one sweep per launch with
-        the sweeps merged where steps meet (K must be 0).  Async."""
+        (0: the library's default).  FP64 grids: one fused step per launch,
+        or one sweep per launch with the sweeps merged where steps meet (K
+        must be 0).  Async."""
         ts_evolve(self.handle, int(steps), int(K), stream or current_stream_ptr())
 
     def evolve_plain(self, steps: int, stream=None):
