@@ -354,15 +354,17 @@ int num_sms()
 
 int tile_blocks(int K, int shape, int nx, int ny) { return (int)tiles_of(K, shapes[shape], nx, ny); }
 
-// Tiles or warp streams?  Tiles of 64 rows in at most K rounds of one block
-// per SM.  Measured, one launch at depth 4 (us), tiles against streams: 256^2
-// 6.0 / 14.9, 512^2 6.7 / 14.7, 1001 x 777 8.3 / 19.4, 1024^2 12.2 / 22.2 (1
-// round of 80 rows), 1500^2 22.4 / 28.6 (3), 2048^2 43 / 31.9 (6).  A tile recomputes its
-// halo (at depth 4 three quarters of its rows and 7/8 of its columns are
-// stored), so once the SMs are full the streams win; at a smaller depth sooner,
-// since a launch has less work to set against its loads (depth 1: 1024^2 7.4 /
-// 7.3, 1500^2 12.4 / 10.0; depth 2: 1024^2 8.7 / 11.2, 1500^2 15.0 / 15.5;
-// depth 3: 1500^2 18.6 / 20.9, 2048^2 32.5 / 24.8).
+// Tiles or warp streams?  Tiles of 64 rows in at most 1, 2, 2 and 3 rounds of one
+// block per SM at depths 1 to 4.  A tile recomputes its halo (at depth 4 three
+// quarters of its rows and 7/8 of its columns are stored), so once the SMs are full
+// the streams win; at a smaller depth sooner, since a launch has less work to set
+// against its loads.  Measured, us per launch, tiles / streams:
+//   depth 4: 512^2 6.7 / 14.7, 1024^2 12.2 / 19.1 (1 round of 80 rows), 1300^2 21.1 /
+//     22.4 (3), 1500^2 22.2 / 25.0 (3), 1600^2 28.2 / 26.2 (4), 2048^2 43 / 33 (6);
+//   depth 3: 1300^2 13.7 / 16.6 (2), 1400^2 18.6 / 18.1 (3), 1600^2 23.5 / 19.6 (4);
+//   depth 2: 1400^2 11.7 / 13.9 (2), 1500^2 14.8 / 15.6 and 1024 x 2048 17.3 / 14.8
+//     (3), 1700^2 18.8 / 17.6 (4);
+//   depth 1: 900^2 4.9 / 6.4 (1), 1024^2 7.2 / 7.2 and 1500^2 10.6 / 10.1 (2 and 3).
 //
 // Which shape?  The least of time = 1.3 + rounds (g + s K) us, fitted to
 // launches from 128^2 to 1500^2 at depths 1 to 4; two blocks of the first shape
@@ -381,7 +383,7 @@ int tile_shape(int K, int n, const int *nx, const int *ny, bool multi)
         if (i == 3 && multi) continue;   // (spills in that kernel)
         int64_t tiles = 0;
         for (int k = 0; k < n; ++k) tiles += tiles_of(K, shapes[i], nx[k], ny[k]);
-        if (i == 2 && tiles > K * sms) return -1;
+        if (i == 2 && tiles > (K + 2) / 2 * sms) return -1;
         double rounds = (double)((tiles + sms - 1) / sms);
         if (i == 0 && rounds > 1.0) rounds *= 0.75;
         const double us = rounds * (g[i] + s[i] * K);
