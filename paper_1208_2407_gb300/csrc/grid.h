@@ -20,10 +20,10 @@ struct RotCoef {
 RotCoef rot_coef(double theta);
 
 // Scaled rotations (fused.cu) serve |theta| <= this, per substep.  A launch
-// takes its scale out by a -= h a, and the rounding of h (ulp(h) / 2, the same
-// at every site) is what they add to the norm: under 1e-9 per step here, where
-// h < 1/8 at depth 4.  The tangents and the edge ratios stay far from their
-// poles.  Larger angles take the lifting form.
+// takes its scale out by a -= h a; the rounding of h is what they add to the
+// norm, and scaled_coef keeps it under 5e-10 per step here, where h < 1/8 at
+// depth 4.  The tangents and the edge ratios stay far from their poles.  Larger
+// angles take the lifting form.
 constexpr double SCALED_MAX_THETA = 0.075;
 // Coefficients of a launch of K substeps with kinetic half angles sub[i].
 void scaled_coef(const double *sub, int K, int64_t nx, int64_t ny, int64_t nz, ScaledCoef &c);
