@@ -238,6 +238,15 @@ __device__ __forceinline__ int lane_class(int xg, int nx)
     return xg < 0 || xg >= nx ? 0 : L && R ? 4 : L && B ? 6 : L ? 2 : R ? 3 : B ? 5 : 1;
 }
 
+// Zeros for the columns past the grid's last one in a lane that starts on the
+// grid (xg < nx): a row's padding holds anything.
+__device__ __forceinline__ void cut_padding(float4 &v, int xg, int nx)
+{
+    if (xg + 1 >= nx) v.y = 0.f;
+    if (xg + 2 >= nx) v.z = 0.f;
+    if (xg + 3 >= nx) v.w = 0.f;
+}
+
 // the entries of a 3 x 3 edge table (rows by columns) for one row of the lane
 __device__ __forceinline__ float4 edge4(const float *tab, int row, int ny, unsigned cols)
 {

@@ -210,24 +210,26 @@ __device__ __forceinline__ void run_tile(const TileGrid &g, const ScaledEdge *ed
         }
         tg[r + 1] = in ? *reinterpret_cast<const float4 *>(g.pg + o) : z;
         tv[r + 1] = in ? *reinterpret_cast<const float4 *>(g.ps + o) : z;
-        if constexpr (TileShared<R, W>::TABS) {   // (read by the lane that writes it)
-            if (r < 0 || r == R) {
-                sh.tab[warp][r == R][0][lane] = tg[r + 1];
-                sh.tab[warp][r == R][1][lane] = tv[r + 1];
-            }
-        }
     }
-    // a lane across the grid's last column: its further columns are padding
+    // a lane across the grid's last column: its further columns are padding,
+    // which holds anything, in the table too (NaN there would reach the last
+    // column: a pair that the grid's edge cuts takes 0 times its partner)
     if (xg < g.nx && xg + 4 > g.nx) {
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            auto cut = [&](float4 &v) {
-                if (xg + 1 >= g.nx) v.y = 0.f;
-                if (xg + 2 >= g.nx) v.z = 0.f;
-                v.w = 0.f;
-            };
-            cut(st[r].re);
-            cut(st[r].im);
+        for (int r = -1; r <= R; ++r) {
+            if (r >= 0 && r < R) {
+                cut_padding(st[r].re, xg, g.nx);
+                cut_padding(st[r].im, xg, g.nx);
+            }
+            cut_padding(tg[r + 1], xg, g.nx);
+            cut_padding(tv[r + 1], xg, g.nx);
+        }
+    }
+    if constexpr (TileShared<R, W>::TABS) {   // (read by the lane that writes it)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            sh.tab[warp][i][0][lane] = tg[i * (R + 1)];
+            sh.tab[warp][i][1][lane] = tv[i * (R + 1)];
         }
     }
     const bool edge = y0 <= 0 || y0 + R * W >= g.ny;   // the same for the whole block

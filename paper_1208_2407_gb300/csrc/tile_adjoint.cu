@@ -229,10 +229,7 @@ tile_adjoint_kernel(const TileAdjoint p, const __grid_constant__ ScaledEdge ed,
         const int64_t o = in ? (int64_t)y * p.pitch + xg : 0;
         auto load = [&](const float *plane) {
             float4 v = in ? *reinterpret_cast<const float4 *>(plane + o) : z;
-            // columns past the last one are padding
-            if (xg + 1 >= p.nx) v.y = 0.f;
-            if (xg + 2 >= p.nx) v.z = 0.f;
-            if (xg + 3 >= p.nx) v.w = 0.f;
+            cut_padding(v, xg, p.nx);
             return v;
         };
         st[r].a.re = load(p.in[0]);
@@ -243,6 +240,13 @@ tile_adjoint_kernel(const TileAdjoint p, const __grid_constant__ ScaledEdge ed,
         cp_async16_zfill(&sh.tab[R * warp + r][1][lane], p.ps + o, in);
     }
     cp_async_commit();
+    // the table's padding, as in tile.cu; a lane reads only the columns that it
+    // (in this or a neighbouring warp) has copied
+    if (xg < p.nx && xg + 4 > p.nx) {
+        cp_async_wait_all();
+        for (int r = 0; r < R; ++r)
+            for (int i = 0; i < 2; ++i) cut_padding(sh.tab[R * warp + r][i][lane], xg, p.nx);
+    }
 
     const bool edge = y0 <= 0 || y0 + ROWS >= p.ny;   // the same for the whole block
     if (edge)
