@@ -66,6 +66,7 @@
 #include "ffloat.cuh"
 #include "internal.h"
 #include "mbar.cuh"
+#include "per_device.h"
 #include "scaled.cuh"
 
 // This file is compiled in parts (build.py), so that its kernels build in
@@ -78,8 +79,7 @@
 namespace ts {
 
 // Resident blocks per SM and SM count of a kernel at its dynamic shared
-// memory size, set up once per kernel (the first caller's function-local
-// static initialisation, which C++ runs exactly once even when threads race).
+// memory size, set up once per kernel and device.
 struct Occupancy {
     cudaError_t err;
     int blocks_per_sm, num_sms;
@@ -1805,7 +1805,9 @@ cudaError_t launch3_k(const FusedLaunch &a, int nz, cudaStream_t st)
 {
     using C = CfgM<1, 6, SC>;
     constexpr int NW = C::WPC, VZ = 2 * NW - 4;
-    static const Occupancy occ = occupancy_of(fused3d_kernel<1, SC>, NW * 32, C::SMEM);
+    static PerDevice<Occupancy> per_device;
+    const Occupancy &occ =
+        per_device.get([] { return occupancy_of(fused3d_kernel<1, SC>, NW * 32, C::SMEM); });
     if (occ.err != cudaSuccess) return occ.err;
     KParams p = {};
     p.out_re = a.out_re;
@@ -1856,7 +1858,9 @@ template <int K, int MODE, bool SC>
 cudaError_t launch_k(const FusedLaunch &a, cudaStream_t st)
 {
     using C = CfgM<K, MODE, SC>;
-    static const Occupancy occ = occupancy_of(fused_kernel<K, MODE, SC>, C::WPC * 32, C::SMEM);
+    static PerDevice<Occupancy> per_device;
+    const Occupancy &occ =
+        per_device.get([] { return occupancy_of(fused_kernel<K, MODE, SC>, C::WPC * 32, C::SMEM); });
     if (occ.err != cudaSuccess) return occ.err;
     const int blocks_per_sm = occ.blocks_per_sm, num_sms = occ.num_sms;
     KParams p;
@@ -1913,8 +1917,8 @@ template <int K, bool SC>
 const Occupancy &multi_occupancy()
 {
     using C = CfgM<K, MULTI_MODE<SC>, SC>;
-    static const Occupancy occ = occupancy_of(fused_multi_kernel<K, SC>, C::WPC * 32, C::SMEM);
-    return occ;
+    static PerDevice<Occupancy> occ;
+    return occ.get([] { return occupancy_of(fused_multi_kernel<K, SC>, C::WPC * 32, C::SMEM); });
 }
 
 template <int K, bool SC>

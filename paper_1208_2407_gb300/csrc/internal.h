@@ -217,7 +217,7 @@ struct TileLaunch {
 // or -1 where the warp streams are faster (or K > TILE_MAX_K).  multi: for
 // launch_tile_multi.
 constexpr int TILE_SHAPES = 4;
-int num_sms();   // of the device current at the first call
+int num_sms();   // of the current device
 int tile_shape(int K, int n, const int *nx, const int *ny, bool multi);
 // Blocks of one grid at that shape.
 int tile_blocks(int K, int shape, int nx, int ny);

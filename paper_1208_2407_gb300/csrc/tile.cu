@@ -30,6 +30,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "per_device.h"
 #include "scaled.cuh"
 
 namespace ts {
@@ -297,10 +298,13 @@ cudaError_t launch_one(int K, const TileLaunch &a, int blocks, int strips, cudaS
     const TileGrid g = {a.in_re, a.in_im, a.pg, a.ps, a.out_re, a.out_im, a.nx, a.ny, a.pitch,
                         c.te_end, c.te_mid, c.to_a, c.to_b};
     constexpr int smem = (int)sizeof(TileShared<R, W>);
-    static const cudaError_t attr = cudaFuncSetAttribute(
-        tile_kernel<R, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (attr != cudaSuccess) return attr;
-    cudaError_t e = launch_pdl(tile_kernel<R, W>, blocks, 32 * W, smem, st, g, c.edge, K, strips);
+    static PerDevice<cudaError_t> attr;
+    cudaError_t e = attr.get([] {
+        return cudaFuncSetAttribute(tile_kernel<R, W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    smem);
+    });
+    if (e != cudaSuccess) return e;
+    e = launch_pdl(tile_kernel<R, W>, blocks, 32 * W, smem, st, g, c.edge, K, strips);
     count_launches(1);
     return e;
 }
@@ -308,10 +312,12 @@ cudaError_t launch_one(int K, const TileLaunch &a, int blocks, int strips, cudaS
 template <int R, int W>
 cudaError_t prepare_multi()
 {
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(tile_multi_kernel<R, W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(TileShared<R, W>));
-    return attr;
+    static PerDevice<cudaError_t> attr;
+    return attr.get([] {
+        return cudaFuncSetAttribute(tile_multi_kernel<R, W>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)sizeof(TileShared<R, W>));
+    });
 }
 
 template <int R, int W>
@@ -344,14 +350,14 @@ int64_t tiles_of(int K, const Shape &s, int nx, int ny)
 
 int num_sms()
 {
-    static const int n = [] {
+    static PerDevice<int> n;
+    return n.get([] {
         int dev = 0, v = 0;
         if (cudaGetDevice(&dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
             v = 1;
         return v;
-    }();
-    return n;
+    });
 }
 
 int tile_blocks(int K, int shape, int nx, int ny) { return (int)tiles_of(K, shapes[shape], nx, ny); }

@@ -15,6 +15,7 @@
 #include "common.cuh"
 #include "ffloat.cuh"
 #include "internal.h"
+#include "per_device.h"
 #include "scaled.cuh"
 
 namespace ts {
@@ -333,12 +334,15 @@ bool tile_adjoint_serves(int K, int nx, int ny)
 cudaError_t launch_tile_adjoint(int K, const TileAdjoint &p, const ScaledCoef &c, cudaStream_t st)
 {
     if (K < 1 || K > MAX_K) return cudaErrorInvalidValue;
-    static const cudaError_t attr = cudaFuncSetAttribute(
-        tile_adjoint_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared));
-    if (attr != cudaSuccess) return attr;
-    const cudaError_t e =
-        launch_pdl(tile_adjoint_kernel, tile_blocks_of(K, p.nx, p.ny), 32 * W, sizeof(Shared),
-                   st, p, c.edge, c.te_end, c.te_mid, c.to_a, c.to_b, K,
+    static PerDevice<cudaError_t> attr;
+    cudaError_t e = attr.get([] {
+        return cudaFuncSetAttribute(tile_adjoint_kernel,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)sizeof(Shared));
+    });
+    if (e != cudaSuccess) return e;
+    e = launch_pdl(tile_adjoint_kernel, tile_blocks_of(K, p.nx, p.ny), 32 * W, sizeof(Shared), st, p,
+                   c.edge, c.te_end, c.te_mid, c.to_a, c.to_b, K,
                    strip_count(p.nx, depth_halo(K)));
     count_launches(1);
     return e;
