@@ -372,7 +372,8 @@ cudaError_t evolve_multi(ts_grid *const *gs, const int64_t *steps, int n, int K,
     if (e != cudaSuccess) return e;
     std::vector<EpochEntry> h;
     std::vector<int> hx, hy;
-    auto run = [&](int depth, const std::vector<int> &idx, int64_t launches) -> cudaError_t {
+    auto run_form = [&](int depth, const std::vector<int> &idx, int64_t launches,
+                        bool scaled) -> cudaError_t {
         h.clear();
         hx.clear();
         hy.clear();
@@ -390,6 +391,16 @@ cudaError_t evolve_multi(ts_grid *const *gs, const int64_t *steps, int n, int K,
                                      gs[idx[0]]->err, st);
         if (err == cudaSuccess && (launches & 1))
             for (int i : idx) gs[i]->cur ^= 1;
+        return err;
+    };
+    // each grid's launches at this depth, in the form that it takes alone
+    auto run = [&](int depth, const std::vector<int> &idx, int64_t launches) -> cudaError_t {
+        std::vector<int> form[2];
+        for (int i : idx)
+            form[scaled && runs_scaled(gs[i]->theta, depth, gs[i]->L.nx, gs[i]->L.ny)].push_back(i);
+        cudaError_t err = cudaSuccess;
+        for (int f = 0; f < 2 && err == cudaSuccess; ++f)
+            if (!form[f].empty()) err = run_form(depth, form[f], launches, f);
         return err;
     };
     int64_t done = 0;
@@ -968,12 +979,13 @@ ts_status fused_run(ts_grid *g, int64_t steps, int K, double theta, const CUtens
     int64_t left = steps;
     while (left > 0) {
         const int k = (int)(left >= K ? K : left);
-        if (scaled && k != sc_k) {
+        const bool sc_form = drive_adt ? scaled : ts::runs_scaled(theta, k, g->L.nx, g->rows());
+        if (sc_form && k != sc_k) {
             ts::scaled_coef(sub, k, g->L.nx, g->rows(), 1, sc);
             sc_k = k;
         }
         ts::FusedLaunch a;
-        a.sc = scaled ? &sc : nullptr;
+        a.sc = sc_form ? &sc : nullptr;
         a.tm_state = &g->tm_state[g->cur];
         a.tm_phase = tm;
         a.out_re = (float *)g->re_other();
@@ -989,7 +1001,7 @@ ts_status fused_run(ts_grid *g, int64_t steps, int K, double theta, const CUtens
         a.err = g->err;
         cudaError_t e;
         const int nx = a.nx, ny = a.ny;
-        const int shape = scaled && !drive_adt ? ts::tile_shape(k, 1, &nx, &ny, false) : -1;
+        const int shape = sc_form && !drive_adt ? ts::tile_shape(k, 1, &nx, &ny, false) : -1;
         if (shape >= 0) {
             const ts::TileLaunch t = {(const float *)g->re(), (const float *)g->im(),
                                       (const float *)pg,

@@ -174,11 +174,23 @@ constexpr uint64_t WAIT_LIMIT_NS = 2000000000ull;    // 2 s per wait
 // each in the phase ring, (re, im) of each in the state ring.
 __host__ __device__ constexpr int phase_planes(int mode)
 {
-    return mode == 3 ? 3 : mode == 6 ? 4 : 2;
+    return mode == 3 || mode == 9 ? 3 : mode == 6 ? 4 : 2;
 }
 // Planes of a state-ring slot: (re, im); the backward adjoint steps (MODE 5)
 // carry two states, the forward state psi and the costate lambda.
 __host__ __device__ constexpr int state_planes(int mode) { return mode == 5 || mode == 6 ? 4 : 2; }
+
+// MODE 8 and 9 are MODE 0 and 3 for long row ranges in the lifting form.  They work
+// through the pipeline's fill: leaving out the stages that have nothing to do yet
+// costs registers there (depth 2: 138 or 128, depth 3: 168 and spills or 165), which
+// short ranges win back and long ones do not (us per step without and with it: depth
+// 2 2048^2 11.0 and 10.7, 8192^2 127.5 and 129.5, 16384^2 530 and 539; depth 3
+// 2048^2 9.3 and 8.9, 4096^2 25.2 and 25.5, 8192^2 88.8 and 92.0, 16384^2 349 and
+// 373; driven, depth 3, 2500^2 19.5 and 20.7, 4096^2 39.0 and 41.0).
+__host__ __device__ constexpr bool skips_fill(int mode) { return mode != 8 && mode != 9; }
+
+// ... and their strips may start left of column 0 (KParams::x_shift).
+__host__ __device__ constexpr bool can_shift(int K, int mode) { return mode == 8 && K <= 2; }
 
 // __launch_bounds__ minimum resident blocks of the single-grid kernel; the
 // backward adjoint steps (MODE 5) carry two states and are not held to the
@@ -286,6 +298,7 @@ struct KParams {
     int64_t units;
     int total_warps;
     int strip_warps;         // > 0: warps per strip of the strip-aligned split
+    int x_shift;             // strip s starts at column s valid - x_shift
     float t1, s1, g1, t2, s2;
     int *err;
     // MODE 5 (backward adjoint steps): the costate's output planes (out_re,
@@ -843,7 +856,7 @@ __device__ __forceinline__ void pipeline_step(const S (&cin)[2 * K], S (&cout)[2
         } else {
             const float4 sv = lds4(sp, 1, row, lane);
             phase4<C::PACKED>(X, lds4(sp, 0, row, lane), CONJ ? neg4(sv) : sv);
-            if constexpr (MODE == 3) drive4<C::PACKED>(X, lds4(sp, 2, row, lane), p.adt[k]);
+            if constexpr (MODE == 3 || MODE == 9) drive4<C::PACKED>(X, lds4(sp, 2, row, lane), p.adt[k]);
         }
     };
     // phase of step 0 on rows (y1, y1+1): rows 0 and 1 of slot j (without
@@ -859,7 +872,7 @@ __device__ __forceinline__ void pipeline_step(const S (&cin)[2 * K], S (&cout)[2
     for (int k = 1; k < K; ++k) {
         // while the pipeline fills, stage k has nothing to do: the first rows
         // that the segment's output needs of it come at row pair 2k - 1
-        if (!INTERIOR && j < 2 * k - 1) return;
+        if (skips_fill(MODE) && !INTERIOR && j < 2 * k - 1) return;
         YO(P, Q, y1, 2 * k - 1);          // Yo of step k-1, aligned on (y1, y1+1), y1 odd
         // X group between two phases: Xo, Xe(merged), Xo
         XO(P, 2 * k - 1);
@@ -893,7 +906,7 @@ __device__ __forceinline__ void pipeline_step(const S (&cin)[2 * K], S (&cout)[2
         }
     }
     // last step, second half: Yo aligned, Ye shifted, Xo, Xe
-    if (!INTERIOR && K > 1 && j < 2 * K - 1) return;
+    if (skips_fill(MODE) && !INTERIOR && K > 1 && j < 2 * K - 1) return;
     YO(P, Q, y1, 2 * K - 1);
     O0 = cin[2 * K - 1];      // rows (y1-1, y1) = (yin-2K, yin-2K+1)
     O1 = P;
@@ -1232,7 +1245,8 @@ __device__ __forceinline__ bool row_pair(WarpRings &r, const Seg &s, const KPara
     bool okp = true;
     if constexpr (LATE_P)
         okp = __all_sync(FULL, mbar_wait(&r.bar_p[r.pos_p], r.par_p, WAIT_LIMIT_NS));
-    S O0 = zero_state<S>(), O1 = zero_state<S>();
+    S O0, O1;
+    if constexpr (skips_fill(MODE)) O0 = O1 = zero_state<S>();
     pipeline_step<K, INTERIOR, MODE, SC>(cin, cout, a, b, yin, j, r.ring_p, r.pos_p, r.ring_b,
                                      r.cnt_b, s.c, p, lane, s.own, O0, O1);
     if constexpr (MODE == 6) {
@@ -1356,7 +1370,8 @@ __device__ __forceinline__ bool run_segment(WarpRings &r, const CUtensorMap *tm_
     s.store_a = sl.store_a;
     s.store_b = sl.store_b;
     s.lane = lane;
-    s.XL = sx * VALID;                   // first loaded column (multiple of 4)
+    constexpr bool SHIFTS = can_shift(K, MODE);
+    s.XL = sx * VALID - (SHIFTS ? p.x_shift : 0);   // first loaded column (multiple of 4)
     s.xg = s.XL + 4 * lane;              // this lane's first column
     s.Y0 = 2 * q0;                       // output rows [Y0, Y1)
     s.Y1 = 2 * q1;
@@ -1379,7 +1394,7 @@ __device__ __forceinline__ bool run_segment(WarpRings &r, const CUtensorMap *tm_
         s.c.Eab = {e0 ? p.tab : 0.f, e0 ? p.sab : 0.f, e1 ? p.tab : 0.f, e1 ? p.sab : 0.f};
     }
     }
-    s.store_lane = (lane >= HALO / 4 || sx == 0) &&
+    s.store_lane = (lane >= HALO / 4 || (sx == 0 && (!SHIFTS || xg >= 0))) &&
                    (lane < 32 - HALO / 4 || s.XL + FUSED_BOX_COLS >= p.nx) && xg < p.nx;
     s.own = {s.Y0, s.Y1, xg, s.store_lane, SC ? col_places(xg, p.nx) : 0u, r.edge,
              SC ? lane_class(xg, p.nx) : 0, r.sums, r.gst};
@@ -1649,6 +1664,7 @@ __device__ __forceinline__ void multi_params(KParams &p, const GridDesc *d, int 
     p.err = err;
     p.n_pairs = (p.ny + 1) / 2;
     p.strip_warps = 0;
+    p.x_shift = 0;
 }
 
 template <int K, bool SC>
@@ -1869,7 +1885,15 @@ cudaError_t launch_k(const FusedLaunch &a, cudaStream_t st)
     p.nx = a.nx;
     p.ny = a.ny;
     p.pitch = a.pitch;
-    p.n_strips = strip_count(a.nx, C::HALO);
+    // At depths 1 and 2 strips that start at column 0 store from 16 bytes into a
+    // 32-byte sector on, so every strip boundary splits a sector between two
+    // warps; on grids far larger than L2 they meet there too late.  Strips that
+    // start 4 columns before the grid store whole sectors, at the price of the
+    // first one's (lifting form, us per step, shifted or not: depth 1 2048^2 19.3
+    // and 17.5, 6000^2 155.6 and 157.0, 16384^2 1287 and 1410; depth 2 16384^2 522 and
+    // 550 to 610).
+    p.x_shift = can_shift(K, MODE) && far_beyond_l2(a.nx, a.ny) ? C::HALO : 0;
+    p.n_strips = strip_count(a.nx, C::HALO, p.x_shift);
     p.n_pairs = (a.ny + 1) / 2;
     p.units = (int64_t)p.n_strips * p.n_pairs;
     int64_t cap = (int64_t)num_sms * blocks_per_sm * C::WPC;
@@ -1881,6 +1905,11 @@ cudaError_t launch_k(const FusedLaunch &a, cudaStream_t st)
     // and 71.9, 8192^2 281 and 264).
     if (SC && MODE == 0 && K <= 2 && 24.0 * a.nx * a.ny > (K == 1 ? 256e6 : 1e9))
         cap = std::min<int64_t>(cap, (int64_t)num_sms * (K == 1 ? 4 : 7));
+    // Driven in the lifting form at depth 3, three warps per scheduler take 1.4 times
+    // as long for a row pair as two (strip_warps_for counts on 1.27): with fewer than
+    // 13 row pairs each, two (2048^2, 12 and 8 warps per SM: 15.0 and 13.9 us per step).
+    if (!SC && (MODE == 3 || MODE == 9) && K == 3 && p.units < 13 * 12 * (int64_t)num_sms)
+        cap = std::min<int64_t>(cap, (int64_t)num_sms * 8);
     p.total_warps = (int)std::min(p.units, cap);
     p.strip_warps = 0;
     if (p.n_strips <= cap) {
@@ -1985,6 +2014,9 @@ TS_KERNEL(1, 0, false)
 TS_KERNEL(2, 0, false)
 TS_KERNEL(3, 0, false)
 TS_KERNEL(4, 0, false)
+TS_KERNEL(1, 8, false)
+TS_KERNEL(2, 8, false)
+TS_KERNEL(3, 8, false)
 #elif TS_FUSED_PART == 13
 TS_MULTI(1, false)
 TS_MULTI(2, false)
@@ -1995,6 +2027,7 @@ TS_KERNEL(1, 3, false)
 TS_KERNEL(2, 3, false)
 TS_KERNEL(3, 3, false)
 TS_KERNEL(4, 3, false)
+TS_KERNEL(3, 9, false)
 #elif TS_FUSED_PART == 15
 TS_KERNEL(5, 4, false)
 TS_KERNEL_3D(false)
@@ -2010,6 +2043,13 @@ TS_KERNEL(4, 5, false)
 
 cudaError_t launch_fused(int K, const FusedLaunch &a, cudaStream_t st)
 {
+    if (!a.sc && K <= 3 && far_beyond_l2(a.nx, a.ny)) {
+        switch (K) {
+        case 1: return launch_k<1, 8, false>(a, st);
+        case 2: return launch_k<2, 8, false>(a, st);
+        case 3: return launch_k<3, 8, false>(a, st);
+        }
+    }
     if (!a.sc) {
         switch (K) {
         case 1: return launch_k<1, 0, false>(a, st);
@@ -2179,7 +2219,10 @@ cudaError_t launch_fused_drive(int K, const FusedLaunch &a, cudaStream_t st)
     switch (K) {
     case 1: return a.sc ? launch_k<1, 3, true>(a, st) : launch_k<1, 3, false>(a, st);
     case 2: return a.sc ? launch_k<2, 3, true>(a, st) : launch_k<2, 3, false>(a, st);
-    case 3: return a.sc ? launch_k<3, 3, true>(a, st) : launch_k<3, 3, false>(a, st);
+    case 3:
+        return a.sc                              ? launch_k<3, 3, true>(a, st)
+               : (int64_t)a.nx * a.ny >= 4000000 ? launch_k<3, 9, false>(a, st)
+                                                 : launch_k<3, 3, false>(a, st);
     case 4: return a.sc ? launch_k<4, 3, true>(a, st) : launch_k<4, 3, false>(a, st);
     default: return cudaErrorInvalidValue;
     }

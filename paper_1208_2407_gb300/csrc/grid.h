@@ -1,6 +1,7 @@
 // The grid handle behind the opaque ts_grid of include/trotter.h (internal).
 #pragma once
 
+#include <cmath>
 #include <cstddef>
 #include <cstdint>
 #include <cuda.h>
@@ -25,6 +26,15 @@ RotCoef rot_coef(double theta);
 // depth 4.  The tangents and the edge ratios stay far from their poles.  Larger
 // angles take the lifting form.
 constexpr double SCALED_MAX_THETA = 0.075;
+// Whether a launch of K plain steps takes them.  Depth 2 on the largest grids does
+// not: its warps wait for HBM, and those of neighbouring strips drift apart and read
+// their shared columns twice, which the lifting form's slower, evener pace avoids
+// (us per step, scaled and lifting: 4096^2 32.0 and 34.1, 6000^2 79 and 66, 8192^2
+// 134 and 125, 16384^2 550 and 522).
+inline bool runs_scaled(double theta, int K, int64_t nx, int64_t ny)
+{
+    return std::fabs(theta) <= SCALED_MAX_THETA && !(K == 2 && far_beyond_l2(nx, ny));
+}
 // Coefficients of a launch of K substeps with kinetic half angles sub[i].
 void scaled_coef(const double *sub, int K, int64_t nx, int64_t ny, int64_t nz, ScaledCoef &c);
 }  // namespace ts

@@ -149,16 +149,19 @@ struct FusedLaunch {
 static_assert(sizeof(FusedLaunch::adt) / sizeof(float) == FUSED_MAX_K, "one a_n dt per step");
 constexpr int FUSED_BOX_COLS = 128;   // columns a warp strip loads (box width)
 // Strips over nx columns at a halo of `halo` columns: strip s loads columns
-// s valid .. s valid + 127, valid = 128 - 2 halo, and stores all but the halo;
-// the first stores its first columns and the last its last ones too, since
-// beyond the grid's edge there is nothing to be wrong about.
+// s valid - shift .. s valid - shift + 127, valid = 128 - 2 halo, and stores all
+// but the halo; the first stores its first columns and the last its last ones
+// too, since beyond the grid's edge there is nothing to be wrong about.  shift is
+// 0, or halo (launch_k in fused.cu).
 TS_HD constexpr int strip_valid(int halo) { return FUSED_BOX_COLS - 2 * halo; }
-TS_HD constexpr int strip_count(int64_t nx, int halo)
+TS_HD constexpr int strip_count(int64_t nx, int halo, int shift = 0)
 {
-    return nx <= FUSED_BOX_COLS
+    return nx + shift <= FUSED_BOX_COLS
                ? 1
-               : (int)((nx - 2 * halo + strip_valid(halo) - 1) / strip_valid(halo));
+               : (int)((nx + shift - 2 * halo + strip_valid(halo) - 1) / strip_valid(halo));
 }
+// A grid whose sweep over memory (24 bytes per site) passes L2 many times over.
+TS_HD constexpr bool far_beyond_l2(int64_t nx, int64_t ny) { return 24 * nx * ny > 800000000; }
 TS_HD constexpr int depth_halo(int K) { return (2 * K + 3) / 4 * 4; }   // of K steps, in whole lanes
 constexpr int FUSED_BOX_ROWS = 2;     // rows per pipeline slot (box height)
 cudaError_t launch_fused(int K, const FusedLaunch &a, cudaStream_t st);

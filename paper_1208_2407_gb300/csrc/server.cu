@@ -330,13 +330,16 @@ void ts_server::enqueue_epoch(std::unique_lock<std::mutex> &lk)
     // grids with scaled rotations, then those in the lifting form: each form
     // has its full launches and its remainder launches (one per distinct
     // depth r below the form's)
+    auto runs_scaled = [](const ReqP &q, int64_t depth) {
+        return q->scaled && ts::runs_scaled(q->r.theta, (int)depth, q->r.nx, q->r.ny);
+    };
     for (const bool scaled : {true, false}) {
         std::vector<ReqP> full;
         std::vector<std::vector<ReqP>> by_rem(K);
         for (auto &q : run_full)
-            if (q->scaled == scaled) full.push_back(q);
+            if (runs_scaled(q, depth(q->scaled)) == scaled) full.push_back(q);
         for (auto &q : run_rem)
-            if (q->scaled == scaled) by_rem[q->rem_left].push_back(q);
+            if (runs_scaled(q, q->rem_left) == scaled) by_rem[q->rem_left].push_back(q);
         if (!full.empty() && e == cudaSuccess) {
             ts::MultiPlan plan{};
             const int slot = upload(full, depth(scaled), scaled, plan);
