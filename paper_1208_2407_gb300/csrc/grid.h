@@ -65,6 +65,10 @@ struct ts_grid {
     double *partials, *result;
     int *err;
     cudaEvent_t host_copied;   // host-input copies done (created on first use)
+    // a batch whose grids take several kernels runs a group of them here, beside
+    // the caller's stream (created by the first such batch that this grid leads)
+    cudaStream_t side;
+    cudaEvent_t fork, join;
     unsigned char *readback;   // pinned: results and error word (taken on first use)
     bool tmaps_ok;
     CUtensorMap tm_state[2], tm_phase;   // (re, im) of pair 0 / 1; (gamma_V, s_V)
@@ -106,4 +110,12 @@ void grid_write_desc(ts_grid *g, cudaStream_t st);
 // together with the multi-grid kernel at depth K (api.cu).
 cudaError_t evolve_multi(ts_grid *const *gs, const int64_t *steps, int n, int K, bool scaled,
                          cudaStream_t st);
+// Launches of grids with scaled rotations and of grids in the lifting form run side
+// by side (on two streams) up to this many sites in all, where they leave parts of
+// the GPU idle; beyond that one after the other.  Half of the grids scaled, us per
+// step, in turn and side by side: 4 x 128^2 5.3 and 3.2, 4 x 512^2 7.1 and 5.4, 16 x
+// 512^2 14.0 and 13.1, 16 x 1024^2 31.0 and 31.3, 16 mixed sizes (13 M sites) 37.9
+// and 41.4.  (Planned for a part of the GPU each, they lost up to 45 %: registers
+// keep few warps of one kernel beside the other's.)
+constexpr double SIDE_BY_SIDE_MAX_SITES = 1e7;
 }  // namespace ts

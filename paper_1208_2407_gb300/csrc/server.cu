@@ -116,7 +116,9 @@ struct ts_server {
     uint64_t next_ticket = 1;
     size_t used = 0, peak = 0;
     bool stop = false, dead = false;
-    cudaStream_t compute = nullptr, copy = nullptr;
+    // lifting: an epoch's grids in the lifting form, where it has both forms
+    cudaStream_t compute = nullptr, lifting = nullptr, copy = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr;
     int *err_host = nullptr, *err_dev = nullptr;   // kernel error word and its pinned copy
     ts::EpochEntry *tab_dev = nullptr, *tab_host = nullptr;
     cudaEvent_t tab_free[kTables] = {};
@@ -137,7 +139,8 @@ struct ts_server {
     // the depth of full launches for grids with scaled rotations or in the
     // lifting form
     int depth(bool scaled) const { return scaled ? K : std::min(K, (int)ts::FUSED_LIFT_MAX_K); }
-    cudaError_t launch_full(int slot, int n, bool scaled, const ts::MultiPlan &plan, int L);
+    cudaError_t launch_full(int slot, int n, bool scaled, const ts::MultiPlan &plan, int L,
+                            cudaStream_t st);
 };
 
 int ts_server::take_table()
@@ -148,23 +151,24 @@ int ts_server::take_table()
     return s;
 }
 
-cudaError_t ts_server::launch_full(int slot, int n, bool scaled, const ts::MultiPlan &plan, int L)
+cudaError_t ts_server::launch_full(int slot, int n, bool scaled, const ts::MultiPlan &plan, int L,
+                                   cudaStream_t st)
 {
     const ts::EpochEntry *tab = tab_dev + (size_t)slot * cfg.max_slots;
     const int K = depth(scaled);
-    if (L == 1) return ts::launch_fused_multi(K, scaled, tab, n, plan, 0, err_dev, compute);
+    if (L == 1) return ts::launch_fused_multi(K, scaled, tab, n, plan, 0, err_dev, st);
     const GraphKey key{slot, n, L, K, scaled, plan.warps, plan.units, plan.aligned, plan.shape};
     for (auto &kv : graphs)
         if (kv.first == key) {
             ++graph_launches;
             ts::count_launches(L);
-            return cudaGraphLaunch(kv.second, compute);
+            return cudaGraphLaunch(kv.second, st);
         }
     cudaGraph_t graph = nullptr;
-    cudaError_t e = cudaStreamBeginCapture(compute, cudaStreamCaptureModeThreadLocal);
+    cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
     for (int t = 0; t < L && e == cudaSuccess; ++t)
-        e = ts::launch_fused_multi(K, scaled, tab, n, plan, t & 1, err_dev, compute);
-    cudaError_t e2 = cudaStreamEndCapture(compute, &graph);
+        e = ts::launch_fused_multi(K, scaled, tab, n, plan, t & 1, err_dev, st);
+    cudaError_t e2 = cudaStreamEndCapture(st, &graph);
     if (e == cudaSuccess) e = e2;
     cudaGraphExec_t exec = nullptr;
     if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
@@ -176,7 +180,7 @@ cudaError_t ts_server::launch_full(int slot, int n, bool scaled, const ts::Multi
     }
     graphs.push_back({key, exec});
     ++graph_launches;
-    return cudaGraphLaunch(exec, compute);
+    return cudaGraphLaunch(exec, st);
 }
 
 // Allocate and fill one admitted request's grid on the copy stream.
@@ -309,8 +313,19 @@ void ts_server::enqueue_epoch(std::unique_lock<std::mutex> &lk)
     for (auto &q : run_full) L = std::min(L, q->full_left);
     lk.unlock();
     cudaError_t e = cudaSuccess;
-    auto upload = [&](const std::vector<ReqP> &set, int depth, bool scaled,
-                      ts::MultiPlan &plan) -> int {
+    auto runs_scaled = [](const ReqP &q, int64_t depth) {
+        return q->scaled && ts::runs_scaled(q->r.theta, (int)depth, q->r.nx, q->r.ny);
+    };
+    double of_form[2] = {};   // sites
+    for (auto &q : run_full) of_form[runs_scaled(q, depth(q->scaled))] += (double)q->r.nx * q->r.ny;
+    for (auto &q : run_rem) of_form[runs_scaled(q, q->rem_left)] += (double)q->r.nx * q->r.ny;
+    // an epoch with both runs them side by side where they leave room (16 requests of
+    // 400 steps, half of them scaled, in turn and side by side: 128^2 3.0 and 2.3 ms,
+    // 512^2 6.4 and 5.9, 128 to 1024 5.4 and 4.7)
+    const bool both = of_form[0] > 0.0 && of_form[1] > 0.0 &&
+                      of_form[0] + of_form[1] <= ts::SIDE_BY_SIDE_MAX_SITES;
+    auto upload = [&](const std::vector<ReqP> &set, int depth, bool scaled, ts::MultiPlan &plan,
+                      cudaStream_t st) -> int {
         const int slot = take_table();
         ts::EpochEntry *h = tab_host + (size_t)slot * cfg.max_slots;
         std::vector<int> nx(set.size()), ny(set.size());
@@ -323,17 +338,20 @@ void ts_server::enqueue_epoch(std::unique_lock<std::mutex> &lk)
         if (plan.warps < 1 && e == cudaSuccess) e = cudaErrorInvalidConfiguration;
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(tab_dev + (size_t)slot * cfg.max_slots, h,
-                                sizeof(ts::EpochEntry) * set.size(), cudaMemcpyHostToDevice, compute);
+                                sizeof(ts::EpochEntry) * set.size(), cudaMemcpyHostToDevice, st);
         ep.tables.push_back(slot);
         return slot;
     };
     // grids with scaled rotations, then those in the lifting form: each form
     // has its full launches and its remainder launches (one per distinct
     // depth r below the form's)
-    auto runs_scaled = [](const ReqP &q, int64_t depth) {
-        return q->scaled && ts::runs_scaled(q->r.theta, (int)depth, q->r.nx, q->r.ny);
-    };
+    if (both) {
+        e = cudaEventRecord(fork, compute);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(lifting, fork, 0);
+        if (e != cudaSuccess) where = "epoch fork";
+    }
     for (const bool scaled : {true, false}) {
+        const cudaStream_t st = both && !scaled ? lifting : compute;
         std::vector<ReqP> full;
         std::vector<std::vector<ReqP>> by_rem(K);
         for (auto &q : run_full)
@@ -342,23 +360,29 @@ void ts_server::enqueue_epoch(std::unique_lock<std::mutex> &lk)
             if (runs_scaled(q, q->rem_left) == scaled) by_rem[q->rem_left].push_back(q);
         if (!full.empty() && e == cudaSuccess) {
             ts::MultiPlan plan{};
-            const int slot = upload(full, depth(scaled), scaled, plan);
+            const int slot = upload(full, depth(scaled), scaled, plan, st);
             if (e != cudaSuccess) where = "epoch table upload";
             if (e == cudaSuccess) {
-                e = launch_full(slot, (int)full.size(), scaled, plan, (int)L);
+                e = launch_full(slot, (int)full.size(), scaled, plan, (int)L, st);
                 if (e != cudaSuccess) where = L > 1 ? "epoch graph" : "epoch launch";
             }
         }
         for (int r = 1; r < K && e == cudaSuccess; ++r) {
             if (by_rem[r].empty()) continue;
             ts::MultiPlan plan{};
-            const int slot = upload(by_rem[r], r, scaled, plan);
+            const int slot = upload(by_rem[r], r, scaled, plan, st);
             if (e == cudaSuccess) {
                 e = ts::launch_fused_multi(r, scaled, tab_dev + (size_t)slot * cfg.max_slots,
-                                           (int)by_rem[r].size(), plan, 0, err_dev, compute);
+                                           (int)by_rem[r].size(), plan, 0, err_dev, st);
                 if (e != cudaSuccess) where = "remainder launch";
             }
         }
+    }
+    if (both) {
+        cudaError_t f = cudaEventRecord(join, lifting);
+        if (f == cudaSuccess) f = cudaStreamWaitEvent(compute, join, 0);
+        if (e == cudaSuccess && f != cudaSuccess) where = "epoch join";
+        if (e == cudaSuccess) e = f;
     }
     ep.err_copy = err_host + (epochs % kTables);
     if (e == cudaSuccess)
@@ -502,7 +526,10 @@ ts_status ts_server_create(const ts_server_cfg *cfg, ts_server **out)
     const int steps_per_epoch = cfg->max_epoch_steps > 0 ? cfg->max_epoch_steps : 32;
     s->L_max = std::max(1, steps_per_epoch / s->K);
     cudaError_t e = cudaStreamCreateWithFlags(&s->compute, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->lifting, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->copy, cudaStreamNonBlocking);
+    for (cudaEvent_t *ev : {&s->fork, &s->join})
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
     if (e == cudaSuccess)
         e = cudaHostAlloc((void **)&s->err_host, sizeof(int) * kTables, cudaHostAllocDefault);
     if (e == cudaSuccess) {
@@ -734,6 +761,7 @@ ts_status ts_server_destroy(ts_server *s)
         s->worker.join();
     }
     if (s->compute) cudaStreamSynchronize(s->compute);
+    if (s->lifting) cudaStreamSynchronize(s->lifting);
     if (s->copy) cudaStreamSynchronize(s->copy);
     for (auto &kv : s->reqs) free_request(s, *kv.second);
     s->reqs.clear();
@@ -745,7 +773,10 @@ ts_status ts_server_destroy(ts_server *s)
     if (s->tab_host) cudaFreeHost(s->tab_host);
     if (s->err_host) cudaFreeHost(s->err_host);
     if (s->err_dev) cudaFree(s->err_dev);
+    for (cudaEvent_t ev : {s->fork, s->join})
+        if (ev) cudaEventDestroy(ev);
     if (s->compute) cudaStreamDestroy(s->compute);
+    if (s->lifting) cudaStreamDestroy(s->lifting);
     if (s->copy) cudaStreamDestroy(s->copy);
     delete s;
     return TS_OK;

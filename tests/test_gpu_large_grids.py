@@ -30,7 +30,11 @@ def _evolve(nx, ny, theta, K, steps=5, batched=False, drive=False):
         if drive:
             g.set_drive(V, np.linspace(0.5, 1.0, steps))
         if batched:
-            trotter.evolve_batched([g], [steps], K)
+            other = trotter.Grid(64, 40, "f32")     # (a grid by itself runs as if alone)
+            other.set_potential(None, 0.05, theta)
+            trotter.evolve_batched([other, g], [steps, steps], K)
+            torch.cuda.synchronize()
+            other.close()
         else:
             g.evolve(steps, K)
         return torch.stack(g.get_state(np.float32, device=True))

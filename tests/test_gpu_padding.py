@@ -66,8 +66,13 @@ def test_evolve(nx, ny, theta):
 @pytest.mark.parametrize("nx,ny", SIDES)
 def test_evolve_batched(nx, ny):
     def run(g):
-        trotter.evolve_batched([g], [11])
-        return g.get_state(np.float64)
+        other = trotter.Grid(64, 40, "f32")     # (a grid by itself runs as if alone)
+        other.set_potential(None, 0.05, 0.03)
+        try:
+            trotter.evolve_batched([g, other], [11, 11])
+            return g.get_state(np.float64)
+        finally:
+            other.close()
 
     _both(nx, ny, run)
 
