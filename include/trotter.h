@@ -121,8 +121,8 @@ ts_status ts_set_state(ts_grid *g, const void *re, const void *im,
 
 /* Read the state into dense arrays of `dst_dtype` (host or device).  Syncs
  * `stream`; reports TS_ERR_TIMEOUT if a bounded wait inside an earlier fused
- * launch gave up, TS_ERR_CUDA for a failed earlier launch.  On either error
- * what the arrays hold is undefined. */
+ * launch gave up, TS_ERR_CUDA for a failed earlier launch, and then leaves the
+ * arrays as they were. */
 ts_status ts_get_state(ts_grid *g, void *re, void *im, ts_dtype dst_dtype,
                        ts_mem where, void *stream);
 

@@ -691,11 +691,15 @@ ts_status ts_get_state(ts_grid *g, void *re, void *im, ts_dtype dst_dtype, ts_me
     const size_t n = (size_t)nx * ny;
     cudaError_t e;
     if (where == TS_DEVICE) {
-        e = ts::launch_convert_out2(g->re(), g->im(), g->f64(), re, im, df, nx, ny, g->L.pitch, st);
+        // (leaves the arrays alone where the read-back will report an error)
+        e = ts::launch_convert_out2(g->re(), g->im(), g->f64(), re, im, df, nx, ny, g->L.pitch,
+                                    g->err, st);
         if (e != cudaSuccess) return cuda_fail(e, "ts_get_state");
         return read_back(g, st);
     }
     if (where != TS_HOST) return fail(TS_ERR_ARG, "ts_get_state: unknown memory kind");
+    ts_status s = read_back(g, st);   // host arrays are written only if all went well
+    if (s != TS_OK) return s;
     if (df == g->f64()) {
         const size_t es = g->esize;
         e = cudaMemcpy2DAsync(re, nx * es, g->re(), g->L.pitch * es, nx * es, ny,
@@ -703,8 +707,9 @@ ts_status ts_get_state(ts_grid *g, void *re, void *im, ts_dtype dst_dtype, ts_me
         if (e == cudaSuccess)
             e = cudaMemcpy2DAsync(im, nx * es, g->im(), g->L.pitch * es, nx * es, ny,
                                   cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) return cuda_fail(e, "ts_get_state: device-to-host copy");
-        return read_back(g, st);
+        return TS_OK;
     }
     // convert on the device into the staging region, then copy out
     const size_t es = df ? 8 : 4;
@@ -715,9 +720,10 @@ ts_status ts_get_state(ts_grid *g, void *re, void *im, ts_dtype dst_dtype, ts_me
         e = ts::launch_convert_out(srcs[c], g->f64(), stage, df, nx, ny, g->L.pitch, st);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(dsts[c], stage, n * es, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess && c == 1) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) return cuda_fail(e, "ts_get_state");
     }
-    return read_back(g, st);
+    return TS_OK;
 }
 
 ts_status ts_set_potential(ts_grid *g, const double *V, ts_mem where, double dt, double theta,

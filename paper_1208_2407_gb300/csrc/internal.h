@@ -36,9 +36,10 @@ cudaError_t launch_convert_out(const void *src, bool src_f64, void *dst, bool ds
 cudaError_t launch_convert_in2(const void *src0, const void *src1, bool src_f64, void *dst0,
                                void *dst1, bool dst_f64, int nx, int ny, int64_t pitch,
                                cudaStream_t st);
+// (launch_convert_out2 writes nothing if *err is not 0 when it runs)
 cudaError_t launch_convert_out2(const void *src0, const void *src1, bool src_f64, void *dst0,
                                 void *dst1, bool dst_f64, int nx, int ny, int64_t pitch,
-                                cudaStream_t st);
+                                const int *err, cudaStream_t st);
 // V (dense FP64) -> (gamma_V, s_V, V) pitched planes of the grid's type
 cudaError_t launch_phase_table(const double *V, void *pg, void *ps, void *vplane, bool f64,
                                int nx, int ny, int64_t pitch, double dt, cudaStream_t st);

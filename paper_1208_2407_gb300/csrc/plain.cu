@@ -67,9 +67,10 @@ __device__ __forceinline__ void store4(T *p, const T (&v)[4])
 template <bool IN, typename Ts, typename Td>
 __global__ void convert_kernel(const Ts *__restrict__ src0, Td *__restrict__ dst0,
                                const Ts *__restrict__ src1, Td *__restrict__ dst1, int nx, int ny,
-                               int64_t pitch, bool vec4)
+                               int64_t pitch, bool vec4, const int *err)
 {
     grid_dep_sync();
+    if (err && *err != 0) return;
     const Ts *src = blockIdx.z ? src1 : src0;
     Td *dst = blockIdx.z ? dst1 : dst0;
     for (int64_t y = blockIdx.y; y < ny; y += gridDim.y) {
@@ -376,7 +377,7 @@ inline dim3 grid2d(int64_t per_row, int rows)
 template <bool IN>
 cudaError_t launch_convert(const void *src0, const void *src1, bool src_f64, void *dst0,
                            void *dst1, bool dst_f64, int nx, int ny, int64_t pitch,
-                           cudaStream_t st)
+                           const int *err, cudaStream_t st)
 {
     auto aligned = [](const void *q) { return ((uintptr_t)q % 16) == 0; };
     const bool vec4 = (nx % 4) == 0 && aligned(src0) && aligned(dst0) &&
@@ -387,7 +388,7 @@ cudaError_t launch_convert(const void *src0, const void *src1, bool src_f64, voi
         using Ts = decltype(s);
         using Td = decltype(d);
         launch_pdl(convert_kernel<IN, Ts, Td>, grid, kThreads, 0, st, (const Ts *)src0, (Td *)dst0,
-                   (const Ts *)src1, (Td *)dst1, nx, ny, pitch, vec4);
+                   (const Ts *)src1, (Td *)dst1, nx, ny, pitch, vec4, err);
     };
     if (src_f64 && dst_f64)
         run(double(), double());
@@ -404,27 +405,29 @@ cudaError_t launch_convert(const void *src0, const void *src1, bool src_f64, voi
 cudaError_t launch_convert_in(const void *src, bool src_f64, void *dst, bool dst_f64, int nx,
                               int ny, int64_t pitch, cudaStream_t st)
 {
-    return launch_convert<true>(src, nullptr, src_f64, dst, nullptr, dst_f64, nx, ny, pitch, st);
+    return launch_convert<true>(src, nullptr, src_f64, dst, nullptr, dst_f64, nx, ny, pitch, nullptr,
+                                st);
 }
 
 cudaError_t launch_convert_out(const void *src, bool src_f64, void *dst, bool dst_f64, int nx,
                                int ny, int64_t pitch, cudaStream_t st)
 {
-    return launch_convert<false>(src, nullptr, src_f64, dst, nullptr, dst_f64, nx, ny, pitch, st);
+    return launch_convert<false>(src, nullptr, src_f64, dst, nullptr, dst_f64, nx, ny, pitch, nullptr,
+                                 st);
 }
 
 cudaError_t launch_convert_in2(const void *src0, const void *src1, bool src_f64, void *dst0,
                                void *dst1, bool dst_f64, int nx, int ny, int64_t pitch,
                                cudaStream_t st)
 {
-    return launch_convert<true>(src0, src1, src_f64, dst0, dst1, dst_f64, nx, ny, pitch, st);
+    return launch_convert<true>(src0, src1, src_f64, dst0, dst1, dst_f64, nx, ny, pitch, nullptr, st);
 }
 
 cudaError_t launch_convert_out2(const void *src0, const void *src1, bool src_f64, void *dst0,
                                 void *dst1, bool dst_f64, int nx, int ny, int64_t pitch,
-                                cudaStream_t st)
+                                const int *err, cudaStream_t st)
 {
-    return launch_convert<false>(src0, src1, src_f64, dst0, dst1, dst_f64, nx, ny, pitch, st);
+    return launch_convert<false>(src0, src1, src_f64, dst0, dst1, dst_f64, nx, ny, pitch, err, st);
 }
 
 cudaError_t launch_phase_table(const double *V, void *pg, void *ps, void *vplane, bool f64, int nx,

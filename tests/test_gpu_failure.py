@@ -64,3 +64,33 @@ def test_limit_out_of_range_is_refused():
         assert trotter.ts_launch_count() == 2         # nothing else was queued
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("device", [True, False])
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+def test_a_failed_read_leaves_the_arrays_alone(device, dtype):
+    import torch
+    rng = np.random.default_rng(5)
+    g = trotter.Grid(130, 66, "f32")
+    try:
+        g.set_state(*random_state(rng, 130, 66))
+        g.set_potential(None, 0.05, 0.025)
+        g.evolve(3)
+        trotter.ts_check_wait_timeout(g.handle, 1_000_000, trotter.current_stream_ptr())
+        if device:
+            out = torch.full((2, 66, 130), 7.0, device="cuda",
+                             dtype=torch.float32 if dtype == np.float32 else torch.float64)
+            ptrs = [trotter._VP(o.data_ptr()) for o in out]
+        else:
+            out = np.full((2, 66, 130), 7.0, dtype)
+            ptrs = [trotter._VP(o.ctypes.data) for o in out]
+        args = (*ptrs, trotter.TS_F32 if dtype == np.float32 else trotter.TS_F64,
+                trotter.TS_DEVICE if device else trotter.TS_HOST, trotter.current_stream_ptr())
+        with pytest.raises(trotter.TrotterError) as e:
+            trotter.ts_get_state(g.handle, *args)
+        assert e.value.status == trotter.TS_ERR_TIMEOUT
+        assert bool((out == 7.0).all())
+        trotter.ts_get_state(g.handle, *args)        # reported once, then cleared
+        assert not bool((out == 7.0).any())
+    finally:
+        g.close()
