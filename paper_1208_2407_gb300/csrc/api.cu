@@ -4,11 +4,11 @@
 // through the grid's own ping-pong planes, kernel dispatch and error
 // reporting.  Every step of the method runs in the kernels of plain.cu,
 // fused.cu and reduce.cu.
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
-#include <mutex>
 #include <new>
 #include <vector>
 
@@ -62,51 +62,60 @@ size_t scratch_bytes()
            round_up(sizeof(ts::GridDesc), 256);
 }
 
-// Pinned slots that read-backs land in, one per grid that reads back.  Blocks of
-// 64 slots; a block whose slots have all been returned is freed, unless it is
-// the only one.
+// Pinned slots that read-backs land in: one block of 64, made when the first grid
+// is (no call after that allocates) and kept.  A call holds a slot while it waits for
+// its copy, so any number of threads and streams may read back; more than 64 at a time
+// get none and read into pageable memory.
 constexpr size_t kSlotBytes = 512;
-constexpr int kBlockSlots = 64;
-struct SlotBlock {
-    unsigned char *base;
-    uint64_t used;
-};
-std::mutex g_slot_mu;
-std::vector<SlotBlock> g_slots;
+constexpr int kSlots = 64;
 
-unsigned char *readback_get()   // nullptr if no pinned memory is to be had
-{
-    std::lock_guard<std::mutex> lk(g_slot_mu);
-    for (SlotBlock &b : g_slots)
-        for (int i = 0; i < kBlockSlots; ++i)
-            if (!(b.used >> i & 1)) {
-                b.used |= uint64_t(1) << i;
-                return b.base + i * kSlotBytes;
+class ReadbackSlot {
+    static std::atomic<uint64_t> &used()
+    {
+        static std::atomic<uint64_t> bits{0};
+        return bits;
+    }
+    int slot_ = -1;
+
+public:
+    static unsigned char *block()   // nullptr if no pinned memory is to be had
+    {
+        static unsigned char *const base = [] {
+            // a capture on this or another thread does not mind this allocation
+            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+            cudaThreadExchangeStreamCaptureMode(&mode);
+            void *p = nullptr;
+            if (cudaHostAlloc(&p, kSlotBytes * kSlots, cudaHostAllocPortable) != cudaSuccess) {
+                cudaGetLastError();
+                p = nullptr;
             }
-    void *p = nullptr;
-    if (cudaHostAlloc(&p, kSlotBytes * kBlockSlots, cudaHostAllocPortable) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
+            cudaThreadExchangeStreamCaptureMode(&mode);
+            return (unsigned char *)p;
+        }();
+        return base;
     }
-    g_slots.push_back({(unsigned char *)p, 1});
-    return (unsigned char *)p;
-}
-
-void readback_put(unsigned char *slot)
-{
-    if (!slot) return;
-    std::lock_guard<std::mutex> lk(g_slot_mu);
-    for (size_t k = 0; k < g_slots.size(); ++k) {
-        SlotBlock &b = g_slots[k];
-        if (slot < b.base || slot >= b.base + kSlotBytes * kBlockSlots) continue;
-        b.used &= ~(uint64_t(1) << (slot - b.base) / kSlotBytes);
-        if (b.used == 0 && g_slots.size() > 1) {
-            cudaFreeHost(b.base);
-            g_slots.erase(g_slots.begin() + (ptrdiff_t)k);
+    ReadbackSlot()
+    {
+        uint64_t bits = used().load();
+        while (~bits) {
+            const int i = __builtin_ctzll(~bits);
+            if (used().compare_exchange_weak(bits, bits | uint64_t(1) << i)) {
+                slot_ = i;
+                return;
+            }
         }
-        return;
     }
-}
+    ~ReadbackSlot()
+    {
+        if (slot_ >= 0) used().fetch_and(~(uint64_t(1) << slot_));
+    }
+    ReadbackSlot(const ReadbackSlot &) = delete;
+    ReadbackSlot &operator=(const ReadbackSlot &) = delete;
+    unsigned char *get() const
+    {
+        return slot_ >= 0 && block() ? block() + slot_ * kSlotBytes : nullptr;
+    }
+};
 
 }  // namespace
 
@@ -117,6 +126,7 @@ ts_status grid_setup(const ts_layout &L, void *slab, bool owns_slab, ts_grid **o
 {
     ts_grid *g = new (std::nothrow) ts_grid();
     if (!g) return fail(TS_ERR_OOM, "grid set-up: host allocation failed");
+    ReadbackSlot::block();
     g->L = L;
     g->esize = L.dtype == TS_F64 ? 8 : 4;
     g->owns_slab = owns_slab;
@@ -130,7 +140,6 @@ ts_status grid_setup(const ts_layout &L, void *slab, bool owns_slab, ts_grid **o
     g->host_copied = nullptr;
     g->side = nullptr;
     g->fork = g->join = nullptr;
-    g->readback = nullptr;
     scr += 256;
     g->desc_dev = (GridDesc *)scr;
     g->cur = 0;
@@ -555,7 +564,6 @@ ts_status ts_destroy_grid(ts_grid *g)
     for (cudaEvent_t ev : {g->host_copied, g->fork, g->join})
         if (ev) cudaEventDestroy(ev);
     if (g->side) cudaStreamDestroy(g->side);
-    readback_put(g->readback);
     delete g;
     if (e != cudaSuccess) return cuda_fail(e, "ts_destroy_grid: cudaFree");
     return TS_OK;
@@ -619,9 +627,9 @@ ts_status stage_in(ts_grid *g, const void *host, ts_dtype src_dtype, void *dst, 
 // pageable memory is staged and took 10 us more).
 ts_status read_back(ts_grid *g, cudaStream_t st, int nq = 0, double *res = nullptr)
 {
-    if (!g->readback) g->readback = readback_get();
+    const ReadbackSlot slot;
     unsigned char local[kSlotBytes];
-    unsigned char *h = g->readback ? g->readback : local;
+    unsigned char *h = slot.get() ? slot.get() : local;
     const size_t off = (size_t)((unsigned char *)g->err - (unsigned char *)g->result);
     const void *src = nq ? (const void *)g->result : (const void *)g->err;
     const size_t word = nq ? off : 0;

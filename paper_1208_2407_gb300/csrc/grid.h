@@ -69,7 +69,6 @@ struct ts_grid {
     // the caller's stream (created by the first such batch that this grid leads)
     cudaStream_t side;
     cudaEvent_t fork, join;
-    unsigned char *readback;   // pinned: results and error word (taken on first use)
     bool tmaps_ok;
     CUtensorMap tm_state[2], tm_phase;   // (re, im) of pair 0 / 1; (gamma_V, s_V)
     ts::GridDesc *desc_dev;              // the same, for multi-grid launches (in the slab)
