@@ -190,10 +190,11 @@ ts_status ts_clear_drive(ts_grid *g);
 /* Evolve `steps` second-order steps (Eq. secondorder) on the grid's current
  * state.  FP32 grids run the fused kernel: K whole steps per HBM round trip
  * on TMA-staged shared-memory tiles (temporal blocking; K = 0 picks the
- * depth automatically: 4, or 3 when |theta| > 0.075 and the grid has fewer
- * than 2^21 sites; 1 <= K <= 8 asks for a
- * depth, of which at most 4 is used when |theta| > 0.075; a remainder of
- * steps % K runs at a smaller depth).  |theta| > pi/4 takes the plain path.
+ * depth automatically: 4, or 3 when |theta| > 0.075 or a side has fewer than 8
+ * sites and the grid has fewer than 2^21; 1 <= K <= 8 asks for a depth, of which
+ * at most 4 is used when |theta| > 0.075 or a side has fewer than 8 sites; a
+ * remainder of steps % K runs at a smaller depth).  |theta| > pi/4 takes the
+ * plain path.
  * Small and middle grids run the same steps on tiles held in registers, with
  * the same results bit for bit.  FP64 grids (K must be 0, else
  * TS_ERR_UNSUPPORTED) run one step per launch and pass over memory when they

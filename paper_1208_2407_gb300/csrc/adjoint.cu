@@ -272,7 +272,7 @@ ts_status ts_adjoint_backward_depth(ts_grid *g, void *ws, size_t ws_bytes, int K
     bw.g_il = (float *)plane(WS_G + 3);
 
     const double th = -g->theta;
-    const bool scaled = std::fabs(th) <= ts::SCALED_MAX_THETA;
+    const bool scaled = ts::scaled_angle(th, nx, ny);
     const double sub[ts::FUSED_ADJ_MAX_K] = {th, th, th, th};
     ts::ScaledCoef sc;
     int sc_k = 0;

@@ -47,7 +47,7 @@ constexpr int64_t kMaxSide = int64_t(1) << 20;
 // 8192^2 92 and 84).
 int auto_depth(const ts_grid *g)
 {
-    const bool scaled = std::fabs(g->theta) <= ts::SCALED_MAX_THETA;
+    const bool scaled = ts::scaled_angle(g->theta, g->L.nx, g->L.ny);
     return scaled || g->L.nx * g->L.ny >= (1 << 21) ? 4 : 3;
 }
 constexpr int kPlanes = 7;   // re_a, im_a, re_b, im_b, gamma_V, s_V, V
@@ -988,7 +988,7 @@ ts_status fused_run(ts_grid *g, int64_t steps, int K, double theta, const CUtens
                     const void *pg, cudaStream_t st, const double *drive_adt = nullptr)
 {
     if (!g->tmaps_ok) return fail(TS_ERR_STATE, "fused path: tensor maps missing");
-    const bool scaled = std::fabs(theta) <= ts::SCALED_MAX_THETA;
+    const bool scaled = ts::scaled_angle(theta, g->L.nx, g->L.ny);
     if (!scaled && K > ts::FUSED_LIFT_MAX_K) K = ts::FUSED_LIFT_MAX_K;
     const ts::RotCoef c = ts::rot_coef(theta);
     const double sub[ts::FUSED_MAX_K] = {theta, theta, theta, theta, theta, theta, theta, theta};
@@ -1067,7 +1067,7 @@ ts_status evolve3_fused(ts_grid *g, int64_t steps, cudaStream_t st)
 {
     if (!g->tmaps_ok) return fail(TS_ERR_STATE, "fused path: tensor maps missing");
     const ts::RotCoef c = grid_coef(g);
-    const bool scaled = std::fabs(g->theta) <= ts::SCALED_MAX_THETA;
+    const bool scaled = ts::scaled_angle(g->theta, g->L.nx, g->L.ny);
     ts::ScaledCoef sc;
     if (scaled) ts::scaled_coef(&g->theta, 1, g->L.nx, g->L.ny, g->L.nz, sc);
     for (int64_t n = 0; n < steps; ++n) {
@@ -1130,7 +1130,7 @@ ts_status fused_u4_steps(ts_grid *g, int64_t steps, cudaStream_t st)
     const double p4 = 1.0 / (4.0 - std::cbrt(4.0));
     const ts::RotCoef AB = ts::rot_coef((1.0 - 3.0 * p4) * g->theta);   // angle a + b
     const double wa = p4 * g->theta, wb = (1.0 - 4.0 * p4) * g->theta;
-    const bool scaled = std::fabs(wb) <= ts::SCALED_MAX_THETA;   // the larger of the two
+    const bool scaled = ts::scaled_angle(wb, g->L.nx, g->L.ny);   // the larger of the two
     const double sub[5] = {wa, wa, wb, wa, wa};
     ts::ScaledCoef sc;
     if (scaled) ts::scaled_coef(sub, 5, g->L.nx, g->rows(), 1, sc);
@@ -1436,7 +1436,9 @@ ts_status ts_evolve_batched(ts_grid *const *gs, int n, const int64_t *steps, int
             if (s != TS_OK) return s;
         } else {
             const int k = K == 0 ? auto_depth(gs[i]) : K;
-            const int form = std::fabs(gs[i]->theta) <= ts::SCALED_MAX_THETA ? 0 : k == 3 ? 1 : 2;
+            const int form = ts::scaled_angle(gs[i]->theta, gs[i]->L.nx, gs[i]->L.ny) ? 0
+                             : k == 3                                                 ? 1
+                                                                                      : 2;
             depth[form] = k;
             multi[form].push_back(gs[i]);
             msteps[form].push_back(steps[i]);

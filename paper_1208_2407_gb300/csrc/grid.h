@@ -22,10 +22,21 @@ RotCoef rot_coef(double theta);
 
 // Scaled rotations (fused.cu) serve |theta| <= this, per substep.  A launch
 // takes its scale out by a -= h a; the rounding of h is what they add to the
-// norm, and scaled_coef keeps it under 5e-10 per step here, where h < 1/8 at
-// depth 4.  The tangents and the edge ratios stay far from their poles.  Larger
+// norm.  The tangents and the edge ratios stay far from their poles.  Larger
 // angles take the lifting form.
 constexpr double SCALED_MAX_THETA = 0.075;
+// ... on grids of at least this many columns and rows.  In the bulk four columns mix
+// two floats h, so that the norm of a |psi|^2 spread evenly over columns mod 4 drifts by
+// at most 5e-10 per step at depths 1, 2 and 4, 9e-10 at the others, 8e-10 per fourth-order
+// step and 1e-9 per 3-D step; the lines at the edges take one float, up to 2e-9 per step for
+// the sites on them, which shows where they are a large part of all (sides of 1 to 4:
+// 1e-9 to 2e-9 per step over theta, 4e-10 to 5e-10 in the lifting form; 16^2 6e-10
+// and 8e-10).
+constexpr int SCALED_MIN_SIDE = 8;
+inline bool scaled_angle(double theta, int64_t nx, int64_t ny)
+{
+    return std::fabs(theta) <= SCALED_MAX_THETA && nx >= SCALED_MIN_SIDE && ny >= SCALED_MIN_SIDE;
+}
 // Whether a launch of K plain steps takes them.  Depth 2 on the largest grids does
 // not: its warps wait for HBM, and those of neighbouring strips drift apart and read
 // their shared columns twice, which the lifting form's slower, evener pace avoids
@@ -33,7 +44,7 @@ constexpr double SCALED_MAX_THETA = 0.075;
 // 134 and 125, 16384^2 550 and 522).
 inline bool runs_scaled(double theta, int K, int64_t nx, int64_t ny)
 {
-    return std::fabs(theta) <= SCALED_MAX_THETA && !(K == 2 && far_beyond_l2(nx, ny));
+    return scaled_angle(theta, nx, ny) && !(K == 2 && far_beyond_l2(nx, ny));
 }
 // Coefficients of a launch of K substeps with kinetic half angles sub[i].
 void scaled_coef(const double *sub, int K, int64_t nx, int64_t ny, int64_t nz, ScaledCoef &c);
@@ -105,7 +116,7 @@ void grid_set_coefficients(ts_grid *g, double dt, double theta, cudaStream_t st)
 // Write the grid's multi-grid descriptor (tensor maps, planes, coefficients)
 // into its slab on stream st (api.cu).
 void grid_write_desc(ts_grid *g, cudaStream_t st);
-// Evolve n FP32 grids (|theta| <= pi/4, with `scaled` <= SCALED_MAX_THETA)
+// Evolve n FP32 grids (|theta| <= pi/4, with `scaled` scaled_angle of each)
 // together with the multi-grid kernel at depth K (api.cu).
 cudaError_t evolve_multi(ts_grid *const *gs, const int64_t *steps, int n, int K, bool scaled,
                          cudaStream_t st);

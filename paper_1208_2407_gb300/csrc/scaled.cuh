@@ -24,7 +24,7 @@ constexpr uint32_t FULL = 0xffffffffu;
 // k < K + 1 is even sweep k, sweep K + 1 + m odd sweep m.
 // Kept small: 2.4 KB is what the fourth-order and the adjoint kernels have
 // beside their rings for 8 blocks per SM.  The modes are those of fused.cu.
-constexpr int LANE_CLASSES = 7;   // see lane_class
+constexpr int LANE_CLASSES = 5;   // see lane_class
 template <int K, int MODE>
 struct EdgeTab {
     static constexpr int SWEEPS = 3 * K + 1, CLASSES = LANE_CLASSES;
@@ -230,12 +230,12 @@ __device__ __forceinline__ unsigned col_places(int xg, int nx)
 }
 
 // Lanes with the same class receive the same coefficients in every sweep:
-// 0 off the grid, 1 inside, 2 holds the first column, 3 the last, 4 both,
-// 5 beside the lane whose first column is the last one, 6 that and the first.
+// 0 off the grid, 1 inside, 2 holds the first column, 3 the last, 4 beside the
+// lane whose first column is the last one.  (nx >= SCALED_MIN_SIDE: no lane is two of
+// these.)
 __device__ __forceinline__ int lane_class(int xg, int nx)
 {
-    const bool L = xg == 0, R = xg < nx && nx <= xg + 4, B = xg + 5 == nx;
-    return xg < 0 || xg >= nx ? 0 : L && R ? 4 : L && B ? 6 : L ? 2 : R ? 3 : B ? 5 : 1;
+    return xg < 0 || xg >= nx ? 0 : xg == 0 ? 2 : nx <= xg + 4 ? 3 : xg + 5 == nx ? 4 : 1;
 }
 
 // Zeros for the columns past the grid's last one in a lane that starts on the

@@ -243,7 +243,7 @@ bool ts_server::admit_one(const ReqP &q)
         q->status = TS_ERR_CUDA;
         return false;
     }
-    q->scaled = std::fabs(r.theta) <= ts::SCALED_MAX_THETA;
+    q->scaled = ts::scaled_angle(r.theta, r.nx, r.ny);
     q->full_left = r.steps / depth(q->scaled);
     q->rem_left = r.steps % depth(q->scaled);
     return true;

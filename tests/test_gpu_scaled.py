@@ -1,8 +1,8 @@
 """Scaled rotations of the fused kernels (|theta| <= 0.075): the lanes and rows
 at the edges of the grid take coefficients of their own, by how the side ends in
-a lane's four columns (sides 1 .. 9, around a strip of 112 or 120 columns) and
+a lane's four columns (sides 8 .. 13 and 32 .. 41, around a strip of 112 or 120 columns) and
 by its parity, at every depth; the largest angle of the form and the first one
-beyond it, which takes the lifting form.
+beyond it, which takes the lifting form, as sides 1 .. 7 do at every angle.
 
 Tolerances.  A step rounds each component about 10 times (six sweeps, the phase
 and the scale) by at most 2^-24 relative, and 13 steps add up like a random
@@ -20,7 +20,11 @@ from gpu_helpers import random_state, rel_l2, run_gpu
 pytestmark = pytest.mark.gpu
 
 STEPS, TOL = 13, 2e-6
-SIDES = [(124, 5), (125, 6), (126, 4), (127, 9), (128, 3), (129, 8), (240, 10), (241, 9), (1, 9), (2, 8), (3, 7), (4, 6), (5, 5), (6, 4), (7, 3), (8, 2), (9, 1), (111, 12),
+SIDES = [(32, 41), (33, 40), (34, 39), (35, 38), (36, 37), (37, 8), (8, 33), (9, 32), (10, 9),
+         (11, 8), (12, 11), (13, 10), (124, 15), (126, 14), (127, 9), (128, 13), (129, 8),
+         (240, 10), (241, 9), (114, 9), (115, 10), (120, 11), (121, 12),
+         (124, 5), (125, 6), (126, 4), (128, 3), (1, 9), (2, 8), (3, 7), (4, 6), (5, 5), (6, 4),
+         (7, 3), (8, 2), (9, 1), (111, 12),
          (112, 13), (113, 14), (114, 5), (115, 6), (116, 33), (119, 8), (120, 7), (121, 6),
          (225, 40), (226, 41)]
 
@@ -104,3 +108,27 @@ def test_default_depth_of_the_lifting_form(nx, ny, depth):
             g.close()
     for r, i in out[1:]:
         assert np.array_equal(r, out[0][0]) and np.array_equal(i, out[0][1])
+
+
+@pytest.mark.parametrize("nx,ny,K,theta", [(2000, 1, 0, 0.0731), (1, 2000, 0, 0.0731),
+                                           (2000, 2, 3, 0.075), (2, 2000, 3, 0.075),
+                                           (2000, 4, 0, 0.0731)])
+def test_norm_on_grids_that_are_mostly_edge(nx, ny, K, theta):
+    """Sides of less than 8 sites take the lifting form, whose steps leave the norm
+    alone: what is left is the phase table's rounding, at most 2 s^2 2^-25 = 3.4e-10
+    per step and site with s = sin(0.075), of either sign, and the random roundings,
+    2^-24 sqrt(10 / (steps sites)) = 7e-11 per step: below 6e-10 together."""
+    steps = 4000
+    rng = np.random.default_rng(nx)
+    re, im = random_state(rng, nx, ny)
+    V = rng.uniform(-0.5, 0.5, (ny, nx))
+    g = trotter.Grid(nx, ny, "f32")
+    try:
+        g.set_state(re, im)
+        g.set_potential(V, 2.0 * theta, theta)
+        before = g.norm()
+        g.evolve(steps, K)
+        drift = (g.norm() / before - 1.0) / steps
+    finally:
+        g.close()
+    assert abs(drift) < 6e-10, drift
