@@ -145,6 +145,7 @@ ts_status grid_setup(const ts_layout &L, void *slab, bool owns_slab, ts_grid **o
     g->cur = 0;
     g->dt = g->theta = g->J = 0.0;
     g->desc_written = false;
+    g->desc_theta = 0.0;
     g->sc_theta = 0.0;   // at theta = 0 every coefficient is 0
     std::memset(g->desc_host.sc, 0, sizeof(g->desc_host.sc));
     g->g1 = g->s1 = g->t1 = g->s2 = g->t2 = 0.0;
@@ -310,7 +311,7 @@ void scaled_coef(const double *sub, int K, int64_t nx, int64_t ny, int64_t nz, S
             }
 }
 
-void grid_set_coefficients(ts_grid *g, double dt, double theta, cudaStream_t st)
+void grid_set_coefficients(ts_grid *g, double dt, double theta)
 {
     g->dt = dt;
     g->theta = theta;
@@ -321,8 +322,7 @@ void grid_set_coefficients(ts_grid *g, double dt, double theta, cudaStream_t st)
     g->t1 = c.t1;
     g->s2 = c.s2;
     g->t2 = c.t2;
-    // the descriptor holds no dt: it stands while the angle does
-    if (!g->f64() && !(g->desc_written && g->sc_theta == g->theta)) grid_write_desc(g, st);
+    if (g->desc_theta != theta) g->desc_written = false;   // (it holds no dt)
 }
 
 void grid_write_desc(ts_grid *g, cudaStream_t st)
@@ -361,6 +361,7 @@ void grid_write_desc(ts_grid *g, cudaStream_t st)
     const cudaError_t e =
         cudaMemcpyAsync(g->desc_dev, &d, sizeof(GridDesc), cudaMemcpyHostToDevice, st);
     g->desc_written = e == cudaSuccess && q == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+    g->desc_theta = g->theta;
 }
 
 cudaError_t evolve_multi(ts_grid *const *gs, const int64_t *steps, int n, int K, bool scaled,
@@ -378,6 +379,11 @@ cudaError_t evolve_multi(ts_grid *const *gs, const int64_t *steps, int n, int K,
         rem[i] = steps[i] % K;
         if (full[i] > max_full) max_full = full[i];
     }
+    // The descriptors are written here and not where the angle is set: who launches on a
+    // grid's state is ordered behind who launched on it before, and so behind the write,
+    // but not behind a write that an unrelated stream has queued.
+    for (int i = 0; i < n; ++i)
+        if (!gs[i]->desc_written) grid_write_desc(gs[i], st);
     EpochEntry *tab = nullptr;
     cudaError_t e = cudaMallocAsync((void **)&tab, sizeof(EpochEntry) * (size_t)n, st);
     if (e != cudaSuccess) return e;
@@ -538,10 +544,7 @@ ts_status ts_create_grid3(int64_t nx, int64_t ny, int64_t nz, ts_dtype dtype, vo
         return st;
     }
     cudaError_t e = cudaMemset(g->slab, 0, L.slab_bytes);
-    if (e == cudaSuccess && !g->f64()) {
-        ts::grid_write_desc(g, nullptr);
-        e = cudaStreamSynchronize(nullptr);
-    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     if (e != cudaSuccess) {
         ts_destroy_grid(g);
         return cuda_fail(e, "ts_create_grid: zero-fill");
@@ -778,7 +781,7 @@ ts_status ts_set_potential_order(ts_grid *g, const double *V, ts_mem where, doub
         }
         g->tab_b = tb;
     }
-    ts::grid_set_coefficients(g, dt, theta, st);
+    ts::grid_set_coefficients(g, dt, theta);
     g->order = order;
     if (order == 4)
         for (int i = 0; i < 2; ++i) g->sub[i] = ts::rot_coef(w[i] * theta);

@@ -85,7 +85,8 @@ struct ts_grid {
     ts::GridDesc *desc_dev;              // the same, for multi-grid launches (in the slab)
     ts::GridDesc desc_host;
     double sc_theta;                     // the angle of desc_host.sc
-    bool desc_written;                   // desc_dev holds desc_host
+    bool desc_written;                   // desc_dev holds desc_host ...
+    double desc_theta;                   // ... of this angle
 
     void *plane(int i) const { return slab + (size_t)i * L.plane_bytes; }
     void *re() const { return plane(2 * cur); }
@@ -111,8 +112,8 @@ namespace ts {
 ts_status grid_setup(const ts_layout &L, void *slab, bool owns_slab, ts_grid **out);
 // Byte offset of the scratch area (partials, result, error word, descriptor).
 size_t grid_scratch_offset(const ts_layout &L);
-// Rotation coefficients for (dt, theta), and the descriptor (api.cu).
-void grid_set_coefficients(ts_grid *g, double dt, double theta, cudaStream_t st);
+// Rotation coefficients for (dt, theta) (api.cu).
+void grid_set_coefficients(ts_grid *g, double dt, double theta);
 // Write the grid's multi-grid descriptor (tensor maps, planes, coefficients)
 // into its slab on stream st (api.cu).
 void grid_write_desc(ts_grid *g, cudaStream_t st);

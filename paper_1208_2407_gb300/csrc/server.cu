@@ -210,7 +210,8 @@ bool ts_server::admit_one(const ReqP &q)
     const size_t n = (size_t)nx * ny;
     const size_t scr = ts::grid_scratch_offset(L);
     e = cudaMemsetAsync(g->slab + scr, 0, L.slab_bytes - scr, copy);
-    ts::grid_set_coefficients(g, r.dt, r.theta, copy);
+    ts::grid_set_coefficients(g, r.dt, r.theta);
+    ts::grid_write_desc(g, copy);
     // potential -> tables (host input staged through the idle ping-pong pair)
     if (e == cudaSuccess && r.V) {
         const double *src = r.V;

@@ -99,3 +99,37 @@ def test_server_equals_solo_runs(name):
         srv.close()
         for g in grids:
             g.close()
+
+
+def test_angle_set_behind_another_streams_work():
+    """The angle is set on a busy stream and again on the stream that evolves: what the
+    batch reads must not be left to the busy stream's queue."""
+    import torch
+    nx, ny, theta, steps = 200, 90, 0.05, 9
+    re, im, V = _inputs(nx, ny)
+    busy, mine = torch.cuda.Stream(), torch.cuda.Stream()
+    on_busy, on_mine = (trotter._VP(s.cuda_stream) for s in (busy, mine))
+    grids = [trotter.Grid(nx, ny, "f32") for _ in range(2)]
+    big = trotter.Grid(8192, 8192, "f32")
+    try:
+        big.set_potential(None, 0.05, 0.025)
+        for g in grids:
+            g.set_potential(V, 0.05, 0.01)
+        trotter.evolve_batched(grids, [steps, steps])
+        torch.cuda.synchronize()
+        big.evolve(4000, stream=on_busy)                   # about 0.3 s
+        grids[0].set_potential(V, 0.05, theta, on_busy)
+        for g in grids:
+            g.set_potential(V, 0.05, theta, on_mine)
+            g.set_state(re, im, on_mine)
+        trotter.evolve_batched(grids, [steps, steps], stream=on_mine)
+        out = [torch.stack(g.get_state(np.float32, device=True, stream=on_mine)) for g in grids]
+        assert not busy.query()
+        torch.cuda.synchronize()
+        grids[1].set_state(re, im)
+        grids[1].evolve(steps)
+        want = torch.stack(grids[1].get_state(np.float32, device=True))
+        assert torch.equal(out[0], want) and torch.equal(out[1], want)
+    finally:
+        for g in grids + [big]:
+            g.close()

@@ -90,7 +90,7 @@ def test_potential_set_under_capture_then_again():
     gen = torch.Generator(device="cuda").manual_seed(1)
     V = torch.rand(n, n, dtype=torch.float64, device="cuda", generator=gen)
     re, im = torch.randn(2, n, n, device="cuda", generator=gen)
-    grids = [trotter.Grid(n, n, "f32") for _ in range(2)]
+    grids = [trotter.Grid(n, n, "f32") for _ in range(3)]
     try:
         for g in grids:
             g.set_state(re, im)
@@ -99,9 +99,9 @@ def test_potential_set_under_capture_then_again():
             grids[0].set_potential(V, 2.0 * theta, theta)
         for g in grids:
             g.set_potential(V, 2.0 * theta, theta)
-        trotter.evolve_batched(grids[:1], [8], 4)
+        trotter.evolve_batched([grids[0], grids[2]], [8, 8], 4)   # (one alone is no batch)
         grids[1].evolve(8, 4)
-        a, b = (g.get_state(np.float32) for g in grids)
+        a, b = (g.get_state(np.float32) for g in grids[:2])
     finally:
         for g in grids:
             g.close()
