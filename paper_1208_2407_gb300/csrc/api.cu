@@ -1054,11 +1054,6 @@ ts_status fused_steps(ts_grid *g, int64_t steps, int K, cudaStream_t st)
     return fused_run(g, steps, K, g->theta, &g->tm_phase, g->pg(), st);
 }
 
-// Fourth-order steps (Eq. fourthorder): the substeps a = U2(p dt) and
-// b = U2((1-4p) dt) in the order a a b a a per step.  The a substeps of
-// neighbouring steps run back to back (a run of 2 at either end, of 4
-// between two b substeps), so on the fused path each run of r substeps is
-// ceil(r / K) launches of near-equal depth; each b substep is one launch.
 // 3-D steps on the fast path (FP32, |theta| <= pi/4, (nz + 32) ny < 2^31):
 // one launch and one HBM round trip per step (fused.cu, fused3d_kernel).  Z
 // factors commute with X and Y factors, so the step
@@ -1112,8 +1107,10 @@ ts_status evolve_driven(ts_grid *g, int64_t steps, int K, bool plain, cudaStream
         s = plain_run(g, steps, grid_coef(g), g->pg(), g->ps(), st, adt.data());
     } else {
         // depth 4 by default: with the drive phase computed per site the
-        // kernel is arithmetic-bound, and 4 measured fastest (8192^2: 4.1e11
-        // site-steps/s against 3.8e11 at depth 3)
+        // kernel is bound by issue, and 4 measured fastest with scaled rotations
+        // (8192^2: 5.5e11 site-steps/s against 5.3e11 at depth 3) and, up to
+        // 3500^2, in the lifting form (4.2e11 and 4.0e11 there, 4.7e11 and 4.9e11
+        // at 8192^2)
         int depth = K == 0 ? ts::FUSED_DRIVE_MAX_K : K;
         if (depth > ts::FUSED_DRIVE_MAX_K) depth = ts::FUSED_DRIVE_MAX_K;
         s = fused_run(g, steps, depth, g->theta, &g->tm_drive, nullptr, st, adt.data());
@@ -1166,6 +1163,11 @@ ts_status fused_u4_steps(ts_grid *g, int64_t steps, cudaStream_t st)
     return TS_OK;
 }
 
+// Fourth-order steps (Eq. fourthorder): the substeps a = U2(p dt) and
+// b = U2((1-4p) dt) in the order a a b a a per step.  The a substeps of
+// neighbouring steps run back to back (a run of 2 at either end, of 4
+// between two b substeps), so on the fused path each run of r substeps is
+// ceil(r / K) launches of near-equal depth; each b substep is one launch.
 ts_status evolve4(ts_grid *g, int64_t steps, int K, bool plain, cudaStream_t st)
 {
     if (!plain && K == 0) return fused_u4_steps(g, steps, st);

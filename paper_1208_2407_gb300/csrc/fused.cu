@@ -1897,14 +1897,13 @@ cudaError_t launch_k(const FusedLaunch &a, cudaStream_t st)
     p.n_pairs = (a.ny + 1) / 2;
     p.units = (int64_t)p.n_strips * p.n_pairs;
     int64_t cap = (int64_t)num_sms * blocks_per_sm * C::WPC;
-    // Depths 1 and 2 wait for HBM, and with every warp in flight neighbouring
-    // strips drift apart: the halo columns they share leave L2 before the second
-    // strip reads them.  On grids far larger than L2 fewer warps keep pace (depth
-    // 1, 8 or 4 warps per SM: 3000 x 2048, 147 MB at 24 B per site, 23.3 and 27.1
-    // us, 4096^2 73.2 and 67.6, 8192^2 290 and 272; depth 2, 8 or 7: 4096^2 64.6
-    // and 71.9, 8192^2 281 and 264).
-    if (SC && MODE == 0 && K <= 2 && 24.0 * a.nx * a.ny > (K == 1 ? 256e6 : 1e9))
-        cap = std::min<int64_t>(cap, (int64_t)num_sms * (K == 1 ? 4 : 7));
+    // Depth 1 waits for HBM, and with every warp in flight neighbouring strips drift
+    // apart: the halo columns they share leave L2 before the second strip reads them.
+    // On grids larger than L2 fewer warps keep pace (8 or 4 warps per SM: 3000 x 2048,
+    // 147 MB at 24 B per site, 23.3 and 27.1 us, 4096^2 73.2 and 67.6, 8192^2 290 and
+    // 272).  (Depth 2 takes the lifting form there, see runs_scaled in grid.h.)
+    if (SC && MODE == 0 && K == 1 && 24.0 * a.nx * a.ny > 256e6)
+        cap = std::min<int64_t>(cap, (int64_t)num_sms * 4);
     // Driven in the lifting form at depth 3, three warps per scheduler take 1.4 times
     // as long for a row pair as two (strip_warps_for counts on 1.27): with fewer than
     // 13 row pairs each, two (2048^2, 12 and 8 warps per SM: 15.0 and 13.9 us per step).

@@ -317,9 +317,13 @@ void count_launches(int64_t n);
 // repeats every 4.1 us, one of 4.9 us every 8.2 us); dependent ones follow
 // 0.4 to 0.7 us after the kernel before, whatever its length: 6 us launches
 // become 4.6 us (depth 1 at 256^2), 27.3 us ones 25.2 us (depth 3 at 2048^2).
-// No kernel lets its successor start early (griddepcontrol.launch_dependents):
-// blocks that become resident during the tail cost more than they hide, 2 to
-// 10 % up to 1024^2 and 40 % for depth 3 at 2048^2.
+// The register tiles (tile.cu, tile_adjoint.cu) let their successor start early, before
+// their stores (griddepcontrol.launch_dependents): its blocks then wait in grid_dep_sync
+// until the stores are visible.  That is safe because every kernel launched here
+// calls grid_dep_sync before its first access to global memory; a kernel without
+// that call must not be launched by launch_pdl.  The other kernels do not: blocks
+// that become resident during the tail cost more than they hide there, 2 to 10 % up
+// to 1024^2 and 40 % for depth 3 at 2048^2.
 template <typename... P, typename... A>
 inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
                               cudaStream_t st, A &&...args)

@@ -235,7 +235,8 @@ __device__ __forceinline__ unsigned col_places(int xg, int nx)
 // these.)
 __device__ __forceinline__ int lane_class(int xg, int nx)
 {
-    return xg < 0 || xg >= nx ? 0 : xg == 0 ? 2 : nx <= xg + 4 ? 3 : xg + 5 == nx ? 4 : 1;
+    const bool L = xg == 0, R = xg < nx && nx <= xg + 4, B = xg + 5 == nx;
+    return xg < 0 || xg >= nx ? 0 : L ? 2 : R ? 3 : B ? 4 : 1;
 }
 
 // Zeros for the columns past the grid's last one in a lane that starts on the
@@ -266,7 +267,7 @@ __device__ __forceinline__ float4 edge_h(const float *tab, int row, int ny, unsi
     return make_float4(at(0), at(1), at(2), at(3));
 }
 
-// asynchronous 16-byte copies to shared memory (zfill: zeros unless `in`)
+// asynchronous 16-byte copies to shared memory
 __device__ __forceinline__ void cp_async16(void *dst, const void *src)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src)
@@ -283,6 +284,7 @@ __device__ __forceinline__ void cp_async_wait_all()
     asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
+// (zeros unless `in`)
 __device__ __forceinline__ void cp_async16_zfill(void *dst, const void *src, bool in)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(dst)), "l"(src),

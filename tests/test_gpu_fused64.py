@@ -1,7 +1,7 @@
 """Fused FP64 steps (one launch per step) against the oracle: sides around the
 strips of 26, 58 and 122 columns and the row ranges, odd and even, sides of one
 to three, positive, negative and largest angles, the fourth-order step, and a
-run long enough to be cut where the scaled state has grown by 2^60.
+run long enough to be cut where the scaled state has grown by 2^30.
 
 Tolerance: about 20 roundings of 2^-53 per component and step that add up like a
 random walk, and coefficients within 2^-53 that add up linearly over the steps:
@@ -54,8 +54,8 @@ def test_order4(nx, ny):
 
 
 def test_long_run_is_cut():
-    # theta = 0.39: a step grows the bulk by 1.5 in the odd and the even sweeps,
-    # so 2^60 is passed every few dozen steps
+    # theta = 0.39: a step grows the bulk by 1.64 per axis (two odd sweeps at theta and
+    # an even one at 2 theta), 2.7 in all, so 2^30 is passed every 21 steps
     rng = np.random.default_rng(2)
     re, im = random_state(rng, 45, 34)
     V = rng.uniform(-0.5, 0.5, (34, 45))
