@@ -249,7 +249,9 @@ ts_status ts_energy(ts_grid *g, double *out, void *stream);   /* e_kin + e_pot *
 /* Evolve n independent grids (steps[i] steps each, fused depth K as in
  * ts_evolve) on one stream.  Second-order 2-D FP32 grids with |theta| <=
  * pi/4 and no drive advance together in multi-grid launches of the fused
- * kernel; every other grid runs ts_evolve on its own (FP64 grids with K = 0,
+ * kernel (of several, if the grids' angles or sizes call for several; one of
+ * them may run on a stream of the library's own that is ordered behind what is
+ * on `stream` and before what follows); every other grid runs ts_evolve on its own (FP64 grids with K = 0,
  * whatever K is given).  Errors: TS_ERR_ARG (n < 0, NULL arrays, a NULL grid
  * or negative steps), then those of ts_evolve.  Async. */
 ts_status ts_evolve_batched(ts_grid *const *g, int n, const int64_t *steps, int K,
@@ -398,7 +400,8 @@ ts_status ts_norm_noalloc(const void *re, const void *im, ts_dtype dtype, int64_
                           int64_t ny, int64_t pitch, double *out, void *stream);
 size_t ts_norm_noalloc_scratch_bytes(void);
 
-/* The fused depth ts_evolve uses when K = 0 (for |theta| <= 0.075). */
+/* The fused depth ts_evolve uses when K = 0 (for |theta| <= 0.075 and sides of 8
+ * sites or more). */
 int ts_fused_default_depth(void);
 
 /* Number of kernels this thread's calls enqueued since the last reset. */

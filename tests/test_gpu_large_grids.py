@@ -15,7 +15,8 @@ from paper_1208_2407_gb300 import trotter
 pytestmark = pytest.mark.gpu
 
 TOL = 2e-6
-SIDES = [(1003, 33501), (33503, 1001), (5801, 5800)]
+SIDES = [(1003, 33501), (33503, 1001), (5801, 5800), (37, 1000003), (124, 280002),
+         (125, 280003)]
 
 
 def _evolve(nx, ny, theta, K, steps=5, batched=False, drive=False):
