@@ -137,6 +137,7 @@ ts_status grid_setup(const ts_layout &L, void *slab, bool owns_slab, ts_grid **o
     g->result = (double *)scr;
     scr += round_up(sizeof(double) * OBS_Q3, 256);
     g->err = (int *)scr;
+    g->served = false;
     g->host_copied = nullptr;
     g->side = nullptr;
     g->fork = g->join = nullptr;
@@ -709,8 +710,10 @@ ts_status ts_get_state(ts_grid *g, void *re, void *im, ts_dtype dst_dtype, ts_me
         return read_back(g, st);
     }
     if (where != TS_HOST) return fail(TS_ERR_ARG, "ts_get_state: unknown memory kind");
-    ts_status s = read_back(g, st);   // host arrays are written only if all went well
-    if (s != TS_OK) return s;
+    if (!g->served) {   // host arrays are written only if all went well
+        ts_status s = read_back(g, st);
+        if (s != TS_OK) return s;
+    }
     if (df == g->f64()) {
         const size_t es = g->esize;
         e = cudaMemcpy2DAsync(re, nx * es, g->re(), g->L.pitch * es, nx * es, ny,

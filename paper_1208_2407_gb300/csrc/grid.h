@@ -75,6 +75,7 @@ struct ts_grid {
     bool driven;
     double *partials, *result;
     int *err;
+    bool served;               // a server's grid: launches report in the server's word, not in err
     cudaEvent_t host_copied;   // host-input copies done (created on first use)
     // a batch whose grids take several kernels runs a group of them here, beside
     // the caller's stream (created by the first such batch that this grid leads)

@@ -206,6 +206,7 @@ bool ts_server::admit_one(const ReqP &q)
         return false;
     }
     ts_grid *g = q->g;
+    g->served = true;   // (a request is fetched only if its epochs reported nothing)
     const int nx = (int)r.nx, ny = (int)r.ny;
     const size_t n = (size_t)nx * ny;
     const size_t scr = ts::grid_scratch_offset(L);
